@@ -178,8 +178,7 @@ typedef struct {
 int lbm_info(lbm_sim* sim, lbm_info_t* out);
 
 /* Use the plain step kernel (variant 0) with this tile (block_x a multiple of 32,
- * block_x * block_y <= 512).  Results do not depend on the tile, except for the order in which the
- * FP64 force partials of the tiles are summed. */
+ * block_x * block_y <= 512).  Results do not depend on the tile. */
 int lbm_set_tile(lbm_sim* sim, int block_x, int block_y);
 
 /* Choose the step kernel.  0: plain kernel, one block per tile of lbm_set_tile's shape, wrapped
@@ -197,9 +196,8 @@ int lbm_set_tile(lbm_sim* sim, int block_x, int block_y);
  * least 12 blocks per SM), 64 x 1 (2 rows), 64 x 1 (4 rows, 10 blocks), 128 x 1 (2 rows), 64 x 1
  * (3 rows, 12 blocks), 64 x 1 (3 rows, 11 blocks) threads (D2Q37);
  * 20: two neighbouring nodes per thread with paired loads and stores, 64 x 4 tiles (D2Q9).
- * Every variant evaluates the same expressions in the same order; results agree to FP32 rounding
- * (the compiler may contract them into different fused multiply-adds in different kernels) and the
- * force also by the order in which tile partials are summed when the tile shape differs.
+ * Every variant evaluates the same rounded operations in the same order and sums the force in the
+ * same order: states and forces are the same bit for bit.
  * LBM_EINVAL if the variant is not built for the simulation's storage type. */
 int lbm_set_variant(lbm_sim* sim, int variant);
 
@@ -474,8 +472,8 @@ void lbm_server_destroy(lbm_server* server);
  * The work is enqueued on `stream` (a cudaStream_t; 0 is the default stream) and the call returns
  * before it runs.
  *
- * Scratch: the kernel's per-tile force partials and its reduction counter live in one static
- * device array of the library (LBM_NOALLOC_MAX_SLOTS * 16 + 256 bytes), held by every GPU that
+ * Scratch: the kernel's force partials and its reduction counter live in one static
+ * device array of the library (LBM_NOALLOC_MAX_SLOTS * 256 + 256 bytes), held by every GPU that
  * loads the library until the process exits.  A geometry with more than LBM_NOALLOC_MAX_SLOTS
  * tiles holding body links is rejected with LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer).
  * All calls in the process share that array: calls whose work overlaps on the GPU (two streams,

@@ -30,7 +30,7 @@ struct Slot {
     long long start = 0;      // batch step of the instance's step 0
     long long nsteps = 0;
     // persistent mode: one allocation holding the per-step constants [nsteps], the band counters
-    // [<= nty], the force ring [kRing][nslots], its tickets [kRing] and finish marks [kRing]
+    // [<= nty], the force ring [kRing][ngroups], its tickets [kRing] and finish marks [kRing]
     unsigned char* d_pb = nullptr;
     size_t off_done = 0, off_ring = 0, off_tickets = 0, off_fin = 0;
     size_t bytes = 0;
@@ -114,12 +114,12 @@ void free_graph(lbm_batch* b) {
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Layout of a persistent-mode instance's allocation (see Slot); returns its size.
-size_t pb_layout(long long nsteps, int nty, int nslots, Slot* s) {
+size_t pb_layout(long long nsteps, int nty, int ring_len, Slot* s) {
     size_t off = align_up((size_t)nsteps * sizeof(StepConst), 256);
     const size_t done = off;
     off = align_up(off + (size_t)nty * sizeof(int), 256);
     const size_t ring = off;
-    off = align_up(off + (size_t)kRing * (size_t)std::max(1, nslots) * sizeof(double2), 256);
+    off = align_up(off + (size_t)kRing * (size_t)std::max(1, ring_len) * sizeof(double2), 256);
     const size_t tickets = off;
     off = align_up(off + kRing * sizeof(unsigned int), 256);
     const size_t fin = off;
@@ -134,7 +134,8 @@ size_t pb_layout(long long nsteps, int nty, int nslots, Slot* s) {
 }
 
 // Device bytes of one instance (populations, geometry arrays, force history, and in the persistent
-// mode its step table, tile counters and force ring; the tile shape bx x by).
+// mode its step table, tile counters and force ring; the tile shape bx x by; the force scratch of an
+// instance is bounded by its tiles).
 size_t footprint(const HostLattice& H, int nx, int ny, int storage, int layout, long nsteps, int bx, int by) {
     const size_t es = storage_size(storage);
     const size_t align = 128 / es;
@@ -175,8 +176,13 @@ int rebuild(lbm_batch* b) {
         const int ntx = v.inst.ntx, S = b->seg_tiles;
         I.band = S;
         I.nseg = ntx;
+        I.fb0 = v.inst.ngroups > 0 ? v.body_row0 / (S * v.by) : 1;
+        I.fb1 = v.inst.ngroups > 0 ? v.body_row1 / (S * v.by) : 0;
         if (!slot_running(b, s)) continue;
-        // the columns of a band follow each other, so that they run side by side
+        // force items first, then the strips: the columns of a band follow each other, so that they run
+        // side by side
+        const int per = kForceItemGroups * (int)(b->kernel.block.x * b->kernel.block.y / 32);
+        for (int g = 0; g < v.inst.ngroups; g += per) segs.push_back(make_int4((int)k, -1, g, 0));
         for (int band = 0; band * S < I.nty; ++band)
             for (int tx = 0; tx < ntx; ++tx) segs.push_back(make_int4((int)k, band, tx, 0));
     }
@@ -390,7 +396,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         // per-step constants, tile counters (0: no step done) and the force ring (entry j free,
         // as if the step j - kRing had left it)
         const SimView v = sim_view(sim);
-        const size_t pb = pb_layout(d->nsteps, (v.ny + v.by - 1) / v.by, v.nslots, &s);
+        const size_t pb = pb_layout(d->nsteps, (v.ny + v.by - 1) / v.by, v.inst.ngroups, &s);
         std::vector<unsigned char> host(pb, 0);
         sim_step_constants(sim, d->nsteps, reinterpret_cast<StepConst*>(host.data()));
         int* fin = reinterpret_cast<int*>(host.data() + s.off_fin);

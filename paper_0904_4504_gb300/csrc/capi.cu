@@ -343,9 +343,11 @@ void build_links(const HostLattice& H, int nx, int ny, const std::vector<uint8_t
 }
 
 // Geometry-only part of the momentum exchange (the rest populations w_i rho0 bounced on body
-// links): -sum over body links of c_i 2 w_i rho0.
-void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, double rho0, double& fx, double& fy) {
-    fx = fy = 0.0;
+// links), -sum over body links of c_i 2 w_i rho0, and the moving-wall part per unit wall velocity,
+// -sum of c_i c_ix 2 w_i rho0 / theta.
+void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, double rho0, double& fx, double& fy,
+                    double& mx, double& my) {
+    fx = fy = mx = my = 0.0;
     for (const LinkNode& ln : links) {
         const uint64_t b = ln.body;
         if (!b) continue;
@@ -353,24 +355,26 @@ void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, do
             if ((b >> i) & 1ull) {
                 fx -= H.c[i][0] * 2.0 * H.w[i] * rho0;
                 fy -= H.c[i][1] * 2.0 * H.w[i] * rho0;
+                mx -= H.c[i][0] * H.c[i][0] * 2.0 * H.w[i] * rho0 / H.theta;
+                my -= H.c[i][1] * H.c[i][0] * 2.0 * H.w[i] * rho0 / H.theta;
             }
     }
 }
 
-void tile_slots(int nx, int ny, int bx, int by, const std::vector<LinkNode>& links, std::vector<int>& slot, int& ntx,
-                int& ntiles, int& nslots) {
-    ntx = (nx + bx - 1) / bx;
-    const int nty = (ny + by - 1) / by;
-    ntiles = ntx * nty;
-    slot.assign(ntiles, -1);
+// Tiles of bx x by nodes that hold body links.
+int body_tiles(int nx, int ny, int bx, int by, const std::vector<LinkNode>& links) {
+    const int ntx = (nx + bx - 1) / bx;
+    std::vector<uint8_t> row(ntx, 0);  // of the current row of tiles (links are in node order)
+    int n = 0, at = -1;
     for (const LinkNode& ln : links) {
         if (!ln.body) continue;
-        const int x = (int)(ln.node % (size_t)nx), y = (int)(ln.node / (size_t)nx);
-        slot[(y / by) * ntx + x / bx] = 0;  // tile with body links
+        const int tx = (int)(ln.node % (size_t)nx) / bx, ty = (int)(ln.node / (size_t)nx) / by;
+        if (ty != at) std::fill(row.begin(), row.end(), 0);
+        at = ty;
+        n += !row[tx];
+        row[tx] = 1;
     }
-    nslots = 0;
-    for (int t = 0; t < ntiles; ++t)
-        if (slot[t] == 0) slot[t] = nslots++;
+    return n;
 }
 
 double drive_value(int drive, double u0, double omega, long n) {
@@ -428,12 +432,16 @@ struct lbm_sim {
     std::vector<uint8_t> labels;
     std::vector<LinkNode> link_nodes;  // boundary nodes and their link masks
     size_t n_fluid = 0, n_boundary = 0;
-    double fconst[2] = {0, 0};
+    double fconst[2] = {0, 0}, fmov[2] = {0, 0};
+    int nbf = 0;                       // boundary nodes with body links, first and last row of them
+    int body_row0 = 0, body_row1 = -1;
+    int link_groups = 0;               // force groups of the two-buffer step
     // device memory
     void* buf[2] = {nullptr, nullptr};
     uint8_t* d_cls = nullptr;
     ulonglong2* d_links = nullptr;
-    int* d_tile_slot = nullptr;
+    uint2* d_bnodes = nullptr;
+    unsigned char* d_flinks = nullptr;
     double2* d_partials = nullptr;
     unsigned int* d_ticket = nullptr;
     int* d_err = nullptr;
@@ -488,7 +496,8 @@ void free_sim(lbm_sim* s) {
     cudaFree(s->buf[1]);
     cudaFree(s->d_cls);
     cudaFree(s->d_links);
-    cudaFree(s->d_tile_slot);
+    cudaFree(s->d_bnodes);
+    cudaFree(s->d_flinks);
     cudaFree(s->d_partials);
     cudaFree(s->d_ticket);
     cudaFree(s->d_err);
@@ -497,28 +506,42 @@ void free_sim(lbm_sim* s) {
     delete s;
 }
 
-// (Re)build the per-tile force slots for the current tile shape.
+// Tiles of the current tile shape.
 int setup_tiles(lbm_sim* s) {
-    std::vector<int> slot;
-    tile_slots(s->nx, s->ny, s->bx, s->by, s->link_nodes, slot, s->ntx, s->ntiles, s->nslots);
-    cudaFree(s->d_tile_slot);
-    cudaFree(s->d_partials);
-    s->d_tile_slot = nullptr;
-    s->d_partials = nullptr;
-    int rc = dev_alloc(s, &s->d_tile_slot, slot.size());
-    if (rc) return rc;
-    // two force partials per slot: the in-place even step records the forces of two steps
-    const size_t np = 2 * (size_t)std::max(1, s->nslots);
-    rc = dev_alloc(s, &s->d_partials, np);
-    if (rc) return rc;
-    CUDA_TRY(cudaMemcpy(s->d_tile_slot, slot.data(), slot.size() * sizeof(int), cudaMemcpyHostToDevice));
-    s->h2d_bytes += slot.size() * sizeof(int);
-    CUDA_TRY(cudaMemset(s->d_partials, 0, np * sizeof(double2)));
-    s->dev.tile_slot = s->d_tile_slot;
-    s->dev.partials = s->d_partials;
+    s->ntx = (s->nx + s->bx - 1) / s->bx;
+    s->ntiles = s->ntx * ((s->ny + s->by - 1) / s->by);
+    s->nslots = body_tiles(s->nx, s->ny, s->bx, s->by, s->link_nodes);
     s->dev.ntx = s->ntx;
     s->dev.ntiles = s->ntiles;
-    s->dev.nslots = s->nslots;
+    return LBM_OK;
+}
+
+// Device list of the body's links (FLinks), sorted by direction, then node.
+int setup_flinks(lbm_sim* s) {
+    const size_t plane = (size_t)s->ny * s->pitch;
+    std::vector<size_t> at(s->Q + 1, 0);
+    for (const LinkNode& ln : s->link_nodes)
+        for (uint64_t m = ln.body; m; m &= m - 1) ++at[__builtin_ctzll(m) + 1];
+    for (int i = 0; i < s->Q; ++i) at[i + 1] += at[i];
+    const size_t n = at[s->Q];
+    std::vector<unsigned char> host(kFLinkTable + n * sizeof(uint2), 0);
+    double2* cw = reinterpret_cast<double2*>(host.data());
+    for (int i = 0; i < s->Q; ++i) cw[i] = make_double2(s->lat.c[i][0] * s->lat.w[i], s->lat.c[i][1] * s->lat.w[i]);
+    uint2* list = reinterpret_cast<uint2*>(host.data() + kFLinkTable);
+    for (const LinkNode& ln : s->link_nodes) {
+        const size_t idx = ln.node / (size_t)s->nx * s->pitch + ln.node % (size_t)s->nx;
+        for (uint64_t m = ln.body; m; m &= m - 1) {
+            const int i = __builtin_ctzll(m);
+            list[at[i]++] = make_uint2((unsigned)(s->lat.opp[i] * plane + idx), (unsigned)(i | (s->lat.c[i][0] + 3) << 8));
+        }
+    }
+    s->dev.nfl = (int)n;
+    s->dev.glen = force_group_len((int)n);
+    int rc = dev_alloc(s, &s->d_flinks, host.size());
+    if (rc) return rc;
+    CUDA_TRY(cudaMemcpy(s->d_flinks, host.data(), host.size(), cudaMemcpyHostToDevice));
+    s->h2d_bytes += host.size();
+    s->dev.flinks = s->d_flinks;
     return LBM_OK;
 }
 
@@ -604,6 +627,9 @@ SimView sim_view(const lbm_sim* s) {
     v.bx = s->bx;
     v.by = s->by;
     v.nslots = s->nslots;
+    v.nlf = s->link_groups;
+    v.body_row0 = s->body_row0;
+    v.body_row1 = s->body_row1;
     v.drive = s->geom.drive;
     v.u0 = s->geom.u0;
     v.omega = s->omega;
@@ -781,7 +807,12 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     std::vector<uint8_t> cls;
     build_links(H, nx, ny, s->labels, cls, s->link_nodes, s->n_fluid);
     s->n_boundary = s->link_nodes.size();
-    constant_force(H, s->link_nodes, g.rho0, s->fconst[0], s->fconst[1]);
+    for (const LinkNode& ln : s->link_nodes) {
+        if (!ln.body) continue;
+        s->body_row1 = (int)(ln.node / (size_t)nx);
+        if (s->nbf++ == 0) s->body_row0 = s->body_row1;
+    }
+    constant_force(H, s->link_nodes, g.rho0, s->fconst[0], s->fconst[1], s->fmov[0], s->fmov[1]);
 
     const int align = (int)(128 / es);
     s->pitch = (nx + align - 1) / align * align;
@@ -819,6 +850,7 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     for (int y = 0; y < ny; ++y) std::copy_n(cls.data() + (size_t)y * nx, nx, cls_p.data() + (size_t)y * s->pitch);
     TRY_OR_FREE(dev_alloc(s, &s->d_cls, plane));
     TRY_OR_FREE(dev_alloc(s, &s->d_links, plane));
+    TRY_OR_FREE(dev_alloc(s, &s->d_bnodes, s->link_nodes.size()));
     TRY_OR_FREE(dev_alloc(s, &s->d_ticket, 1));
     TRY_OR_FREE(dev_alloc(s, &s->d_err, 1));
     bool up = cudaMemcpy(s->d_cls, cls_p.data(), plane, cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -826,18 +858,26 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
               cudaMemset(s->d_ticket, 0, sizeof(unsigned)) == cudaSuccess &&
               cudaMemset(s->d_err, 0, sizeof(int)) == cudaSuccess;
     s->h2d_bytes += plane;
+    // list of boundary nodes, body nodes first
+    std::vector<uint2> list(std::max<size_t>(1, s->link_nodes.size()));
     std::vector<ulonglong2> row(s->pitch);
+    size_t body_place = 0, wall_place = (size_t)s->nbf;
     for (size_t k = 0; up && k < s->link_nodes.size();) {
         const size_t y = s->link_nodes[k].node / (size_t)nx;
         std::fill(row.begin(), row.end(), make_ulonglong2(0, 0));
         for (; k < s->link_nodes.size() && s->link_nodes[k].node / (size_t)nx == y; ++k) {
             const LinkNode& ln = s->link_nodes[k];
-            row[ln.node % (size_t)nx] = make_ulonglong2(ln.body, ln.wall);
+            const unsigned x = (unsigned)(ln.node % (size_t)nx);
+            list[ln.body ? body_place++ : wall_place++] = make_uint2(x, (unsigned)y);
+            row[x] = make_ulonglong2(ln.body, ln.wall);
         }
         up = cudaMemcpy(s->d_links + y * s->pitch, row.data(), s->pitch * sizeof(ulonglong2),
                         cudaMemcpyHostToDevice) == cudaSuccess;
         s->h2d_bytes += s->pitch * sizeof(ulonglong2);
     }
+    up = up && cudaMemcpy(s->d_bnodes, list.data(), s->link_nodes.size() * sizeof(uint2), cudaMemcpyHostToDevice) ==
+                   cudaSuccess;
+    s->h2d_bytes += s->link_nodes.size() * sizeof(uint2);
     if (!up) {
         free_sim(s);
         return set_error(LBM_ECUDA, "upload of geometry failed");
@@ -848,7 +888,12 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     d.links = s->d_links;
     d.ticket = s->d_ticket;
     d.err = s->d_err;
+    d.bnodes = s->d_bnodes;
+    d.nb = (int)s->link_nodes.size();
+    d.nbf = s->nbf;
     d.fconst = make_double2(s->fconst[0], s->fconst[1]);
+    const bool mw = g.drive == LBM_DRIVE_WALL && g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
+    d.fmov = mw ? make_double2(s->fmov[0], s->fmov[1]) : make_double2(0.0, 0.0);
     d.plane = (long long)plane;
     d.nx = nx;
     d.ny = ny;
@@ -893,6 +938,19 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
         }
     }
     TRY_OR_FREE(setup_tiles(s));
+    // force groups: by links for the two-buffer bounce-back step, by nodes (32 a group) otherwise
+    const bool by_links = g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
+    if (by_links) TRY_OR_FREE(setup_flinks(s));
+    s->link_groups = by_links ? force_groups(d.nfl, d.glen) : (s->nbf + 31) / 32;
+    d.ngroups = s->aa ? (s->nbf + 31) / 32 : s->link_groups;
+    // (two forces per group: the in-place even step records two steps)
+    const size_t np = 2 * (size_t)std::max(1, d.ngroups);
+    TRY_OR_FREE(dev_alloc(s, &s->d_partials, np));
+    if (cudaMemset(s->d_partials, 0, np * sizeof(double2)) != cudaSuccess) {
+        free_sim(s);
+        return set_error(LBM_ECUDA, "memset");
+    }
+    d.partials = s->d_partials;
     TRY_OR_FREE(ensure_capacity(s, 1024));
     *out = s;
     return LBM_OK;
@@ -966,10 +1024,13 @@ int lbm_step(lbm_sim* s, long n) {
             const int phase = (int)(s->steps_done & 1);
             s->dev.src = s->buf[0];
             s->dev.dst = s->buf[0];
-            s->dev.dv = drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done);
-            s->dev.dv_f = (float)s->dev.dv;
-            s->dev.dv2 = drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done + 1);
-            s->dev.dv2_f = (float)s->dev.dv2;
+            // the drive of the next step, then that of this one
+            set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done + 1));
+            s->dev.dv2 = s->dev.dv;
+            s->dev.dv2_f = s->dev.dv_f;
+            std::copy_n(s->dev.mw, 4, s->dev.mw2);
+            std::copy_n(s->dev.mw_f, 4, s->dev.mw2_f);
+            set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));
             s->dev.stream_off = s->stream_off ? 1 : 0;
             if (s->stream_off) {
                 stream_offset_cx(s, s->U_stream, s->dev.Hl, s->dev.HM);
@@ -987,8 +1048,7 @@ int lbm_step(lbm_sim* s, long n) {
     for (long k = 0; k < n; ++k) {
         s->dev.src = s->buf[s->cur];
         s->dev.dst = s->buf[s->cur ^ 1];
-        s->dev.dv = drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done);
-        s->dev.dv_f = (float)s->dev.dv;
+        set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));
         s->dev.stream_off = s->stream_off ? 1 : 0;
         if (s->stream_off) {
             stream_offset_cx(s, s->U_stream, s->dev.Hl, s->dev.HM);

@@ -6,8 +6,8 @@
 // is already fully reserved, or a loop with a fixed memory budget where an allocation that can fail
 // or stall is not acceptable.  lbm_step itself may allocate (it grows the force history), so these
 // callers step the lattice through this entry point instead: the populations and the force live in
-// buffers the caller owns, and the only other memory the step kernel needs -- its per-tile force
-// partials and the ticket of its last-tile reduction -- lives in one file-scope device array below,
+// buffers the caller owns, and the only other memory the step kernel needs -- its force
+// partials and the ticket of their reduction -- lives in one file-scope device array below,
 // loaded with the library and held by every GPU that uses it until the process exits.
 //
 // The kernel is the library's step kernel itself; only the scratch pointers differ.
@@ -21,9 +21,11 @@
 
 namespace {
 
-// Scratch: LBM_NOALLOC_MAX_SLOTS per-tile force partials (16 B each), then the ticket counter and
-// the non-finite flag.  Shared by every call in the process on a given device.
-constexpr size_t kPartialBytes = (size_t)LBM_NOALLOC_MAX_SLOTS * sizeof(double2);
+// Scratch: the group partials of the force (16 B each), then the ticket counter and the non-finite
+// flag.  With bounce-back walls a step has at most kMaxForceGroups groups; with diffuse walls one per 32
+// nodes with body links, and a geometry is accepted with up to LBM_NOALLOC_MAX_SLOTS tiles holding such
+// nodes, 512 in a tile at most.  Shared by every call in the process on a given device.
+constexpr size_t kPartialBytes = (size_t)LBM_NOALLOC_MAX_SLOTS * 16 * sizeof(double2);
 constexpr size_t kScratchBytes = kPartialBytes + 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -87,8 +89,8 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     P.ticket = reinterpret_cast<unsigned int*>(b + kPartialBytes);
     P.err = reinterpret_cast<int*>(b + kPartialBytes + 128);
     P.force_out = reinterpret_cast<double2*>(force_out);
-    P.dv = drive_value(v.drive, v.u0, v.omega, n);
-    P.dv_f = (float)P.dv;
+    P.ngroups = v.nlf;
+    set_drive(P, drive_value(v.drive, v.u0, v.omega, n));
     P.stream_off = 0;  // caller buffers hold plain scaled deviations: no offsets
     for (int m = 0; m < 4; ++m) P.He[m] = P.Ho[m] = 0.f;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -96,7 +98,7 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     // that never completed); the partials are always written before they are read
     cudaError_t e = cudaMemsetAsync(b + kPartialBytes, 0, 256, st);
     if (e == cudaSuccess) e = fn(P, dim3(v.bx, v.by), st);
-    if (e == cudaSuccess && v.nslots == 0) e = cudaMemsetAsync(force_out, 0, 2 * sizeof(double), st);
+    if (e == cudaSuccess && v.nlf == 0) e = cudaMemsetAsync(force_out, 0, 2 * sizeof(double), st);
     if (cur != v.device) cudaSetDevice(cur);
     if (e != cudaSuccess) return set_error(LBM_ECUDA, "lbm_step_noalloc: %s", cudaGetErrorString(e));
     return LBM_OK;

@@ -17,13 +17,12 @@
 // order, every item a strip waits for was taken earlier by a running block, so the wait always
 // ends; no co-residency of the grid is needed.
 //
-// The force of a step is reduced as in the single-instance kernels (per-tile FP64 slot, fixed-
-// order sum by the last slot tile), into a ring of force slots indexed by n mod kRing, so that
-// tiles of different steps of one instance can be in flight at once; an item of an instance with
-// body links first waits for the sum of step n - kRing to have left its ring entry.
-//
-// Every wait is bounded: a wait that runs out sets a bit of the error word and the block returns
-// (the blocks waiting on its items then run out too); the host reports LBM_ETIMEOUT.
+// The force of a step is summed as in the single-instance kernels (warps over the list of body links,
+// then over the groups, in a fixed order) by work items of its own, which come first among the items of
+// an instance's step: they wait for the bands that hold body links to have finished the previous step,
+// and the strips of those bands wait for them before they overwrite, one step later, the populations the
+// force was read from.  Partials go to a ring entry indexed by n mod kRing, so that the forces of several
+// steps of one instance can be in flight at once.
 //
 // The tile code is that of the single-instance kernels (staged TMA tiles of BX x NR nodes, one
 // thread per column, or plain tiles of 32 x 4 nodes with global loads), so every instance is
@@ -62,8 +61,8 @@ struct alignas(64) PInst {
     const StepConst* steps;    // [nsteps]
     double2* history;          // [nsteps] force of each local step
     int* done;                 // [bands] strips of each band completed, over all steps
-    double2* ring;             // [kRing][nslots] force partials
-    unsigned int* tickets;     // [kRing] slot tiles of the ring entry's step that have finished
+    double2* ring;             // [kRing][ngroups] force partials
+    unsigned int* tickets;     // [kRing] groups of the ring entry's step that have finished
     int* fin;                  // [kRing] 1 + the last step whose force left the entry
     long long start;           // batch step at which local step 0 runs
     long long nsteps;          // local steps to run
@@ -71,7 +70,10 @@ struct alignas(64) PInst {
     int bx, by;                // tile shape in nodes
     int band;                  // tile rows per band (the tiles of one strip)
     int nseg;                  // strips per band (tile columns)
+    int fb0, fb1;              // bands that hold body links (fb0 <= fb1; none: fb0 > fb1)
 };
+
+constexpr int kForceItemGroups = 4;  // force groups per warp of a force item
 
 enum PbPath { PB_STAGED = 0, PB_PLAIN = 1 };
 
@@ -104,49 +106,55 @@ __device__ __forceinline__ int halo_bands(int band, int h, int ny, int R, int (&
     return k;
 }
 
-// Warp 0: wait until every band within reach of band b of the instance has completed local step
-// n - 1, i.e. counted n x nseg strips (lanes 0-3, one band each; only for n >= 1), and until the
-// sum of the force of step n - kRing has left ring entry n mod kRing (lane 4; instances with body
-// links, n >= kRing).
-// Returns false (in every lane) if a wait ran out.
+// One lane: wait until *p has reached `need`; false if the wait ran out.
+__device__ __forceinline__ bool wait_for(const int* p, int need, long long limit) {
+    const long long t0 = clock64();
+    while (true) {
+        if (clock64() - t0 >= limit) return false;  // the clock first: a limit of 0 gives up at once
+        if (ld_acquire(p) >= need) return true;
+        __nanosleep(32);
+    }
+}
+
+// Warp 0, before a strip: wait until every band within reach of band b of the instance has completed
+// local step n - 1, i.e. counted n x nseg strips (lanes 0-3, one band each; only for n >= 1), and, if the
+// band holds body links, until the force of step n - 1 has been read from the populations this step
+// overwrites (lane 4).  Returns false (in every lane) if a wait ran out.
 template <class L>
-__device__ __forceinline__ bool wait_item(const PInst& I, int band, long long n, long long limit) {
+__device__ __forceinline__ bool wait_strip(const PInst& I, int band, long long n, long long limit) {
     int bands[4];
     const int nb = n > 0 ? halo_bands(band, I.band * I.by, I.base.ny, L::R, bands) : 0;
     const int lane = threadIdx.x & 31;
-    const int* p = nullptr;
-    int need = 0;
+    bool ok = true;
     if (lane < nb) {
         int b = bands[0];
 #pragma unroll
         for (int j = 1; j < 4; ++j)
             if (lane == j) b = bands[j];
-        p = I.done + b;
-        need = (int)n * I.nseg;
-    } else if (lane == 4 && I.base.nslots > 0 && n >= kRing) {
-        p = I.fin + (int)(n % kRing);
-        need = (int)(n - kRing + 1);
+        ok = wait_for(I.done + b, (int)n * I.nseg, limit);
+    } else if (lane == 4 && n > 0 && band >= I.fb0 && band <= I.fb1) {
+        ok = wait_for(I.fin + (int)((n - 1) % kRing), (int)n, limit);
     }
+    return __all_sync(0xffffffffu, ok);
+}
+
+// Warp 0, before a force item of local step n: wait until the bands that hold body links have completed
+// step n - 1, and until the force of step n - kRing has left the ring entry.
+__device__ __forceinline__ bool wait_force(const PInst& I, long long n, long long limit) {
+    const int lane = threadIdx.x & 31;
     bool ok = true;
-    if (p) {
-        const long long t0 = clock64();
-        while (true) {
-            if (clock64() - t0 >= limit) {  // the clock first: a limit of 0 gives up at once
-                ok = false;
-                break;
-            }
-            if (ld_acquire(p) >= need) break;
-            __nanosleep(32);
-        }
-    }
+    if (n > 0)
+        for (int b = I.fb0 + lane; ok && b <= I.fb1; b += 32) ok = wait_for(I.done + b, (int)n * I.nseg, limit);
+    if (ok && lane == 0 && n >= kRing) ok = wait_for(I.fin + (int)(n % kRing), (int)(n - kRing + 1), limit);
     return __all_sync(0xffffffffu, ok);
 }
 
 // Launch parameters of the persistent kernel.
 struct PbArgs {
     const PInst* insts;
-    const int4* segs;             // (instance, band, tile column, 0) of every strip
-    int nsegs;                    // strips per batch step
+    const int4* segs;             // per work item of a batch step: (instance, band, tile column, 0) of a
+                                  // strip, (instance, -1, first force group, 0) of a force item
+    int nsegs;                    // work items per batch step
     int nsteps;                   // batch steps of this launch
     long long step0;              // batch step of the launch's first step
     unsigned long long* queue;    // item counter (monotonic over launches)
@@ -208,10 +216,10 @@ __global__ void __launch_bounds__(PbShape<L, ST, COLL, PATH, BX, NR, MINB>::THRE
         const int band = it.y, tx = it.z;
         const int ring = (int)(n % kRing);
         const bool fresh = it.x != s_inst || n != s_n;  // P holds another instance or step
-        // dependencies (warp 0, wait_item); the other warps meanwhile copy the instance's constants
+        // dependencies (warp 0); the other warps meanwhile copy the instance's constants
         // into shared memory
         if (tid < 32) {
-            const bool ok = wait_item<L>(I, band, n, A.limit);
+            const bool ok = band < 0 ? wait_force(I, n, A.limit) : wait_strip<L>(I, band, n, A.limit);
             if (!ok && tid == 0) {
                 atomicOr(A.err, 8);
                 s_fail = 1;
@@ -232,11 +240,10 @@ __global__ void __launch_bounds__(PbShape<L, ST, COLL, PATH, BX, NR, MINB>::THRE
                 I.steps[n].H[tid];
         } else if (tid == nthreads - 1) {
             const StepConst& S = I.steps[n];
-            P.dv = S.dv;
-            P.dv_f = S.dv_f;
+            set_drive(P, S.dv);
             P.src = I.buf[n & 1];
             P.dst = const_cast<void*>(I.buf[(n + 1) & 1]);
-            P.partials = I.ring + (size_t)ring * (size_t)(I.base.nslots > 0 ? I.base.nslots : 1);
+            P.partials = I.ring + (size_t)ring * (size_t)I.base.ngroups;
             P.ticket = I.tickets + ring;
             s_map = &I.maps[n & 1];
             s_force = I.history + n;
@@ -249,12 +256,20 @@ __global__ void __launch_bounds__(PbShape<L, ST, COLL, PATH, BX, NR, MINB>::THRE
         // visible to this block by warp 0's acquire: order the async proxy after it, once per item
         if (PATH == PB_STAGED && tid == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
         __syncthreads();
+        if (band < 0) {
+            // force groups: kForceItemGroups per warp from group it.z
+            const int g0 = it.z + (tid >> 5) * kForceItemGroups;
+            for (int g = g0; g < min(g0 + kForceItemGroups, P.ngroups); ++g)
+                if (link_force<L, ST, true>(P, P.src, g, s_force, tid & 31, [] {}) && (tid & 31) == 0) {
+                    __threadfence();
+                    st_release(s_fin, s_fin_val);
+                }
+            continue;
+        }
         const int ntx = P.ntx;
         const int ty0 = band * I.band, ty1 = min(ty0 + I.band, I.nty);
         for (int ty = ty0; ty < ty1; ++ty) {
             const int t = ty * ntx + tx;
-            const int slot = P.tile_slot[t];
-            double Fx = 0.0, Fy = 0.0;
             if constexpr (PATH == PB_STAGED) {
                 const int x = tx * BX + threadIdx.x;
                 const int yt = ty * NR;
@@ -290,7 +305,7 @@ __global__ void __launch_bounds__(PbShape<L, ST, COLL, PATH, BX, NR, MINB>::THRE
                         gather_smem<G, L, ST>(smem, threadIdx.x, r, h);
                     else
                         gather_global<L, ST, true>(P, static_cast<const ST*>(P.src), x, y, h);
-                    collide_store<L, ST, COLL, 0, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h, Fx, Fy);
+                    tile_node<L, ST, COLL, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h);
                 }
             } else {
                 const int x = tx * 32 + threadIdx.x;
@@ -300,13 +315,9 @@ __global__ void __launch_bounds__(PbShape<L, ST, COLL, PATH, BX, NR, MINB>::THRE
                     if (c != NODE_SOLID) {
                         typename StoreT<ST>::CT h[L::Q];
                         gather_global<L, ST, true>(P, static_cast<const ST*>(P.src), x, y, h);
-                        collide_store<L, ST, COLL, 0, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h, Fx, Fy);
+                        tile_node<L, ST, COLL, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h);
                     }
                 }
-            }
-            if (tile_epilogue(P, slot, s_force, Fx, Fy) && tid == 0) {
-                __threadfence();
-                st_release(s_fin, s_fin_val);
             }
             if (PATH == PB_STAGED) __syncthreads();  // the stage is free for the next tile
         }

@@ -34,9 +34,9 @@ struct LinkNode {
 };
 void build_links(const HostLattice& H, int nx, int ny, const std::vector<uint8_t>& lab, std::vector<uint8_t>& cls,
                  std::vector<LinkNode>& links, size_t& n_fluid);
-void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, double rho0, double& fx, double& fy);
-void tile_slots(int nx, int ny, int bx, int by, const std::vector<LinkNode>& links, std::vector<int>& slot, int& ntx,
-                int& ntiles, int& nslots);
+void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, double rho0, double& fx, double& fy,
+                    double& mx, double& my);
+int body_tiles(int nx, int ny, int bx, int by, const std::vector<LinkNode>& links);
 double drive_value(int drive, double u0, double omega, long n);
 int fit_sincos(const double* fx, size_t stride, long n0, long n1, double omega, double coef[3]);
 
@@ -44,6 +44,8 @@ int fit_sincos(const double* fx, size_t stride, long n0, long n1, double omega, 
 // parameters of its step kernel (device pointers to its geometry arrays included).
 struct SimView {
     int device, Q, storage, collision, nx, ny, pitch, bx, by, nslots, drive;
+    int body_row0, body_row1;  // rows that hold nodes with body links
+    int nlf;                   // force groups of the two-buffer bounce-back step (noalloc)
     double u0, omega;
     InstDev inst;
     void* buf[2];

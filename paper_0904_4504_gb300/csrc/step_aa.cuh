@@ -45,84 +45,95 @@ __device__ __forceinline__ void neighbour_table(const InstDev& P, int x, int y, 
     }
 }
 
-// Collision outputs of one node pushed to their targets.  BND: the node has blocked links, and an
+// Collision outputs of one node pushed to their targets.  BND: the node has blocked links lk, and an
 // output whose link x -> x + c_i is blocked (exactly when pull link opp(i) is) comes back into the
-// node's own slot A[x][opp(i)] with the wall term of step n + 1; its momentum exchange goes to
-// (Gx, Gy), the force of step n + 1.  Bulk nodes push every output without tests.
+// node's own slot A[x][opp(i)] with the wall term of step n + 1; its momentum exchange (less the part
+// of the moving-wall term) is returned, part of the force of step n + 1.  Bulk nodes push every output
+// without tests.
 template <class L, class ST, int COLL, bool BND>
-__device__ __forceinline__ void aa_push(const InstDev& P, ST* A, int idx, const int (&roff)[2 * L::R + 1],
-                                        const int (&col)[2 * L::R + 1], const Coef<typename StoreT<ST>::CT>& C,
-                                        const typename StoreT<ST>::CT (&h)[L::Q], double& Gx, double& Gy) {
+__device__ __forceinline__ double2 aa_push(const InstDev& P, ST* A, int idx, ulonglong2 lk,
+                                           const int (&roff)[2 * L::R + 1], const int (&col)[2 * L::R + 1],
+                                           const Coef<typename StoreT<ST>::CT>& C,
+                                           const typename StoreT<ST>::CT (&h)[L::Q]) {
     using S = StoreT<ST>;
     using T = typename S::CT;
     constexpr int R = L::R;
     const long long plane = P.plane;
     const bool off = sizeof(ST) == 2 && P.stream_off;
-    ulonglong2 lk = make_ulonglong2(0ull, 0ull);
-    if (BND) lk = P.links[idx];
     const unsigned long long blk = lk.x | lk.y;
+    LinkSum G;
 
-    // v: output i relative to the stored state's stream offset (16-bit), as eval_pair returns it
+    // v: output i relative to the stored state's stream offset (16-bit)
     auto push = [&](int i, T v) {
         const int j = opp_of<L>(i);
-        if (BND && ((blk >> j) & 1ull)) {
-            double mw = 0.0;
+        const bool blocked = BND && ((blk >> j) & 1ull);
+        if (BND) {
             const T hi = off ? (T)off_s<L>(P, i) : (T)0;
-            if ((lk.x >> j) & 1ull) {
-                if (P.moving) mw = P.mw_k * cx_of<L>(j) * P.dv2;
-                // the value the two-buffer step would read back: v rounded to the storage type
-                const T own = S::rnd(v) + hi;
-                const double hs = 2.0 * (double)own + mw;
-                const double ws = w_of<L>(j) * P.s;
-                Gx -= cx_of<L>(j) * ws * hs;
-                Gy -= cy_of<L>(j) * ws * hs;
+            const bool body = (lk.x >> j) & 1ull;
+            // the value the two-buffer step would read back: v rounded to the storage type
+            G.add<L>(j, body, vadd(S::rnd(v), hi));
+            T back = vadd(v, hi);
+            const int cx = cx_of<L>(j), m = cx < 0 ? -cx : cx;
+            if (cx && body) {
+                const T term = kconst<T>(P.mw2[m], P.mw2_f[m]);
+                back = cx > 0 ? vadd(back, term) : vsub(back, term);
             }
-            S::st(A + j * plane + idx, v + hi + (T)mw - (off ? (T)off_s<L>(P, j) : (T)0));
-        } else {
-            S::st(A + i * plane + roff[R - cy_of<L>(i)] + col[R - cx_of<L>(i)], v);
+            if (blocked) S::st(A + j * plane + idx, off ? vsub(back, (T)off_s<L>(P, j)) : back);
         }
+        if (!blocked) S::st(A + i * plane + roff[R - cy_of<L>(i)] + col[R - cx_of<L>(i)], v);
     };
-    emit_outputs<L, ST, COLL>(C, h, [&](int i, T v) {
+    emit_outputs<L, ST, COLL, T>(P, C, h, [&](int i, T v) {
         if (i == 0)
             S::st(A + idx, v);
         else
             push(i, v);
     });
+    const double k = -2.0 * P.s;
+    return BND ? make_double2(__dmul_rn(k, G.x), __dmul_rn(k, G.y)) : make_double2(0.0, 0.0);
 }
 
 // Even step of one node: pull h_i = A[x - c_i][opp(i)], wall fix-up from the node's own plane i,
-// collide, push.  (Fx, Fy) gets the force of step n, (Gx, Gy) that of step n + 1.  The neighbour
-// table is built twice, for the pull and again for the push, rather than kept live through the
-// collision (registers).
-template <class L, class ST, int COLL>
-__device__ __forceinline__ void aa_pull_push(const InstDev& P, ST* A, int x, int y, int cls, double& Fx,
-                                             double& Fy, double& Gx, double& Gy) {
+// collide, push.  BND: F[0] gets the node's part of the force of step n, F[1] that of step n + 1.  The
+// neighbour table is built twice, for the pull and again for the push, rather than kept live through
+// the collision (registers).
+template <class L, class ST, int COLL, bool BND>
+__device__ __forceinline__ void aa_pull_push(const InstDev& P, ST* A, int x, int y, ulonglong2 lk, double2 (&F)[2]) {
     using S = StoreT<ST>;
     using T = typename S::CT;
     constexpr int Q = L::Q, R = L::R;
     const long long plane = P.plane;
     const int idx = y * P.pitch + x;
     T h[Q];
-    {
+    if (BND) {
+        gather_boundary<L, ST, OWN_SWAPPED>(P, A, x, y, lk.x | lk.y, h);
+        LinkSum G;
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            T own = h[i];
+            if (sizeof(ST) == 2 && P.stream_off) own = vadd(own, (T)off_l<L>(P, opp_of<L>(i)));
+            G.add<L>(i, (lk.x >> i) & 1ull, own);
+        }
+        const double k = -2.0 * P.s;
+        F[0] = make_double2(__dmul_rn(k, G.x), __dmul_rn(k, G.y));
+    } else {
         int roff[2 * R + 1], col[2 * R + 1];
         neighbour_table<R>(P, x, y, roff, col);
 #pragma unroll
         for (int i = 0; i < Q; ++i)
             h[i] = S::ld(A + opp_of<L>(i) * plane + roff[cy_of<L>(i) + R] + col[cx_of<L>(i) + R]);
     }
-    Coef<T> C;
-    prepare<L, ST, COLL, 0, OWN_SWAPPED>(P, A, x, y, cls, P.dv, P.dv_f, h, Fx, Fy, C);
+    add_offset<L, ST, COLL>(P, lk.x | lk.y, h);
+    if (BND) bb_apply<L, ST, COLL>(P, lk, h);
+    const Coef<T> C = coefficients<L, ST, COLL, T>(P, P.dv, P.dv_f, moments<L, T>(h));
     int roff[2 * R + 1], col[2 * R + 1];
     neighbour_table<R>(P, x, y, roff, col);
-    if (cls == NODE_BOUNDARY)
-        aa_push<L, ST, COLL, true>(P, A, idx, roff, col, C, h, Gx, Gy);
-    else
-        aa_push<L, ST, COLL, false>(P, A, idx, roff, col, C, h, Gx, Gy);
+    const double2 G = aa_push<L, ST, COLL, BND>(P, A, idx, lk, roff, col, C, h);
+    if (BND) F[1] = G;
 }
 
 // Odd step of one node: local read, collide, store directions swapped.
 template <class L, class ST, int COLL>
-__device__ __forceinline__ void aa_local(const InstDev& P, ST* A, int x, int y, int cls) {
+__device__ __forceinline__ void aa_local(const InstDev& P, ST* A, int x, int y) {
     using S = StoreT<ST>;
     using T = typename S::CT;
     constexpr int Q = L::Q;
@@ -131,37 +142,53 @@ __device__ __forceinline__ void aa_local(const InstDev& P, ST* A, int x, int y, 
     T h[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) h[i] = S::ld(A + i * plane + idx);
-    Coef<T> C;
-    double Fx = 0.0, Fy = 0.0;  // no fix-up on this step: stays zero
-    prepare<L, ST, COLL, 0, OWN_NONE>(P, A, x, y, cls, P.dv, P.dv_f, h, Fx, Fy, C);
+    add_offset<L, ST, COLL>(P, 0ull, h);
     // output i goes to plane opp(i)
-    emit_outputs<L, ST, COLL>(C, h, [&](int i, T v) { S::st(A + opp_of<L>(i) * plane + idx, v); });
+    collide_emit<L, ST, COLL, T>(P, P.dv, P.dv_f, h, [&](int i, T v) { S::st(A + opp_of<L>(i) * plane + idx, v); });
 }
 
 // One launch = one step; PHASE 0 the even (pull-push) step, 1 the odd (local) one.  P.dst is the
-// single buffer; force_out[0] and force_out[1] get the forces of steps n and n + 1 (PHASE 0 only).
+// single buffer; force_out[0] and force_out[1] get the forces of steps n and n + 1 (PHASE 0 only).  The
+// even step computes the boundary nodes in blocks of their own (step_kernel.cuh); the odd step knows no
+// links.
 template <class L, class ST, int COLL, int PHASE>
 __global__ void __launch_bounds__(512) step_kernel_aa(const __grid_constant__ InstDev P) {
-    pdl_wait_then_release();
-    const int tile = blockIdx.x;
-    const int slot = P.tile_slot[tile];
-    const int tx = tile % P.ntx, ty = tile / P.ntx;
-    const int x = tx * blockDim.x + threadIdx.x;
-    const int y = ty * blockDim.y + threadIdx.y;
-    const int cls = (x < P.nx && y < P.ny) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
     ST* A = static_cast<ST*>(P.dst);
+    const int nbb = PHASE == 0 ? boundary_blocks(P.nb, blockDim.x * blockDim.y) : 0;
+    if (PHASE == 0 && (int)blockIdx.x < nbb) {
+        const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+        const int lane = tid & 31;
+        const int k = blockIdx.x * (blockDim.x * blockDim.y) + tid;
+        uint2 at = make_uint2(0u, 0u);
+        ulonglong2 lk = make_ulonglong2(0ull, 0ull);
+        if (k < P.nb) {
+            at = P.bnodes[k];
+            lk = P.links[at.y * P.pitch + at.x];
+        }
+        pdl_wait_then_release();
+        double2 F[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+        if (k < P.nb) aa_pull_push<L, ST, COLL, true>(P, A, at.x, at.y, lk, F);
+        const int g = (k - lane) >> 5;
+        if (g < P.ngroups) group_force<2>(P, g, P.force_out, F, 1.0, lane);
+        return;
+    }
+    const int tile = blockIdx.x - nbb;
+    const int x = (tile % P.ntx) * blockDim.x + threadIdx.x;
+    const int y = (tile / P.ntx) * blockDim.y + threadIdx.y;
+    const int cls = (x < P.nx && y < P.ny) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
+    pdl_wait_then_release();
     if (PHASE == 0) {
-        double F[4] = {0.0, 0.0, 0.0, 0.0};
-        if (cls != NODE_SOLID) aa_pull_push<L, ST, COLL>(P, A, x, y, cls, F[0], F[1], F[2], F[3]);
-        tile_epilogue_n<2>(P, slot, P.force_out, F);
+        double2 F[2];
+        if (cls == NODE_BULK) aa_pull_push<L, ST, COLL, false>(P, A, x, y, make_ulonglong2(0ull, 0ull), F);
     } else if (cls != NODE_SOLID) {
-        aa_local<L, ST, COLL>(P, A, x, y, cls);
+        aa_local<L, ST, COLL>(P, A, x, y);
     }
 }
 
 template <class L, class ST, int COLL, int PHASE>
 cudaError_t launch_step_aa(const InstDev& P, dim3 block, cudaStream_t stream) {
-    return launch_pdl(step_kernel_aa<L, ST, COLL, PHASE>, dim3(P.ntiles), block, 0, stream, P);
+    const int nbb = PHASE == 0 ? boundary_blocks(P.nb, block.x * block.y) : 0;
+    return launch_pdl(step_kernel_aa<L, ST, COLL, PHASE>, dim3(P.ntiles + nbb), block, 0, stream, P);
 }
 
 // Launcher of the in-place step for (lattice Q, storage, collision, phase); nullptr if not built.

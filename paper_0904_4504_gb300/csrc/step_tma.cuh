@@ -1,14 +1,13 @@
-// step_tma.cuh -- the fused step with TMA-staged, double-buffered tile loads (sm_103a).
+// step_tma.cuh -- the fused step with TMA-staged tile loads (sm_103a).
 //
-// A persistent CTA walks tiles of BX x BY nodes.  For a tile that lies at least the lattice reach
-// inside the grid, one thread issues Q bulk tensor copies (cp.async.bulk.tensor.3d, one box per
-// direction plane): box i is the BY rows y0 - c_iy .. and the BX + 2 PAD columns x0 - PAD .., so
-// it holds every pulled population h_i(x - c_i) of the tile.  The copies complete on an mbarrier;
-// while they fly the CTA computes the previous tile (STAGES-deep ring).  Threads then read their
-// populations from shared memory at compile-time offsets (no address arithmetic per direction),
-// and run the same bounce-back, collision, store and force code as the plain kernel.  Tiles that
-// touch the periodic edges use the plain wrapped global loads.  The arithmetic is the plain
-// kernel's (same source), so results agree with it to FP32 rounding.
+// A block computes a tile of BX x BY nodes.  For a tile that lies at least the lattice reach inside
+// the grid, one thread issues Q bulk tensor copies (cp.async.bulk.tensor.3d, one box per direction
+// plane): box i is the BY rows y0 - c_iy .. and the BX + 2 PAD columns x0 - PAD .., so it holds every
+// pulled population h_i(x - c_i) of the tile.  The copies complete on an mbarrier.  Threads then read
+// their populations from shared memory at compile-time offsets (no address arithmetic per direction),
+// apply the wall rule to the tile's boundary nodes and run the collision of the plain kernel.  Tiles
+// that touch the periodic edges use the plain wrapped global loads.  Results are the plain kernel's bit
+// for bit (collision.cuh).
 //
 // Every wait on an mbarrier is bounded; a wait that runs out sets bit 2 of the error word, the
 // CTA waits (again bounded) for its own copies in flight and returns.
@@ -84,6 +83,9 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int c0, int
                  : "memory");
 }
 
+// Grid of a staged kernel: force blocks, then one block per tile.
+inline dim3 tile_grid(const InstDev& P, int threads) { return dim3(P.ntiles + force_blocks(P.ngroups, threads)); }
+
 constexpr long long kTmaWaitLimit = 4000000000ll;  // clock cycles (about 2 s)
 
 // Tile t lies at least the lattice reach inside the grid (its boxes need no periodic wrap).
@@ -116,99 +118,6 @@ __device__ __forceinline__ void gather_smem(const unsigned char* stage, int tx, 
     }
 }
 
-// The tiles of one step of one instance, for a persistent CTA: tiles blockIdx.x, +gridDim.x, ...
-// Returns false if a wait timed out (the CTA must return).
-template <class L, class ST, int COLL, class G>
-__device__ __forceinline__ bool run_tiles_tma(const InstDev& P, const CUtensorMap* map, const void* src, void* dst,
-                                              double dv, float dv_f, double2* force_out, unsigned char* smem,
-                                              uint64_t* bars, uint32_t& phase) {
-    const int tid = threadIdx.y * G::BX + threadIdx.x;
-    const int first = blockIdx.x, stride = gridDim.x;
-    unsigned pending = 0;  // stages with copies in flight (thread 0's view)
-    // prologue: the first STAGES-1 tiles of this CTA
-    if (tid == 0) {
-#pragma unroll
-        for (int j = 0; j < G::STAGES - 1; ++j) {
-            const int t = first + j * stride;
-            if (t < P.ntiles && tile_interior<G, L>(P, t)) {
-                issue_tile<G, L>(P, map, t, smem + j * G::STAGE, &bars[j]);
-                pending |= 1u << j;
-            }
-        }
-    }
-    bool ok_all = true;
-    int k = 0;
-    for (int t = first; t < P.ntiles; t += stride, ++k) {
-        const int s = k % G::STAGES;
-        // refill the stage freed by the previous iteration with the tile STAGES-1 ahead
-        if (tid == 0) {
-            const int ks = (k + G::STAGES - 1) % G::STAGES;
-            const int tn = t + (G::STAGES - 1) * stride;
-            if (tn < P.ntiles && tile_interior<G, L>(P, tn)) {
-                issue_tile<G, L>(P, map, tn, smem + ks * G::STAGE, &bars[ks]);
-                pending |= 1u << ks;
-            }
-        }
-        const int tx = t % P.ntx, ty = t / P.ntx;
-        const int x = tx * G::BX + threadIdx.x;
-        const int y = ty * G::BY + threadIdx.y;
-        const int cls = (x < P.nx && y < P.ny) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
-        double Fx = 0.0, Fy = 0.0;
-        typename StoreT<ST>::CT h[L::Q];
-        if (tile_interior<G, L>(P, t)) {
-            const bool ok = mbar_wait(&bars[s], (phase >> s) & 1u, kTmaWaitLimit);
-            phase ^= 1u << s;
-            if (tid == 0) pending &= ~(1u << s);
-            if (!__syncthreads_and(ok)) {
-                ok_all = false;
-                break;
-            }
-            if (cls != NODE_SOLID) {
-                gather_smem<G, L, ST>(smem + s * G::STAGE, threadIdx.x, threadIdx.y, h);
-                collide_store<L, ST, COLL>(P, src, dst, x, y, cls, dv, dv_f, h, Fx, Fy);
-            }
-        } else if (cls != NODE_SOLID) {
-            gather_global<L, ST>(P, static_cast<const ST*>(src), x, y, h);
-            collide_store<L, ST, COLL>(P, src, dst, x, y, cls, dv, dv_f, h, Fx, Fy);
-        }
-        tile_epilogue(P, P.tile_slot[t], force_out, Fx, Fy);
-        __syncthreads();  // stage s may be refilled now
-    }
-    if (!ok_all) {
-        if (tid == 0) {
-            atomicOr(P.err, 4);
-            // wait (bounded) for this CTA's own copies still in flight before its shared memory goes away
-            for (int j = 0; j < G::STAGES; ++j)
-                if (pending & (1u << j)) mbar_wait(&bars[j], (phase >> j) & 1u, kTmaWaitLimit);
-        }
-        __syncthreads();
-        return false;
-    }
-    return true;
-}
-
-template <class G>
-__device__ __forceinline__ void init_bars(uint64_t* bars) {
-    if (threadIdx.x == 0 && threadIdx.y == 0) {
-#pragma unroll
-        for (int j = 0; j < G::STAGES; ++j) mbar_init(&bars[j], 1);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-}
-
-// Single-instance step, persistent CTAs over the tiles.
-template <class L, class ST, int COLL, int STAGES>
-__global__ void __launch_bounds__(256) step_kernel_tma(const __grid_constant__ InstDev P,
-                                                       const __grid_constant__ CUtensorMap map) {
-    using G = TmaGeom<L, ST, STAGES>;
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[STAGES];
-    init_bars<G>(bars);
-    uint32_t phase = 0;
-    run_tiles_tma<L, ST, COLL, G>(P, &map, P.src, P.dst, P.dv, P.dv_f, P.force_out, smem, bars, phase);
-}
-
 // Single-instance step, one block per tile: an interior tile is staged by one set of Q bulk
 // copies, waited for and computed; latency is hidden by the other resident blocks.
 template <class L, class ST, int COLL, int BX, int BY>
@@ -217,14 +126,16 @@ __global__ void __launch_bounds__(BX * BY) step_kernel_tma1(const __grid_constan
     using G = TmaGeom<L, ST, 1, BX, BY>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
+    const int t = (int)blockIdx.x - force_blocks(P.ngroups, blockDim.x * blockDim.y);
+    if (t < 0) {
+        force_block<L, ST>(P, blockIdx.x);
+        return;
+    }
     pdl_wait_then_release();  // before the tile's copies: they read the previous step's output
-    const int t = blockIdx.x;
-    const int slot = P.tile_slot[t];  // read early: the epilogue would otherwise wait for it
     const int tid = threadIdx.y * BX + threadIdx.x;
     const int x = (t % P.ntx) * BX + threadIdx.x;
     const int y = (t / P.ntx) * BY + threadIdx.y;
     const int cls = (x < P.nx && y < P.ny) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
-    double Fx = 0.0, Fy = 0.0;
     typename StoreT<ST>::CT h[L::Q];
     if (tile_interior<G, L>(P, t)) {
         if (tid == 0) {
@@ -244,13 +155,12 @@ __global__ void __launch_bounds__(BX * BY) step_kernel_tma1(const __grid_constan
         }
         if (cls != NODE_SOLID) {
             gather_smem<G, L, ST>(smem, threadIdx.x, threadIdx.y, h);
-            collide_store<L, ST, COLL>(P, P.src, P.dst, x, y, cls, P.dv, P.dv_f, h, Fx, Fy);
+            tile_node<L, ST, COLL>(P, P.src, P.dst, x, y, cls, P.dv, P.dv_f, h);
         }
     } else if (cls != NODE_SOLID) {
         gather_global<L, ST>(P, static_cast<const ST*>(P.src), x, y, h);
-        collide_store<L, ST, COLL>(P, P.src, P.dst, x, y, cls, P.dv, P.dv_f, h, Fx, Fy);
+        tile_node<L, ST, COLL>(P, P.src, P.dst, x, y, cls, P.dv, P.dv_f, h);
     }
-    tile_epilogue(P, slot, P.force_out, Fx, Fy);
 }
 
 // Single-instance step, one block per tile of BX x (NR BY) nodes: the tile is staged by one set of
@@ -265,10 +175,13 @@ __global__ void __launch_bounds__(BX * BY, MINB) step_kernel_tman(const __grid_c
     using G = TmaGeom<L, ST, 1, BX, BY * NR>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
-    // The geometry (tile slots, node classes) is written by the host only: it is read before the
+    // The geometry (node classes) is written by the host only: it is read before the
     // wait for the previous step's grid, while that grid drains.
-    const int t = blockIdx.x;
-    const int slot = P.tile_slot[t];  // read early: the epilogue would otherwise wait for it
+    const int t = (int)blockIdx.x - force_blocks(P.ngroups, blockDim.x * blockDim.y);
+    if (t < 0) {
+        force_block<L, ST>(P, blockIdx.x);
+        return;
+    }
     const int tid = threadIdx.y * BX + threadIdx.x;
     const int x = (t % P.ntx) * BX + threadIdx.x;
     const int yt = (t / P.ntx) * (BY * NR);
@@ -297,7 +210,6 @@ __global__ void __launch_bounds__(BX * BY, MINB) step_kernel_tman(const __grid_c
             return;
         }
     }
-    double Fx = 0.0, Fy = 0.0;
 #pragma unroll 1
     for (int r = 0; r < NR; ++r) {
         const int ty = threadIdx.y + r * BY;
@@ -311,9 +223,8 @@ __global__ void __launch_bounds__(BX * BY, MINB) step_kernel_tman(const __grid_c
             gather_smem<G, L, ST>(smem, threadIdx.x, ty, h);
         else
             gather_global<L, ST>(P, static_cast<const ST*>(P.src), x, y, h);
-        collide_store<L, ST, COLL>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h, Fx, Fy);
+        tile_node<L, ST, COLL>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h);
     }
-    tile_epilogue(P, slot, P.force_out, Fx, Fy);
 }
 
 // Eq. 17 from a staged tile for the two neighbouring nodes (2 tx, 2 tx + 1) of a thread; a
@@ -348,16 +259,18 @@ __global__ void __launch_bounds__(TX * TY) step_kernel_pair(const __grid_constan
     using T = typename S::CT;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
+    const int t = (int)blockIdx.x - force_blocks(P.ngroups, blockDim.x * blockDim.y);
+    if (t < 0) {
+        force_block<L, ST>(P, blockIdx.x);
+        return;
+    }
     pdl_wait_then_release();  // before the tile's copies: they read the previous step's output
-    const int t = blockIdx.x;
-    const int slot = P.tile_slot[t];  // read early: the epilogue would otherwise wait for it
     const int tid = threadIdx.y * TX + threadIdx.x;
     const int x = (t % P.ntx) * (2 * TX) + 2 * threadIdx.x;
     const int y = (t / P.ntx) * TY + threadIdx.y;
     const bool row = y < P.ny;
     const int cls0 = (row && x < P.nx) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
     const int cls1 = (row && x + 1 < P.nx) ? (int)P.cls[y * P.pitch + x + 1] : (int)NODE_SOLID;
-    double Fx = 0.0, Fy = 0.0;
     T h0[L::Q], h1[L::Q];
     if (tile_interior<G, L>(P, t)) {
         if (tid == 0) {
@@ -381,24 +294,21 @@ __global__ void __launch_bounds__(TX * TY) step_kernel_pair(const __grid_constan
         if (cls1 != NODE_SOLID) gather_global<L, ST>(P, static_cast<const ST*>(P.src), x + 1, y, h1);
     }
     if (cls0 != NODE_SOLID || cls1 != NODE_SOLID) {
-        Coef<T> C0, C1;
-        if (cls0 != NODE_SOLID) prepare<L, ST, COLL>(P, P.src, x, y, cls0, P.dv, P.dv_f, h0, Fx, Fy, C0);
-        if (cls1 != NODE_SOLID) prepare<L, ST, COLL>(P, P.src, x + 1, y, cls1, P.dv, P.dv_f, h1, Fx, Fy, C1);
-        const bool f0 = cls0 != NODE_SOLID, f1 = cls1 != NODE_SOLID;
+        // solid nodes keep g = 0 (a stored 0 means h = H there; solid values are never read)
+        T o0[L::Q] = {}, o1[L::Q] = {};
+        if (cls0 != NODE_SOLID) {
+            tile_fixup<L, ST, COLL>(P, P.src, x, y, cls0, h0);
+            collide_emit<L, ST, COLL, T>(P, P.dv, P.dv_f, h0, [&](int i, T v) { o0[i] = v; });
+        }
+        if (cls1 != NODE_SOLID) {
+            tile_fixup<L, ST, COLL>(P, P.src, x + 1, y, cls1, h1);
+            collide_emit<L, ST, COLL, T>(P, P.dv, P.dv_f, h1, [&](int i, T v) { o1[i] = v; });
+        }
         ST* __restrict__ dst = static_cast<ST*>(P.dst) + y * P.pitch + x;
         const long long plane = P.plane;
-        // solid nodes keep g = 0 (a stored 0 means h = H there; solid values are never read)
-        S::st2(dst, f0 ? eval_rest<L, COLL, T>(C0, h0[0]) : (T)0, f1 ? eval_rest<L, COLL, T>(C1, h1[0]) : (T)0);
 #pragma unroll
-        for (int k = 0; k < L::NP; ++k) {
-            T p0 = 0, m0 = 0, p1 = 0, m1 = 0;
-            if (f0) eval_pair<L, COLL, T>(C0, k, h0[1 + 2 * k], h0[2 + 2 * k], p0, m0);
-            if (f1) eval_pair<L, COLL, T>(C1, k, h1[1 + 2 * k], h1[2 + 2 * k], p1, m1);
-            S::st2(dst + (1 + 2 * k) * plane, p0, p1);
-            S::st2(dst + (2 + 2 * k) * plane, m0, m1);
-        }
+        for (int i = 0; i < L::Q; ++i) S::st2(dst + i * plane, o0[i], o1[i]);
     }
-    tile_epilogue(P, slot, P.force_out, Fx, Fy);
 }
 
 template <class L, class ST, int COLL, int TX, int TY>
@@ -411,7 +321,7 @@ cudaError_t launch_step_pair(const InstDev& P, const CUtensorMap& map, const CUt
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    return launch_pdl(step_kernel_pair<L, ST, COLL, TX, TY>, dim3(P.ntiles), dim3(TX, TY), G::SMEM, stream, P, map);
+    return launch_pdl(step_kernel_pair<L, ST, COLL, TX, TY>, tile_grid(P, TX * TY), dim3(TX, TY), G::SMEM, stream, P, map);
 }
 
 // Launch of a staged step: `map` addresses the source buffer with the load boxes, `store_map` the
@@ -429,7 +339,7 @@ cudaError_t launch_step_tma1(const InstDev& P, const CUtensorMap& map, const CUt
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    return launch_pdl(step_kernel_tma1<L, ST, COLL, BX, BY>, dim3(P.ntiles), dim3(BX, BY), G::SMEM, stream, P, map);
+    return launch_pdl(step_kernel_tma1<L, ST, COLL, BX, BY>, tile_grid(P, BX * BY), dim3(BX, BY), G::SMEM, stream, P, map);
 }
 
 template <class L, class ST, int COLL, int BX, int BY, int NR, int MINB>
@@ -442,7 +352,7 @@ cudaError_t launch_step_tman(const InstDev& P, const CUtensorMap& map, const CUt
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    return launch_pdl(step_kernel_tman<L, ST, COLL, BX, BY, NR, MINB>, dim3(P.ntiles), dim3(BX, BY), G::SMEM, stream,
+    return launch_pdl(step_kernel_tman<L, ST, COLL, BX, BY, NR, MINB>, tile_grid(P, BX * BY), dim3(BX, BY), G::SMEM, stream,
                       P, map);
 }
 
@@ -468,14 +378,16 @@ __global__ void __launch_bounds__(BX * BY) step_kernel_tma1s(const __grid_consta
     using T = typename S::CT;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
+    const int t = (int)blockIdx.x - force_blocks(P.ngroups, blockDim.x * blockDim.y);
+    if (t < 0) {
+        force_block<L, ST>(P, blockIdx.x);
+        return;
+    }
     pdl_wait_then_release();  // before the tile's copies: they read the previous step's output
-    const int t = blockIdx.x;
-    const int slot = P.tile_slot[t];  // read early: the epilogue would otherwise wait for it
     const int tid = threadIdx.y * BX + threadIdx.x;
     const int x = (t % P.ntx) * BX + threadIdx.x;
     const int y = (t / P.ntx) * BY + threadIdx.y;
     const int cls = (x < P.nx && y < P.ny) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
-    double Fx = 0.0, Fy = 0.0;
     T h[L::Q];
     if (tile_interior<G, L>(P, t)) {
         if (tid == 0) {
@@ -497,8 +409,9 @@ __global__ void __launch_bounds__(BX * BY) step_kernel_tma1s(const __grid_consta
         const int o = threadIdx.y * BX + threadIdx.x;
         if (cls != NODE_SOLID) {
             gather_smem<G, L, ST>(smem, threadIdx.x, threadIdx.y, h);
-            collide_emit<L, ST, COLL>(P, P.src, x, y, cls, P.dv, P.dv_f, h, Fx, Fy,
-                                      [&](int i, T v) { S::st(reinterpret_cast<ST*>(out + i * O::OSLOT) + o, v); });
+            tile_fixup<L, ST, COLL>(P, P.src, x, y, cls, h);
+            collide_emit<L, ST, COLL, T>(P, P.dv, P.dv_f, h,
+                                         [&](int i, T v) { S::st(reinterpret_cast<ST*>(out + i * O::OSLOT) + o, v); });
         } else {
 #pragma unroll
             for (int i = 0; i < L::Q; ++i) S::st(reinterpret_cast<ST*>(out + i * O::OSLOT) + o, (T)0);
@@ -516,9 +429,8 @@ __global__ void __launch_bounds__(BX * BY) step_kernel_tma1s(const __grid_consta
         }
     } else if (cls != NODE_SOLID) {
         gather_global<L, ST>(P, static_cast<const ST*>(P.src), x, y, h);
-        collide_store<L, ST, COLL>(P, P.src, P.dst, x, y, cls, P.dv, P.dv_f, h, Fx, Fy);
+        tile_node<L, ST, COLL>(P, P.src, P.dst, x, y, cls, P.dv, P.dv_f, h);
     }
-    tile_epilogue(P, slot, P.force_out, Fx, Fy);
 }
 
 template <class L, class ST, int COLL, int BX, int BY>
@@ -532,31 +444,8 @@ cudaError_t launch_step_tma1s(const InstDev& P, const CUtensorMap& map, const CU
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    return launch_pdl(step_kernel_tma1s<L, ST, COLL, BX, BY>, dim3(P.ntiles), dim3(BX, BY), O::SMEM, stream, P, map,
+    return launch_pdl(step_kernel_tma1s<L, ST, COLL, BX, BY>, tile_grid(P, BX * BY), dim3(BX, BY), O::SMEM, stream, P, map,
                       smap);
-}
-
-// Launch with one CTA per SM slot the kernel's shared memory allows (at most one per tile).
-template <class L, class ST, int COLL, int STAGES>
-cudaError_t launch_step_tma(const InstDev& P, const CUtensorMap& map, const CUtensorMap&, cudaStream_t stream) {
-    using G = TmaGeom<L, ST, STAGES>;
-    static int grid_cap = 0;  // per instantiation: SMs x resident CTAs
-    if (!grid_cap) {
-        cudaError_t e = cudaFuncSetAttribute(step_kernel_tma<L, ST, COLL, STAGES>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0, dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel_tma<L, ST, COLL, STAGES>,
-                                                                 G::THREADS, G::SMEM)) != cudaSuccess)
-            return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        grid_cap = per_sm * sms;
-    }
-    const int grid = P.ntiles < grid_cap ? P.ntiles : grid_cap;
-    step_kernel_tma<L, ST, COLL, STAGES><<<grid, dim3(G::BX, G::BY), G::SMEM, stream>>>(P, map);
-    return cudaGetLastError();
 }
 
 }  // namespace lbm

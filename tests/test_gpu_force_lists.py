@@ -1,0 +1,84 @@
+"""Boundary nodes and the force are computed from lists (of boundary nodes, of body links), in blocks of
+32 entries per warp: geometries whose lists are empty, shorter than a warp, exactly full, just over, longer
+than a block or a force group, one-sided (no force) or split between a body and a static wall.  Every kernel
+variant must give the same bits as the plain kernel, and the plain kernel the oracle's force."""
+import numpy as np
+import pytest
+
+import oracle as orc
+from paper_0904_4504_gb300 import lbm as L
+
+from test_gpu_parity import assert_force_close, assert_state_close, run_both
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+
+def _mask(nx, ny, *blocks):
+    m = np.zeros((ny, nx), np.uint8)
+    for label, x0, y0, w, h in blocks:
+        m[y0:y0 + h, x0:x0 + w] = label
+    return m
+
+
+# (lattice, mask): boundary nodes of a w x h block are (w + 2R)(h + 2R) less its corners' unreached nodes
+GEOMETRIES = {
+    "empty": (37, _mask(41, 30)),
+    "wall-only": (37, _mask(41, 30, (2, 10, 8, 9, 7))),
+    "one-body-row-q9": (9, _mask(32, 9, (1, 0, 0, 32, 1))),       # 2 x 32 nodes, 3 links each: 192 links
+    "short-q9": (9, _mask(33, 20, (1, 7, 6, 1, 1))),              # 8 nodes, 8 links
+    "body-and-wall": (37, _mask(131, 47, (1, 20, 17, 14, 11), (2, 80, 5, 30, 29))),
+    "long": (37, _mask(257, 35, (1, 0, 0, 257, 3), (2, 0, 32, 257, 3))),  # over 1028 listed nodes
+    "seam": (37, _mask(70, 41, (1, 0, 0, 5, 4), (1, 65, 0, 5, 4), (1, 0, 37, 5, 4), (1, 65, 37, 5, 4))),
+}
+
+
+def _run(Q, mask, storage, drive, variant, steps=6):
+    ny, nx = mask.shape
+    geom = L.make_geometry(kind=L.LBM_GEOM_MASK, mask=mask, drive=drive, u0=2e-3, eq_order=4 if Q == 37 else 2,
+                           storage=storage)
+    h = L.lbm_create(Q, nx, ny, 0.8, 0.05, geom)
+    try:
+        if variant == "tile":
+            L.lbm_set_tile(h, 64, 3)
+        elif variant is not None:
+            L.lbm_set_variant(h, variant)
+        L.lbm_step(h, steps)
+        return L.lbm_get_state(h), L.lbm_force_history(h)
+    finally:
+        L.lbm_destroy(h)
+
+
+@pytest.mark.parametrize("drive", [L.LBM_DRIVE_WALL, L.LBM_DRIVE_BODYFORCE], ids=["wall", "body"])
+@pytest.mark.parametrize("storage", [L.LBM_STORE_F32, L.LBM_STORE_F16], ids=["f32", "f16"])
+@pytest.mark.parametrize("name", GEOMETRIES)
+def test_variants_agree_bitwise(name, storage, drive):
+    Q, mask = GEOMETRIES[name]
+    g0, F0 = _run(Q, mask, storage, drive, 0)
+    if not (mask == 1).any():
+        assert not F0.any()
+    tried = 0
+    for v in [None, "tile", 1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27, 28, 30]:
+        try:
+            g, F = _run(Q, mask, storage, drive, v)
+        except L.LbmError as e:
+            assert e.code == L.LBM_EINVAL  # not built for this lattice / storage
+            continue
+        tried += 1
+        assert (g == g0).all() and (F == F0).all(), v
+    assert tried >= 4
+
+
+@pytest.mark.parametrize("name", [n for n in GEOMETRIES if n != "wall-only" and n != "empty"])
+def test_force_against_oracle(name):
+    Q, mask = GEOMETRIES[name]
+    ny, nx = mask.shape
+    g_gpu, g_or, F_gpu, F_or, lab, g0 = run_both(Q, nx, ny, 0.8, 0.05, L.LBM_GEOM_MASK, 6, mask=mask,
+                                                 drive=L.LBM_DRIVE_WALL, u0=2e-3, eq_order=4 if Q == 37 else 2,
+                                                 collision=L.LBM_COLL_REGULARIZED, storage=L.LBM_STORE_F64, init_exp=-17,
+                                                 seed=12)
+    assert_state_close(Q, g_gpu, g_or, lab, L.LBM_STORE_F64, 6, g0)
+    assert_force_close(F_gpu, F_or, Q, lab, L.LBM_STORE_F64, 6)
