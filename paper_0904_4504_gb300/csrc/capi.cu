@@ -1032,6 +1032,7 @@ int lbm_step(lbm_sim* s, long n) {
             std::copy_n(s->dev.mw_f, 4, s->dev.mw2_f);
             set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));
             s->dev.stream_off = s->stream_off ? 1 : 0;
+            s->dev.flip = (int)(s->steps_done & 1);
             if (s->stream_off) {
                 stream_offset_cx(s, s->U_stream, s->dev.Hl, s->dev.HM);
                 stream_offset_cx(s, s->U_stream + s->dev.dv, s->dev.Hs, nullptr);
@@ -1050,6 +1051,7 @@ int lbm_step(lbm_sim* s, long n) {
         s->dev.dst = s->buf[s->cur ^ 1];
         set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));
         s->dev.stream_off = s->stream_off ? 1 : 0;
+        s->dev.flip = (int)(s->steps_done & 1);
         if (s->stream_off) {
             stream_offset_cx(s, s->U_stream, s->dev.Hl, s->dev.HM);
             stream_offset_cx(s, s->U_stream + s->dev.dv, s->dev.Hs, nullptr);

@@ -90,6 +90,7 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     P.err = reinterpret_cast<int*>(b + kPartialBytes + 128);
     P.force_out = reinterpret_cast<double2*>(force_out);
     P.ngroups = v.nlf;
+    P.flip = (int)(n & 1);
     set_drive(P, drive_value(v.drive, v.u0, v.omega, n));
     P.stream_off = 0;  // caller buffers hold plain scaled deviations: no offsets
     for (int m = 0; m < 4; ++m) P.He[m] = P.Ho[m] = 0.f;

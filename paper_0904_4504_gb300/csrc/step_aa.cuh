@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(512) step_kernel_aa(const __grid_constant__ In
         if (g < P.ngroups) group_force<2>(P, g, P.force_out, F, 1.0, lane);
         return;
     }
-    const int tile = blockIdx.x - nbb;
+    const int tile = P.flip ? P.ntiles - 1 - (int)(blockIdx.x - nbb) : blockIdx.x - nbb;
     const int x = (tile % P.ntx) * blockDim.x + threadIdx.x;
     const int y = (tile / P.ntx) * blockDim.y + threadIdx.y;
     const int cls = (x < P.nx && y < P.ny) ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;

@@ -406,7 +406,10 @@ template <class L, class ST, int COLL, int WALL>
 __device__ __forceinline__ bool edge_block(const InstDev& P, int threads, int& tile) {
     const int nbb = boundary_blocks(P.nb, threads), nfb = WALL ? 0 : force_blocks(P.ngroups, threads);
     tile = (int)blockIdx.x - nbb - nfb;
-    if (tile >= 0) return false;
+    if (tile >= 0) {
+        if (P.flip) tile = P.ntiles - 1 - tile;
+        return false;
+    }
     if ((int)blockIdx.x < nbb) boundary_block<L, ST, COLL, WALL>(P);
     else force_block<L, ST>(P, blockIdx.x - nbb);
     return true;
