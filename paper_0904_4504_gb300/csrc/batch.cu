@@ -376,12 +376,12 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         // it runs (for staged tiles also the load boxes)
         rc = b->pvariant ? lbm_set_variant(sim, b->pvariant) : lbm_set_tile(sim, 32, 4);
     } else {
-        // default kernels, fastest measured in this mode: for D2Q37, the staged kernel with three
-        // rows per thread (27) for 16-bit storage and the plain kernel with 7 resident blocks per SM
-        // (2) for FP32; 16-bit D2Q9 takes the four-nodes-per-thread kernel (30); else the plain
-        // kernel
+        // default kernels, fastest measured in this mode: for D2Q37 with 16-bit storage the staged
+        // kernel with two nodes per thread (32; plain BGK: the staged one with three rows per thread,
+        // 27), with FP32 the plain kernel with 7 resident blocks per SM (2); 16-bit D2Q9 takes the
+        // four-nodes-per-thread kernel (30); else the plain kernel
         const int want = b->variant >= 0 ? b->variant
-                         : half ? (b->Q == 37 ? 27 : 30)
+                         : half ? (b->Q != 37 ? 30 : b->collision == LBM_COLL_REGULARIZED ? 32 : 27)
                          : (b->Q == 37 && b->storage == LBM_STORE_F32) ? 2 : 0;
         if (want == 0 || lbm_set_variant(sim, want) != LBM_OK) rc = lbm_set_tile(sim, b->bx, b->by);
     }
@@ -625,7 +625,7 @@ int lbm_batch_tune(lbm_batch* b, const lbm_instance_desc* descs, int n, int step
     // (staged 27 and 28, plain 2 and 0) times the strip lengths
     std::vector<lbm_batch_tune_entry> cand;
     if (b->mode == LBM_BATCH_STREAMS) {
-        for (int v : {0, 1, 2, 10, 20, 26, 27, 28, 30}) cand.push_back(lbm_batch_tune_entry{v, 0, 0.0});
+        for (int v : {0, 1, 2, 10, 20, 26, 27, 28, 30, 31, 32}) cand.push_back(lbm_batch_tune_entry{v, 0, 0.0});
     } else {
         for (int v : {27, 28, 2, 0})
             if (find_pbatch_kernel(b->Q, b->storage, b->collision, v).func)

@@ -86,6 +86,8 @@ static bool variant_tile(int variant, int* bx, int* by) {
         case 28: *bx = 128; *by = 3; return true;
         case 20: *bx = 64; *by = 4; return true;
         case 30: *bx = 128; *by = 4; return true;
+        case 31: *bx = 64; *by = 1; return true;
+        case 32: *bx = 128; *by = 2; return true;
         case 21: *bx = 64; *by = 2; return true;
         case 22: *bx = 128; *by = 2; return true;
         default: return false;
@@ -137,7 +139,7 @@ static void* find_launcher(int Q, int storage, int coll) {
 }
 
 StepLaunchFn find_occ_launcher(int Q, int storage, int coll, int variant) {
-    if (Q != 37 || variant < 1 || variant > 4 || !q37_table(storage)) return nullptr;
+    if (Q != 37 || !(variant >= 1 && variant <= 4 || variant == 31) || !q37_table(storage)) return nullptr;
     return reinterpret_cast<StepLaunchFn>(q37_table(storage)->occ(coll, variant));
 }
 
@@ -604,6 +606,38 @@ void stream_offset_eo(const float* H7, float* He, float* Ho) {
     }
 }
 
+// Switch to a kernel variant other than 0 (two-buffer layout, bounce-back walls).
+int use_variant(lbm_sim* s, int variant) {
+    if ((variant >= 1 && variant <= 4) || variant == 30 || variant == 31) {
+        StepLaunchFn f = variant == 30 ? (s->Q == 9 ? reinterpret_cast<StepLaunchFn>(find_q9v_launcher(
+                                                          s->geom.storage, s->geom.collision, variant))
+                                                    : nullptr)
+                                       : find_occ_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
+        if (!f) return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
+        variant_tile(variant, &s->bx, &s->by);
+        s->variant = variant;
+        s->tma_launch = nullptr;
+        s->launch = f;
+        return setup_tiles(s);
+    }
+    int bx, by, bw, pad, rc;
+    TmaStepLaunchFn fn = find_tma_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
+    if (!fn || !variant_tile(variant, &bx, &by))
+        return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
+    tma_box(s->Q, s->geom.storage, bx, &bw, &pad);
+    for (int k = 0; k < 2; ++k) {
+        if ((rc = encode_map(&s->maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bw, by)))
+            return rc;
+        if ((rc = encode_map(&s->store_maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bx, by)))
+            return rc;
+    }
+    s->bx = bx;
+    s->by = by;
+    s->variant = variant;
+    s->tma_launch = fn;
+    return setup_tiles(s);
+}
+
 int check_sim(lbm_sim* s) {
     if (!s) return set_error(LBM_EINVAL, "null simulation");
     CUDA_TRY(cudaSetDevice(s->device));
@@ -919,23 +953,16 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     d.stream_off = s->stream_off ? 1 : 0;
     // default kernel: the fastest measured single-instance form -- for D2Q37 the plain kernel with
     // an occupancy floor on the default 32 x 4 tile (variant 1 for FP32, 2 for 16-bit storage), for
-    // 16-bit D2Q9 the four-nodes-per-thread kernel on 128 x 4 tiles (variant 30)
+    // the regularized collision of 16-bit storage two nodes per thread (31; 32, staged, where the two
+    // buffers hold over 200 MB; step_q37v.cuh has the measurements), for 16-bit D2Q9 the
+    // four-nodes-per-thread kernel on 128 x 4 tiles (variant 30)
     if (!s->aa && g.wall_scheme == LBM_SCHEME_BOUNCEBACK) {
-        if (lattice == LBM_D2Q9 && es == 2) {
-            StepLaunchFn f = reinterpret_cast<StepLaunchFn>(find_q9v_launcher(g.storage, g.collision, 30));
-            if (f) {
-                s->launch = f;
-                s->variant = 30;
-                variant_tile(30, &s->bx, &s->by);
-            }
-        } else {
-            const int v = es == 4 ? 1 : es == 2 ? 2 : 0;
-            StepLaunchFn f = v ? find_occ_launcher(lattice, g.storage, g.collision, v) : nullptr;
-            if (f) {
-                s->launch = f;
-                s->variant = v;
-            }
-        }
+        int v = 0;
+        if (lattice == LBM_D2Q9) v = es == 2 ? 30 : 0;
+        else if (es == 4) v = 1;
+        else if (es == 2)
+            v = g.collision != LBM_COLL_REGULARIZED || nx < 48 ? 2 : 2 * plane * H.Q * es > (size_t)200000000 ? 32 : 31;
+        if (v) TRY_OR_FREE(use_variant(s, v));
     }
     TRY_OR_FREE(setup_tiles(s));
     // force groups: by links for the two-buffer bounce-back step, by nodes (32 a group) otherwise
@@ -978,36 +1005,8 @@ int lbm_set_variant(lbm_sim* s, int variant) {
     if (s->aa) return set_error(LBM_EINVAL, "the in-place (AA) layout runs the plain kernel (variant 0) only");
     if (s->geom.wall_scheme != LBM_SCHEME_BOUNCEBACK)
         return set_error(LBM_EINVAL, "kernel variants are built for bounce-back walls only");
-    if ((variant >= 1 && variant <= 4) || variant == 30) {
-        StepLaunchFn f = variant >= 30 ? (s->Q == 9 ? reinterpret_cast<StepLaunchFn>(find_q9v_launcher(
-                                                          s->geom.storage, s->geom.collision, variant))
-                                                    : nullptr)
-                                       : find_occ_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
-        if (!f) return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
-        CUDA_TRY(cudaStreamSynchronize(s->stream));
-        variant_tile(variant, &s->bx, &s->by);
-        s->variant = variant;
-        s->tma_launch = nullptr;
-        s->launch = f;
-        return setup_tiles(s);
-    }
-    int bx, by, bw, pad;
-    TmaStepLaunchFn fn = find_tma_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
-    if (!fn || !variant_tile(variant, &bx, &by))
-        return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
-    tma_box(s->Q, s->geom.storage, bx, &bw, &pad);
     CUDA_TRY(cudaStreamSynchronize(s->stream));
-    for (int k = 0; k < 2; ++k) {
-        if ((rc = encode_map(&s->maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bw, by)))
-            return rc;
-        if ((rc = encode_map(&s->store_maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bx, by)))
-            return rc;
-    }
-    s->bx = bx;
-    s->by = by;
-    s->variant = variant;
-    s->tma_launch = fn;
-    return setup_tiles(s);
+    return use_variant(s, variant);
 }
 
 int lbm_step(lbm_sim* s, long n) {
@@ -1220,7 +1219,7 @@ int lbm_tune(lbm_sim* s, int steps, lbm_tune_entry* out, int cap, int* n_out) {
     if (steps < 1 || !n_out || (cap > 0 && !out)) return set_error(LBM_EINVAL, "need steps >= 1 and an output");
     // candidates: plain kernel tiles, then every staged variant built for this storage type
     const int tiles[][2] = {{32, 4}, {32, 8}, {64, 2}, {64, 4}, {128, 1}, {32, 2}};
-    const int variants[] = {1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27};
+    const int variants[] = {1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27, 31, 32};
     std::vector<lbm_tune_entry> cand;
     for (auto& t : tiles) cand.push_back(lbm_tune_entry{0, t[0], t[1], 0.0});
     for (int v : variants)

@@ -109,16 +109,17 @@ struct Moments {
     V m0, jx, jy, pxx, pxy, pyy;
 };
 
-template <class L, class V>
-__device__ __forceinline__ Moments<V> moments(const V (&h)[L::Q]) {
+// (h(i): the population that arrived along direction i.)
+template <class L, class V, class H>
+__device__ __forceinline__ Moments<V> moments(H&& h) {
     Moments<V> M;
-    M.m0 = vmulk(L::w0(), h[0]);
+    M.m0 = vmulk(L::w0(), h(0));
 #pragma unroll
     for (int k = 0; k < L::NP; k += 2) {
         const int m = L::px(k), n = L::py(k);
         const double w = L::wp(k);
-        const V sp1 = vadd(h[1 + 2 * k], h[2 + 2 * k]), dm1 = vsub(h[1 + 2 * k], h[2 + 2 * k]);
-        const V sp2 = vadd(h[3 + 2 * k], h[4 + 2 * k]), dm2 = vsub(h[3 + 2 * k], h[4 + 2 * k]);
+        const V a1 = h(1 + 2 * k), b1 = h(2 + 2 * k), a2 = h(3 + 2 * k), b2 = h(4 + 2 * k);
+        const V sp1 = vadd(a1, b1), dm1 = vsub(a1, b1), sp2 = vadd(a2, b2), dm2 = vsub(a2, b2);
         if (n == 0) {
             // (m, 0) and (0, m); the first group starts the sums
             M.m0 = vfmak(w, sp2, vfmak(w, sp1, M.m0));
@@ -265,8 +266,8 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
 // to the stream offset of the stored state when it is on: He and Ho of |c_x| leave the even and odd
 // parts).  Plain BGK reads the pulled populations h (absolute ones), the regularized collision does
 // not.
-template <class L, class ST, int COLL, class V, class Emit>
-__device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C, const V (&h)[L::Q], Emit&& emit) {
+template <class L, class ST, int COLL, class V, class H, class Emit>
+__device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C, H&& h, Emit&& emit) {
     using T = typename Lane<V>::T;
     constexpr int R = L::R;
     constexpr bool H4 = R == 3;
@@ -302,7 +303,8 @@ __device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C,
             emit(i, eq);
         } else {
             // Eq. 14 discretized: f - (f - f^eq)/tau + source
-            V v = vfma(vset<V>(om), vsub(eq, h[i]), h[i]);
+            const V hi = h(i);
+            V v = vfma(vset<V>(om), vsub(eq, hi), hi);
             if (source) v = vadd(v, sign > 0 ? vadd(src_even, src_odd) : vsub(src_even, src_odd));
             emit(i, v);
         }
@@ -310,7 +312,8 @@ __device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C,
     if (REG) {
         emit(0, EA[0]);
     } else {
-        V v = vfma(vset<V>(om), vsub(C.c0, h[0]), h[0]);
+        const V h0 = h(0);
+        V v = vfma(vset<V>(om), vsub(C.c0, h0), h0);
         if (source) v = vadd(v, Sa[0]);
         emit(0, v);
     }

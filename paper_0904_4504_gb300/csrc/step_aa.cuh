@@ -82,7 +82,7 @@ __device__ __forceinline__ double2 aa_push(const InstDev& P, ST* A, int idx, ulo
         }
         if (!blocked) S::st(A + i * plane + roff[R - cy_of<L>(i)] + col[R - cx_of<L>(i)], v);
     };
-    emit_outputs<L, ST, COLL, T>(P, C, h, [&](int i, T v) {
+    emit_outputs<L, ST, COLL, T>(P, C, [&](int i) { return h[i]; }, [&](int i, T v) {
         if (i == 0)
             S::st(A + idx, v);
         else
@@ -124,7 +124,7 @@ __device__ __forceinline__ void aa_pull_push(const InstDev& P, ST* A, int x, int
     }
     add_offset<L, ST, COLL>(P, lk.x | lk.y, h);
     if (BND) bb_apply<L, ST, COLL>(P, lk, h);
-    const Coef<T> C = coefficients<L, ST, COLL, T>(P, P.dv, P.dv_f, moments<L, T>(h));
+    const Coef<T> C = coefficients<L, ST, COLL, T>(P, P.dv, P.dv_f, moments<L, T>([&](int i) { return h[i]; }));
     int roff[2 * R + 1], col[2 * R + 1];
     neighbour_table<R>(P, x, y, roff, col);
     const double2 G = aa_push<L, ST, COLL, BND>(P, A, idx, lk, roff, col, C, h);

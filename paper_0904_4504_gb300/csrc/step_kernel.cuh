@@ -201,8 +201,9 @@ __device__ __forceinline__ void add_offset(const InstDev& P, unsigned long long 
 // that arrived at it: emit(i, v) receives output i in storage units.
 template <class L, class ST, int COLL, class V, class Emit>
 __device__ __forceinline__ void collide_emit(const InstDev& P, double dv, float dv_f, const V (&h)[L::Q], Emit&& emit) {
-    const Coef<V> C = coefficients<L, ST, COLL, V>(P, dv, dv_f, moments<L, V>(h));
-    emit_outputs<L, ST, COLL, V>(P, C, h, emit);
+    const auto at = [&](int i) { return h[i]; };
+    const Coef<V> C = coefficients<L, ST, COLL, V>(P, dv, dv_f, moments<L, V>(at));
+    emit_outputs<L, ST, COLL, V>(P, C, at, emit);
 }
 
 // The same, stored at the node's place (element offset y pitch + x).
@@ -378,12 +379,12 @@ __device__ __forceinline__ void force_block(const InstDev& P, int f) {
 // Boundary blocks of a grid of blocks of `threads`.
 __host__ __device__ inline int boundary_blocks(int nb, int threads) { return (nb + threads - 1) / threads; }
 
-// A boundary block: listed nodes blockIdx.x * threads + thread.  The list and the links (host-written)
-// are read before the wait for the previous step's grid.
+// The b-th boundary block: listed nodes b * threads + thread.  The list and the links (host-written) are
+// read before the wait for the previous step's grid.
 template <class L, class ST, int COLL, int WALL>
-__device__ __forceinline__ void boundary_block(const InstDev& P) {
+__device__ __forceinline__ void boundary_block(const InstDev& P, int b) {
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int k = blockIdx.x * (blockDim.x * blockDim.y) + tid;
+    const int k = b * (blockDim.x * blockDim.y) + tid;
     const bool has = k < P.nb;
     const uint2 at = has ? P.bnodes[k] : make_uint2(0u, 0u);
     const ulonglong2 lk = has ? P.links[at.y * P.pitch + at.x] : make_ulonglong2(0ull, 0ull);
@@ -410,7 +411,7 @@ __device__ __forceinline__ bool edge_block(const InstDev& P, int threads, int& t
         if (P.flip) tile = P.ntiles - 1 - tile;
         return false;
     }
-    if ((int)blockIdx.x < nbb) boundary_block<L, ST, COLL, WALL>(P);
+    if ((int)blockIdx.x < nbb) boundary_block<L, ST, COLL, WALL>(P, blockIdx.x);
     else force_block<L, ST>(P, blockIdx.x - nbb);
     return true;
 }

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "pbatch.cuh"
+#include "step_q37v.cuh"
 
 namespace lbm {
 
@@ -49,7 +50,8 @@ void* q37_plain_ds(int coll) {
 }
 
 // Plain step with an occupancy floor: variant 1 = 6, 2 = 7 blocks of 128 threads per SM; 3, 4 = 7
-// blocks, each thread computing 2 or 4 nodes of its column (tiles of 32 x 8, 32 x 16 nodes).
+// blocks, each thread computing 2 or 4 nodes of its column (tiles of 32 x 8, 32 x 16 nodes); 31 = two
+// neighbouring nodes per thread (16-bit storage, regularized collision).
 template <class ST, int COLL>
 void* q37_occ_c(int variant) {
     switch (variant) {
@@ -57,6 +59,9 @@ void* q37_occ_c(int variant) {
         case 2: return (void*)&launch_step_occ<D2Q37, ST, COLL, 7>;
         case 3: return (void*)&launch_step_occn<D2Q37, ST, COLL, 7, 2>;
         case 4: return (void*)&launch_step_occn<D2Q37, ST, COLL, 7, 4>;
+        case 31:
+            if constexpr (sizeof(ST) == 2 && COLL == COLL_REG) return (void*)&launch_step_pair16<D2Q37, ST, COLL>;
+            return nullptr;
         default: return nullptr;
     }
 }
@@ -65,7 +70,8 @@ void* q37_occ_c(int variant) {
 // 13 = 64 x 2 with the outputs stored through TMA; 18, 23, 24, 25 = several nodes per thread, one
 // row apart: blocks of 64 x 1 (4 rows), 64 x 1 (2 rows), 64 x 1 (4 rows, 10 blocks per SM),
 // 128 x 1 (2 rows) threads; 26, 27 = 64 x 1 threads, 3 rows, at least 12 or 11 blocks per SM;
-// 28 = 128 x 1 threads, 3 rows, 6 blocks per SM.
+// 28 = 128 x 1 threads, 3 rows, 6 blocks per SM; 32 = two neighbouring nodes per thread, 128 x 2 tiles (16-bit
+// storage, regularized collision).
 template <class ST, int COLL>
 void* q37_tma_c(int variant) {
     switch (variant) {
@@ -80,6 +86,9 @@ void* q37_tma_c(int variant) {
         case 26: return (void*)&launch_step_tman<D2Q37, ST, COLL, 64, 1, 3, 12>;
         case 27: return (void*)&launch_step_tman<D2Q37, ST, COLL, 64, 1, 3, 11>;
         case 28: return (void*)&launch_step_tman<D2Q37, ST, COLL, 128, 1, 3, 6>;
+        case 32:
+            if constexpr (sizeof(ST) == 2 && COLL == COLL_REG) return (void*)&launch_step_pair16s<D2Q37, ST, COLL, 64, 2, 9>;
+            return nullptr;
         default: return nullptr;
     }
 }

@@ -15,24 +15,6 @@
 
 namespace lbm {
 
-template <class ST> struct Half16;
-template <> struct Half16<__half> {
-    static __device__ __forceinline__ float lo(unsigned w) { return __half2float(__ushort_as_half((unsigned short)(w & 0xffffu))); }
-    static __device__ __forceinline__ float hi(unsigned w) { return __half2float(__ushort_as_half((unsigned short)(w >> 16))); }
-    static __device__ __forceinline__ unsigned pack(float a, float b) {
-        const __half2 h = __floats2half2_rn(a, b);
-        return *reinterpret_cast<const unsigned*>(&h);
-    }
-};
-template <> struct Half16<__nv_bfloat16> {
-    static __device__ __forceinline__ float lo(unsigned w) { return __uint_as_float(w << 16); }
-    static __device__ __forceinline__ float hi(unsigned w) { return __uint_as_float(w & 0xffff0000u); }
-    static __device__ __forceinline__ unsigned pack(float a, float b) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-        return *reinterpret_cast<const unsigned*>(&h);
-    }
-};
-
 // The source rows of one thread's four nodes: per direction the four stored values of its pulled
 // row (w0: elements 0, 1; w1: elements 2, 3) and the value shifted in by c_x (h(x0 - 1) for
 // c_x = +1, h(x0 + 4) for c_x = -1).

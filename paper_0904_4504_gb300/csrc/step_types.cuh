@@ -53,7 +53,7 @@ struct InstDev {
     int ntiles;
     int flip;                    // 1: the tiles are taken from the last to the first.  lbm_step alternates: the
                                  // step starts with what the previous one wrote last and is still in L2
-                                 // (1024^2 D2Q37 FP32 47.7 -> 45.4 us a step, FP16 34.9 -> 33; 1001 x 777
+                                 // (1024^2 D2Q37 FP32 47.7 -> 45.4 us a step, FP16 30.0 -> 27; 1001 x 777
                                  // in place 42.5 -> 34.8; 2048^2 FP32 186.9 -> 184)
     int eq_order;                // 2 or 4
     int moving;                  // 1: body links carry the moving-wall term (wall drive)
@@ -251,6 +251,25 @@ template <> struct StoreT<__half> {
     }
     static __device__ __forceinline__ void st2(__half* p, float a, float b) {
         *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
+    }
+};
+
+// Two 16-bit values in one word: the lower, the upper, and a word of two rounded FP32 values.
+template <class ST> struct Half16;
+template <> struct Half16<__half> {
+    static __device__ __forceinline__ float lo(unsigned w) { return __low2float(*reinterpret_cast<const __half2*>(&w)); }
+    static __device__ __forceinline__ float hi(unsigned w) { return __high2float(*reinterpret_cast<const __half2*>(&w)); }
+    static __device__ __forceinline__ unsigned pack(float a, float b) {
+        const __half2 h = __floats2half2_rn(a, b);
+        return *reinterpret_cast<const unsigned*>(&h);
+    }
+};
+template <> struct Half16<__nv_bfloat16> {
+    static __device__ __forceinline__ float lo(unsigned w) { return __uint_as_float(w << 16); }
+    static __device__ __forceinline__ float hi(unsigned w) { return __uint_as_float(w & 0xffff0000u); }
+    static __device__ __forceinline__ unsigned pack(float a, float b) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        return *reinterpret_cast<const unsigned*>(&h);
     }
 };
 

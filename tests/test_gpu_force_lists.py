@@ -61,7 +61,7 @@ def test_variants_agree_bitwise(name, storage, drive):
     if not (mask == 1).any():
         assert not F0.any()
     tried = 0
-    for v in [None, "tile", 1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27, 28, 30]:
+    for v in [None, "tile", 1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27, 28, 30, 31, 32]:
         try:
             g, F = _run(Q, mask, storage, drive, v)
         except L.LbmError as e:
