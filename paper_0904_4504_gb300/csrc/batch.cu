@@ -375,6 +375,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         // the instance's tile shape is the persistent kernel's: that of the variant whose tile code
         // it runs (for staged tiles also the load boxes)
         rc = b->pvariant ? lbm_set_variant(sim, b->pvariant) : lbm_set_tile(sim, 32, 4);
+        if (rc == LBM_OK) rc = sim_tile_links(sim);
     } else {
         // default kernels, fastest measured in this mode: for D2Q37 with 16-bit storage the staged
         // kernel with two nodes per thread (32; plain BGK: the staged one with three rows per thread,

@@ -232,42 +232,72 @@ size_t storage_size(int storage) {
 // geometry: labels, node classes and blocked links
 // ---------------------------------------------------------------------------------------------
 
-int build_labels(int Q, int nx, int ny, const lbm_geometry& g, std::vector<uint8_t>& lab) {
-    HostLattice H;
-    host_lattice(Q, H);
-    lab.assign((size_t)nx * ny, 0);
+static uint8_t max_label(const uint8_t* m, int n) {
+    uint8_t v = 0;
+    for (int x = 0; x < n; ++x) v = std::max(v, m[x]);
+    return v;
+}
+
+int check_geometry(const HostLattice& H, int nx, int ny, const lbm_geometry& g) {
     switch (g.kind) {
         case LBM_GEOM_NONE:
-            break;
+            return LBM_OK;
         case LBM_GEOM_PLATE:
             if (ny < 2 * H.R + 1) return set_error(LBM_EINVAL, "plate needs ny >= %d", 2 * H.R + 1);
-            for (int y = 0; y < H.R; ++y)
-                for (int x = 0; x < nx; ++x) {
-                    lab[(size_t)y * nx + x] = LBM_BODY;
-                    lab[(size_t)(ny - 1 - y) * nx + x] = LBM_WALL;
-                }
-            break;
-        case LBM_GEOM_BEAM: {
+            return LBM_OK;
+        case LBM_GEOM_BEAM:
             if (g.lx < 1 || g.ly < 1 || g.lx > nx - 2 * H.R || g.ly > ny - 2 * H.R)
                 return set_error(LBM_EINVAL, "beam %dx%d does not fit a %dx%d box with a %d-node gap", g.lx, g.ly,
                                  nx, ny, H.R);
-            const int x0 = (nx - g.lx) / 2, y0 = (ny - g.ly) / 2;
-            for (int y = y0; y < y0 + g.ly; ++y)
-                for (int x = x0; x < x0 + g.lx; ++x) lab[(size_t)y * nx + x] = LBM_BODY;
-            break;
-        }
+            return LBM_OK;
         case LBM_GEOM_MASK:
             if (!g.mask) return set_error(LBM_EINVAL, "LBM_GEOM_MASK needs a mask");
-            for (size_t k = 0; k < lab.size(); ++k) {
-                if (g.mask[k] > LBM_WALL) return set_error(LBM_EINVAL, "mask label %d at %zu", g.mask[k], k);
-                lab[k] = g.mask[k];
+            for (int y = 0; y < ny; ++y) {
+                if (max_label(g.mask + (size_t)y * nx, nx) <= LBM_WALL) continue;
+                for (size_t k = (size_t)y * nx;; ++k)
+                    if (g.mask[k] > LBM_WALL) return set_error(LBM_EINVAL, "mask label %d at %zu", g.mask[k], k);
             }
-            break;
+            return LBM_OK;
         default:
             return set_error(LBM_EINVAL, "unknown geometry kind %d", g.kind);
     }
-    return LBM_OK;
 }
+
+// Labels of row y of a checked geometry; returns false (row not written) if the row is all fluid.
+bool label_row(const HostLattice& H, int nx, int ny, const lbm_geometry& g, int y, uint8_t* row) {
+    switch (g.kind) {
+        case LBM_GEOM_PLATE:
+            // (the static wall is written last: on the smallest boxes the two do not meet)
+            if (y >= H.R && y < ny - H.R) return false;
+            std::fill_n(row, nx, (uint8_t)(y >= ny - H.R ? LBM_WALL : LBM_BODY));
+            return true;
+        case LBM_GEOM_BEAM: {
+            const int x0 = (nx - g.lx) / 2, y0 = (ny - g.ly) / 2;
+            if (y < y0 || y >= y0 + g.ly) return false;
+            std::fill_n(row, nx, (uint8_t)0);
+            std::fill_n(row + x0, g.lx, (uint8_t)LBM_BODY);
+            return true;
+        }
+        case LBM_GEOM_MASK: {
+            const uint8_t* m = g.mask + (size_t)y * nx;
+            if (!max_label(m, nx)) return false;
+            std::copy_n(m, nx, row);
+            return true;
+        }
+        default:
+            return false;
+    }
+}
+
+// Node classes and blocked links of a geometry.  Only rows within R of a row holding a solid node can
+// have solid or boundary nodes; the others are bulk fluid and are not visited (a large domain around a
+// small body is mostly such rows).
+struct GeomScan {
+    std::vector<int> rows;          // the visited rows, increasing
+    std::vector<uint8_t> cls;       // [rows][nx] NodeClass
+    std::vector<LinkNode> links;    // boundary nodes in increasing node order
+    size_t n_fluid = 0;
+};
 
 static int gcd_int(int a, int b) {
     while (b) {
@@ -279,92 +309,122 @@ static int gcd_int(int a, int b) {
 }
 
 // For every fluid node, the links whose pull source, or a lattice node strictly between source and
-// node, is solid; the first solid node met walking back from the node decides body or wall.  Only
-// rows within R of a row holding a solid node can have solid or boundary nodes; the others are bulk
-// fluid and are not visited (a large domain around a small body is mostly such rows).  `links`
-// lists the boundary nodes in increasing node order.
-void build_links(const HostLattice& H, int nx, int ny, const std::vector<uint8_t>& lab, std::vector<uint8_t>& cls,
-                 std::vector<LinkNode>& links, size_t& n_fluid) {
-    const size_t N = (size_t)nx * ny;
-    cls.assign(N, NODE_BULK);
-    links.clear();
+// node, is solid; the first solid node met walking back from the node decides body or wall.
+void scan_geometry(const HostLattice& H, int nx, int ny, const lbm_geometry& g, GeomScan& out) {
+    const int R = H.R;
     auto wrap = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };  // nx, ny > R
-    // solid within R along x of each node of the rows holding a solid, scattered from the solids
-    std::vector<uint8_t> rowsolid(ny, 0), rownear(N, 0), near(nx);
+    // labels of the rows holding a solid, the solids within R along x of their nodes, and whether a
+    // row's labels are all the same
+    struct Row {
+        int y;
+        bool uniform;
+        int lo, hi;                 // columns [lo, hi) outside of which nothing is near a solid of this row
+    };
+    std::vector<Row> solid;
+    std::vector<int> at(ny, -1);    // y -> index in solid
+    std::vector<uint8_t> lab, near, row(nx);
     size_t n_solid = 0;
     for (int y = 0; y < ny; ++y) {
-        const uint8_t* L = lab.data() + (size_t)y * nx;
-        uint8_t* O = rownear.data() + (size_t)y * nx;
+        if (!label_row(H, nx, ny, g, y, row.data())) continue;
+        at[y] = (int)solid.size();
+        const bool uniform = std::all_of(row.begin(), row.end(), [&](uint8_t l) { return l == row[0]; });
+        lab.insert(lab.end(), row.begin(), row.end());
+        near.resize(lab.size(), 0);
+        uint8_t* O = near.data() + near.size() - nx;
         for (int x = 0; x < nx; ++x) {
-            if (!L[x]) continue;
-            rowsolid[y] = 1;
+            if (!row[x]) continue;
             ++n_solid;
-            for (int d = -H.R; d <= H.R; ++d) O[wrap(x + d, nx)] = 1;
+            for (int d = -R; d <= R; ++d) O[wrap(x + d, nx)] = 1;
+        }
+        const int lo = (int)(std::find(O, O + nx, 1) - O);
+        int hi = nx;
+        while (hi > lo && !O[hi - 1]) --hi;
+        solid.push_back(Row{y, uniform, lo, hi});
+    }
+    out.n_fluid = (size_t)nx * ny - n_solid;
+    out.rows.clear();
+    out.cls.clear();
+    out.links.clear();
+    // nodes of a link walking back from its node, nearest first: (x, y) steps
+    struct Walk {
+        int n, dx[3], dy[3];
+    };
+    std::vector<Walk> walk(H.Q);
+    for (int i = 1; i < H.Q; ++i) {
+        const int cx = H.c[i][0], cy = H.c[i][1], n = gcd_int(std::abs(cx), std::abs(cy));
+        walk[i].n = n;
+        for (int k = 1; k <= n; ++k) {
+            walk[i].dx[k - 1] = -k * cx / n;
+            walk[i].dy[k - 1] = -k * cy / n;
         }
     }
-    n_fluid = N - n_solid;
+    std::vector<uint8_t> visit(ny, 0);
+    for (const Row& r : solid)
+        for (int d = -R; d <= R; ++d) visit[wrap(r.y + d, ny)] = 1;
     for (int y = 0; y < ny; ++y) {
-        // solid within R of each node of row y: the rows within R along y or-ed together
-        bool any = false;
-        for (int d = -H.R; d <= H.R; ++d) any = any || rowsolid[wrap(y + d, ny)];
-        if (!any) continue;
-        std::fill(near.begin(), near.end(), 0);
-        for (int d = -H.R; d <= H.R; ++d) {
-            const int ys = wrap(y + d, ny);
-            if (!rowsolid[ys]) continue;
-            const uint8_t* I = rownear.data() + (size_t)ys * nx;
-            for (int x = 0; x < nx; ++x) near[x] |= I[x];
+        if (!visit[y]) continue;
+        out.rows.push_back(y);
+        const size_t base = out.cls.size();
+        out.cls.resize(base + nx, NODE_BULK);
+        uint8_t* cls = out.cls.data() + base;
+        const uint8_t* L[7];        // label rows y - R .. y + R (null: all fluid)
+        bool uniform = true;
+        int lo = nx, hi = 0;
+        std::fill(row.begin(), row.end(), 0);
+        for (int d = -R; d <= R; ++d) {
+            const int k = at[wrap(y + d, ny)];
+            L[d + R] = k < 0 ? nullptr : lab.data() + (size_t)k * nx;
+            if (k < 0) continue;
+            uniform = uniform && solid[k].uniform;
+            const uint8_t* I = near.data() + (size_t)k * nx;
+            for (int x = solid[k].lo; x < solid[k].hi; ++x) row[x] |= I[x];
+            lo = std::min(lo, solid[k].lo);
+            hi = std::max(hi, solid[k].hi);
         }
-        for (int x = 0; x < nx; ++x) {
-            const size_t node = (size_t)y * nx + x;
-            if (lab[node]) {
-                cls[node] = NODE_SOLID;
+        uint64_t b = 0, w = 0;
+        for (int x = lo; x < hi; ++x) {
+            if (L[R] && L[R][x]) {
+                cls[x] = NODE_SOLID;
                 continue;
             }
-            if (!near[x]) continue;
-            uint64_t b = 0, w = 0;
-            for (int i = 1; i < H.Q; ++i) {
-                const int cx = H.c[i][0], cy = H.c[i][1];
-                const int g = gcd_int(std::abs(cx), std::abs(cy));
-                for (int k = 1; k <= g; ++k) {
-                    const int sx = wrap(x - k * cx / g, nx);
-                    const int sy = wrap(y - k * cy / g, ny);
-                    const uint8_t l = lab[(size_t)sy * nx + sx];
-                    if (l) {
-                        (l == LBM_BODY ? b : w) |= 1ull << i;
-                        break;
+            if (!row[x]) continue;
+            if (x == 0 || !uniform) {  // the nodes of a row among uniform rows all have the same links
+                b = w = 0;
+                for (int i = 1; i < H.Q; ++i)
+                    for (int k = 0; k < walk[i].n; ++k) {
+                        const uint8_t* l = L[walk[i].dy[k] + R];
+                        const uint8_t v = l ? l[wrap(x + walk[i].dx[k], nx)] : 0;
+                        if (v) {
+                            (v == LBM_BODY ? b : w) |= 1ull << i;
+                            break;
+                        }
                     }
-                }
             }
             if (b | w) {
-                cls[node] = NODE_BOUNDARY;
-                links.push_back(LinkNode{node, b, w});
+                cls[x] = NODE_BOUNDARY;
+                out.links.push_back(LinkNode{(size_t)y * nx + x, b, w});
             }
         }
     }
 }
 
 // Geometry-only part of the momentum exchange (the rest populations w_i rho0 bounced on body
-// links), -sum over body links of c_i 2 w_i rho0, and the moving-wall part per unit wall velocity,
+// links, count[i] of direction i), -sum over body links of c_i 2 w_i rho0, and the moving-wall part per unit wall velocity,
 // -sum of c_i c_ix 2 w_i rho0 / theta.
-void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, double rho0, double& fx, double& fy,
+void constant_force(const HostLattice& H, const std::vector<size_t>& count, double rho0, double& fx, double& fy,
                     double& mx, double& my) {
     fx = fy = mx = my = 0.0;
-    for (const LinkNode& ln : links) {
-        const uint64_t b = ln.body;
-        if (!b) continue;
-        for (int i = 1; i < H.Q; ++i)
-            if ((b >> i) & 1ull) {
-                fx -= H.c[i][0] * 2.0 * H.w[i] * rho0;
-                fy -= H.c[i][1] * 2.0 * H.w[i] * rho0;
-                mx -= H.c[i][0] * H.c[i][0] * 2.0 * H.w[i] * rho0 / H.theta;
-                my -= H.c[i][1] * H.c[i][0] * 2.0 * H.w[i] * rho0 / H.theta;
-            }
+    for (int i = 1; i < H.Q; ++i) {
+        const double n = (double)count[i] * 2.0 * H.w[i] * rho0;
+        fx -= H.c[i][0] * n;
+        fy -= H.c[i][1] * n;
+        mx -= H.c[i][0] * H.c[i][0] * n / H.theta;
+        my -= H.c[i][1] * H.c[i][0] * n / H.theta;
     }
 }
 
 // Tiles of bx x by nodes that hold body links.
-int body_tiles(int nx, int ny, int bx, int by, const std::vector<LinkNode>& links) {
+static int body_tiles(int nx, int bx, int by, const std::vector<LinkNode>& links) {
     const int ntx = (nx + bx - 1) / bx;
     std::vector<uint8_t> row(ntx, 0);  // of the current row of tiles (links are in node order)
     int n = 0, at = -1;
@@ -431,23 +491,21 @@ struct lbm_sim {
     lbm_geometry geom{};
     HostLattice lat{};
     size_t esize = 0;
-    std::vector<uint8_t> labels;
+    std::vector<uint8_t> labels;       // LBM_GEOM_MASK: a copy; else filled when first asked for (labels_of)
     std::vector<LinkNode> link_nodes;  // boundary nodes and their link masks
     size_t n_fluid = 0, n_boundary = 0;
     double fconst[2] = {0, 0}, fmov[2] = {0, 0};
     int nbf = 0;                       // boundary nodes with body links, first and last row of them
     int body_row0 = 0, body_row1 = -1;
     int link_groups = 0;               // force groups of the two-buffer step
-    // device memory
+    // device memory: one block for everything small (and the populations, where they are small too)
+    unsigned char* d_block = nullptr;
     void* buf[2] = {nullptr, nullptr};
-    uint8_t* d_cls = nullptr;
-    ulonglong2* d_links = nullptr;
-    uint2* d_bnodes = nullptr;
-    unsigned char* d_flinks = nullptr;
-    double2* d_partials = nullptr;
-    unsigned int* d_ticket = nullptr;
-    int* d_err = nullptr;
+    bool own_buf = false;              // the populations have allocations of their own
     double2* d_history = nullptr;
+    bool own_history = false;          // the history has outgrown the block
+    ulonglong2* d_links = nullptr;     // [ny][pitch] links by node: tile kernels only (ensure_links)
+    int* d_err = nullptr;
     size_t cap = 0;
     size_t device_bytes = 0;
     size_t h2d_bytes = 0, d2h_bytes = 0;  // host<->device traffic over the simulation's life
@@ -456,7 +514,8 @@ struct lbm_sim {
     int cur = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    int bx = 32, by = 4, ntx = 0, ntiles = 0, nslots = 0;
+    int bx = 32, by = 4, ntx = 0, ntiles = 0;
+    mutable int body_tiles = -1, body_tiles_bx = 0, body_tiles_by = 0;  // sim_body_tiles
     int plain_bx = 32, plain_by = 4;   // tile of the plain kernel (lbm_set_tile)
     int variant = 0;                   // 0 plain kernel, else a staged variant (lbm_set_variant)
     bool stream_off = false;           // 16-bit body frame: store h - H(U(n)), see InstDev
@@ -494,42 +553,66 @@ int dev_alloc(lbm_sim* s, T** p, size_t count) {
 void free_sim(lbm_sim* s) {
     if (!s) return;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    cudaFree(s->buf[0]);
-    cudaFree(s->buf[1]);
-    cudaFree(s->d_cls);
+    if (s->own_buf) {
+        cudaFree(s->buf[0]);
+        cudaFree(s->buf[1]);
+    }
+    if (s->own_history) cudaFree(s->d_history);
     cudaFree(s->d_links);
-    cudaFree(s->d_bnodes);
-    cudaFree(s->d_flinks);
-    cudaFree(s->d_partials);
-    cudaFree(s->d_ticket);
-    cudaFree(s->d_err);
-    cudaFree(s->d_history);
+    cudaFree(s->d_block);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     delete s;
+}
+
+// The labels the simulation runs with.
+const std::vector<uint8_t>& labels_of(lbm_sim* s) {
+    if (s->labels.empty()) {
+        s->labels.assign((size_t)s->nx * s->ny, 0);
+        for (int y = 0; y < s->ny; ++y) label_row(s->lat, s->nx, s->ny, s->geom, y, s->labels.data() + (size_t)y * s->nx);
+    }
+    return s->labels;
+}
+
+// Links by node (InstDev::links), which the tile kernels read.
+__global__ void scatter_links(const uint2* nodes, const ulonglong2* links, int n, int pitch, ulonglong2* out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) out[(size_t)nodes[k].y * pitch + nodes[k].x] = links[k];
+}
+
+int ensure_links(lbm_sim* s) {
+    if (s->d_links) return LBM_OK;
+    const size_t plane = (size_t)s->ny * s->pitch;
+    int rc = dev_alloc(s, &s->d_links, plane);
+    if (rc) return rc;
+    CUDA_TRY(cudaMemsetAsync(s->d_links, 0, plane * sizeof(ulonglong2), s->stream));
+    if (s->dev.nb > 0) scatter_links<<<(s->dev.nb + 127) / 128, 128, 0, s->stream>>>(s->dev.bnodes, s->dev.blinks, s->dev.nb, s->pitch, s->d_links);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    s->dev.links = s->d_links;
+    return LBM_OK;
 }
 
 // Tiles of the current tile shape.
 int setup_tiles(lbm_sim* s) {
     s->ntx = (s->nx + s->bx - 1) / s->bx;
     s->ntiles = s->ntx * ((s->ny + s->by - 1) / s->by);
-    s->nslots = body_tiles(s->nx, s->ny, s->bx, s->by, s->link_nodes);
     s->dev.ntx = s->ntx;
     s->dev.ntiles = s->ntiles;
     return LBM_OK;
 }
 
-// Device list of the body's links (FLinks), sorted by direction, then node.
-int setup_flinks(lbm_sim* s) {
+// Bytes of the list of the body's links (InstDev::flinks), and the list, sorted by direction, then node.
+size_t flinks_bytes(size_t n) { return kFLinkTable + n * sizeof(uint2); }
+
+void fill_flinks(const lbm_sim* s, const std::vector<size_t>& count, unsigned char* host) {
     const size_t plane = (size_t)s->ny * s->pitch;
+    double2* cw = reinterpret_cast<double2*>(host);
     std::vector<size_t> at(s->Q + 1, 0);
-    for (const LinkNode& ln : s->link_nodes)
-        for (uint64_t m = ln.body; m; m &= m - 1) ++at[__builtin_ctzll(m) + 1];
-    for (int i = 0; i < s->Q; ++i) at[i + 1] += at[i];
-    const size_t n = at[s->Q];
-    std::vector<unsigned char> host(kFLinkTable + n * sizeof(uint2), 0);
-    double2* cw = reinterpret_cast<double2*>(host.data());
-    for (int i = 0; i < s->Q; ++i) cw[i] = make_double2(s->lat.c[i][0] * s->lat.w[i], s->lat.c[i][1] * s->lat.w[i]);
-    uint2* list = reinterpret_cast<uint2*>(host.data() + kFLinkTable);
+    for (int i = 0; i < s->Q; ++i) {
+        cw[i] = make_double2(s->lat.c[i][0] * s->lat.w[i], s->lat.c[i][1] * s->lat.w[i]);
+        at[i + 1] = at[i] + count[i];
+    }
+    uint2* list = reinterpret_cast<uint2*>(host + kFLinkTable);
     for (const LinkNode& ln : s->link_nodes) {
         const size_t idx = ln.node / (size_t)s->nx * s->pitch + ln.node % (size_t)s->nx;
         for (uint64_t m = ln.body; m; m &= m - 1) {
@@ -537,14 +620,6 @@ int setup_flinks(lbm_sim* s) {
             list[at[i]++] = make_uint2((unsigned)(s->lat.opp[i] * plane + idx), (unsigned)(i | (s->lat.c[i][0] + 3) << 8));
         }
     }
-    s->dev.nfl = (int)n;
-    s->dev.glen = force_group_len((int)n);
-    int rc = dev_alloc(s, &s->d_flinks, host.size());
-    if (rc) return rc;
-    CUDA_TRY(cudaMemcpy(s->d_flinks, host.data(), host.size(), cudaMemcpyHostToDevice));
-    s->h2d_bytes += host.size();
-    s->dev.flinks = s->d_flinks;
-    return LBM_OK;
 }
 
 // Make room for the force history of `need` steps.
@@ -559,9 +634,10 @@ int ensure_capacity(lbm_sim* s, size_t need) {
     const size_t keep = std::min(s->cap, (size_t)s->steps_done + (s->aa ? 1 : 0));
     if (s->d_history && keep > 0)
         CUDA_TRY(cudaMemcpy(hist, s->d_history, keep * sizeof(double2), cudaMemcpyDeviceToDevice));
-    cudaFree(s->d_history);
-    s->device_bytes += (cap - s->cap) * sizeof(double2);
+    if (s->own_history) cudaFree(s->d_history);
+    s->device_bytes += (cap - (s->own_history ? s->cap : 0)) * sizeof(double2);
     s->d_history = hist;
+    s->own_history = true;
     s->cap = cap;
     return LBM_OK;
 }
@@ -631,6 +707,8 @@ int use_variant(lbm_sim* s, int variant) {
         if ((rc = encode_map(&s->store_maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bx, by)))
             return rc;
     }
+    // (32 leaves the boundary nodes to their own blocks; the others' tiles read their links)
+    if (variant != 32 && (rc = ensure_links(s))) return rc;
     s->bx = bx;
     s->by = by;
     s->variant = variant;
@@ -660,7 +738,6 @@ SimView sim_view(const lbm_sim* s) {
     v.pitch = s->pitch;
     v.bx = s->bx;
     v.by = s->by;
-    v.nslots = s->nslots;
     v.nlf = s->link_groups;
     v.body_row0 = s->body_row0;
     v.body_row1 = s->body_row1;
@@ -683,6 +760,17 @@ SimView sim_view(const lbm_sim* s) {
 }
 
 int sim_reserve(lbm_sim* s, size_t steps) { return ensure_capacity(s, steps); }
+
+int sim_tile_links(lbm_sim* s) { return ensure_links(s); }
+
+int sim_body_tiles(const lbm_sim* s) {
+    if (s->body_tiles < 0 || s->body_tiles_bx != s->bx || s->body_tiles_by != s->by) {
+        s->body_tiles = body_tiles(s->nx, s->bx, s->by, s->link_nodes);
+        s->body_tiles_bx = s->bx;
+        s->body_tiles_by = s->by;
+    }
+    return s->body_tiles;
+}
 
 void sim_disable_stream_offset(lbm_sim* s) {
     if (s->steps_done == 0) s->stream_off = false;
@@ -731,21 +819,23 @@ int lbm_geometry_links(int lattice, int nx, int ny, const lbm_geometry* geom, un
     if ((long long)nx * ny > (1ll << 31) / 2) return set_error(LBM_EINVAL, "grid %dx%d too large", nx, ny);
     const size_t N = (size_t)nx * ny;
     if ((cls || body || wall) && count < N) return set_error(LBM_EINVAL, "outputs hold %zu < %zu nodes", count, N);
-    std::vector<uint8_t> lab, c;
-    std::vector<LinkNode> links;
-    size_t nf = 0;
-    int rc = build_labels(lattice, nx, ny, *geom, lab);
+    int rc = check_geometry(H, nx, ny, *geom);
     if (rc) return rc;
-    build_links(H, nx, ny, lab, c, links, nf);
-    if (cls) std::copy(c.begin(), c.end(), cls);
+    GeomScan scan;
+    scan_geometry(H, nx, ny, *geom, scan);
+    if (cls) {
+        std::fill(cls, cls + N, (unsigned char)NODE_BULK);
+        for (size_t k = 0; k < scan.rows.size(); ++k)
+            std::copy_n(scan.cls.data() + k * nx, nx, cls + (size_t)scan.rows[k] * nx);
+    }
     if (body) std::fill(body, body + N, 0ull);
     if (wall) std::fill(wall, wall + N, 0ull);
-    for (const LinkNode& ln : links) {
+    for (const LinkNode& ln : scan.links) {
         if (body) body[ln.node] = ln.body;
         if (wall) wall[ln.node] = ln.wall;
     }
-    if (n_fluid) *n_fluid = nf;
-    if (n_boundary) *n_boundary = links.size();
+    if (n_fluid) *n_fluid = scan.n_fluid;
+    if (n_boundary) *n_boundary = scan.links.size();
     return LBM_OK;
 }
 
@@ -834,20 +924,8 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     s->aa_launch[1] = aa1;
     int rc = cudaGetDevice(&s->device) == cudaSuccess ? LBM_OK : LBM_ECUDA;
     if (rc) { delete s; return set_error(rc, "no CUDA device"); }
-    rc = build_labels(lattice, nx, ny, g, s->labels);
+    rc = check_geometry(H, nx, ny, g);
     if (rc) { delete s; return rc; }
-    g.mask = nullptr;
-    s->geom = g;
-    std::vector<uint8_t> cls;
-    build_links(H, nx, ny, s->labels, cls, s->link_nodes, s->n_fluid);
-    s->n_boundary = s->link_nodes.size();
-    for (const LinkNode& ln : s->link_nodes) {
-        if (!ln.body) continue;
-        s->body_row1 = (int)(ln.node / (size_t)nx);
-        if (s->nbf++ == 0) s->body_row0 = s->body_row1;
-    }
-    constant_force(H, s->link_nodes, g.rho0, s->fconst[0], s->fconst[1], s->fmov[0], s->fmov[1]);
-
     const int align = (int)(128 / es);
     s->pitch = (nx + align - 1) / align * align;
     const size_t plane = (size_t)ny * s->pitch;
@@ -855,6 +933,35 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
         delete s;
         return set_error(LBM_EINVAL, "grid %dx%d: %d x %zu populations exceed 2^32", nx, ny, H.Q, plane);
     }
+    GeomScan scan;
+    scan_geometry(H, nx, ny, g, scan);
+    if (g.kind == LBM_GEOM_MASK) s->labels.assign(g.mask, g.mask + (size_t)nx * ny);
+    g.mask = nullptr;
+    s->geom = g;
+    s->n_fluid = scan.n_fluid;
+    s->link_nodes.swap(scan.links);
+    s->n_boundary = s->link_nodes.size();
+    std::vector<size_t> link_count(H.Q, 0);
+    for (const LinkNode& ln : s->link_nodes) {
+        if (!ln.body) continue;
+        s->body_row1 = (int)(ln.node / (size_t)nx);
+        if (s->nbf++ == 0) s->body_row0 = s->body_row1;
+        for (uint64_t m = ln.body; m; m &= m - 1) ++link_count[__builtin_ctzll(m)];
+    }
+    constant_force(H, link_count, g.rho0, s->fconst[0], s->fconst[1], s->fmov[0], s->fmov[1]);
+
+    InstDev& d = s->dev;
+    const size_t nb = s->link_nodes.size();
+    const bool by_links = g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
+    size_t nfl = 0;
+    for (size_t n : link_count) nfl += by_links ? n : 0;
+    // force groups: by links for the two-buffer bounce-back step, by nodes (32 a group) otherwise
+    d.nb = (int)nb;
+    d.nbf = s->nbf;
+    d.nfl = (int)nfl;
+    d.glen = force_group_len((int)nfl);
+    s->link_groups = by_links ? force_groups(d.nfl, d.glen) : (s->nbf + 31) / 32;
+    d.ngroups = s->aa ? (s->nbf + 31) / 32 : s->link_groups;
 
     if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) {
         delete s;
@@ -871,60 +978,85 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
         }                       \
     } while (0)
 
-    for (int b = 0; b < (s->aa ? 1 : 2); ++b) {
-        TRY_OR_FREE(dev_alloc(s, (char**)&s->buf[b], plane * H.Q * es));
-        if (cudaMemset(s->buf[b], 0, plane * H.Q * es) != cudaSuccess) {
-            free_sim(s);
-            return set_error(LBM_ECUDA, "memset");
-        }
+    // One block: node classes, then the uploaded lists (boundary nodes, their links, body links), then what
+    // starts at zero (group partials -- two forces per group: the in-place even step records two steps --,
+    // ticket, error word, history).  Populations of up to 64 MB join it; larger ones are allocated by
+    // themselves.  (An allocation or its release costs about 30 us, 100 us and more above 256 MB; a grid
+    // of 256^2 took ten of them.)
+    auto up256 = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t pop = up256(plane * H.Q * es), nbuf = s->aa ? 1 : 2;
+    const bool together = nbuf * pop <= (size_t)64 << 20;
+    const size_t o_nodes = up256(plane), o_links = up256(o_nodes + nb * sizeof(uint2));
+    const size_t o_flinks = up256(o_links + nb * sizeof(ulonglong2));
+    const size_t o_zero = up256(o_flinks + (by_links ? flinks_bytes(nfl) : 0));
+    const size_t np = 2 * (size_t)std::max(1, d.ngroups);
+    const size_t o_hist = up256(o_zero + 256 + np * sizeof(double2));
+    s->cap = 1024;
+    const size_t o_pop = up256(o_hist + s->cap * sizeof(double2));
+    const size_t block = o_pop + (together ? nbuf * pop : 0);
+    TRY_OR_FREE(dev_alloc(s, &s->d_block, block));
+    for (size_t k = 0; k < nbuf; ++k) {
+        if (together) s->buf[k] = s->d_block + o_pop + k * pop;
+        else TRY_OR_FREE(dev_alloc(s, (unsigned char**)&s->buf[k], pop));
+        s->own_buf = !together;
     }
-    // node classes in the padded layout (padding solid); link masks zeroed on the device, then only
-    // the rows holding boundary nodes uploaded
-    std::vector<uint8_t> cls_p(plane, NODE_SOLID);
-    for (int y = 0; y < ny; ++y) std::copy_n(cls.data() + (size_t)y * nx, nx, cls_p.data() + (size_t)y * s->pitch);
-    TRY_OR_FREE(dev_alloc(s, &s->d_cls, plane));
-    TRY_OR_FREE(dev_alloc(s, &s->d_links, plane));
-    TRY_OR_FREE(dev_alloc(s, &s->d_bnodes, s->link_nodes.size()));
-    TRY_OR_FREE(dev_alloc(s, &s->d_ticket, 1));
-    TRY_OR_FREE(dev_alloc(s, &s->d_err, 1));
-    bool up = cudaMemcpy(s->d_cls, cls_p.data(), plane, cudaMemcpyHostToDevice) == cudaSuccess &&
-              cudaMemset(s->d_links, 0, plane * sizeof(ulonglong2)) == cudaSuccess &&
-              cudaMemset(s->d_ticket, 0, sizeof(unsigned)) == cudaSuccess &&
-              cudaMemset(s->d_err, 0, sizeof(int)) == cudaSuccess;
-    s->h2d_bytes += plane;
-    // list of boundary nodes, body nodes first
-    std::vector<uint2> list(std::max<size_t>(1, s->link_nodes.size()));
-    std::vector<ulonglong2> row(s->pitch);
+    d.cls = s->d_block;
+    d.bnodes = reinterpret_cast<const uint2*>(s->d_block + o_nodes);
+    d.blinks = reinterpret_cast<const ulonglong2*>(s->d_block + o_links);
+    d.flinks = s->d_block + o_flinks;
+    d.ticket = reinterpret_cast<unsigned int*>(s->d_block + o_zero);
+    d.err = s->d_err = reinterpret_cast<int*>(s->d_block + o_zero + 128);
+    d.partials = reinterpret_cast<double2*>(s->d_block + o_zero + 256);
+    s->d_history = reinterpret_cast<double2*>(s->d_block + o_hist);
+
+    // lists of boundary nodes, body nodes first, and of body links
+    std::vector<unsigned char> host(o_zero - o_nodes, 0);
+    uint2* nodes = reinterpret_cast<uint2*>(host.data());
+    ulonglong2* links = reinterpret_cast<ulonglong2*>(host.data() + (o_links - o_nodes));
     size_t body_place = 0, wall_place = (size_t)s->nbf;
-    for (size_t k = 0; up && k < s->link_nodes.size();) {
-        const size_t y = s->link_nodes[k].node / (size_t)nx;
-        std::fill(row.begin(), row.end(), make_ulonglong2(0, 0));
-        for (; k < s->link_nodes.size() && s->link_nodes[k].node / (size_t)nx == y; ++k) {
-            const LinkNode& ln = s->link_nodes[k];
-            const unsigned x = (unsigned)(ln.node % (size_t)nx);
-            list[ln.body ? body_place++ : wall_place++] = make_uint2(x, (unsigned)y);
-            row[x] = make_ulonglong2(ln.body, ln.wall);
-        }
-        up = cudaMemcpy(s->d_links + y * s->pitch, row.data(), s->pitch * sizeof(ulonglong2),
-                        cudaMemcpyHostToDevice) == cudaSuccess;
-        s->h2d_bytes += s->pitch * sizeof(ulonglong2);
+    for (const LinkNode& ln : s->link_nodes) {
+        const size_t k = ln.body ? body_place++ : wall_place++;
+        nodes[k] = make_uint2((unsigned)(ln.node % (size_t)nx), (unsigned)(ln.node / (size_t)nx));
+        links[k] = make_ulonglong2(ln.body, ln.wall);
     }
-    up = up && cudaMemcpy(s->d_bnodes, list.data(), s->link_nodes.size() * sizeof(uint2), cudaMemcpyHostToDevice) ==
-                   cudaSuccess;
-    s->h2d_bytes += s->link_nodes.size() * sizeof(uint2);
+    if (by_links) fill_flinks(s, link_count, host.data() + (o_flinks - o_nodes));
+
+    // node classes: bulk, the padding solid, then the visited rows, run by run (many runs: all rows at once)
+    cudaStream_t st = s->stream;
+    bool up = cudaMemsetAsync(s->d_block, NODE_BULK, plane, st) == cudaSuccess &&
+              (s->pitch == nx || cudaMemset2DAsync(s->d_block + nx, s->pitch, NODE_SOLID, s->pitch - nx, ny, st) == cudaSuccess);
+    std::vector<std::pair<size_t, size_t>> runs;  // [first, last) of scan.rows
+    for (size_t k = 0; k < scan.rows.size(); ++k) {
+        if (k == 0 || scan.rows[k] != scan.rows[k - 1] + 1) runs.emplace_back(k, k);
+        runs.back().second = k + 1;
+    }
+    if (runs.size() <= 8) {
+        for (const auto& r : runs)
+            up = up && cudaMemcpy2DAsync(s->d_block + (size_t)scan.rows[r.first] * s->pitch, s->pitch,
+                                         scan.cls.data() + r.first * nx, nx, nx, r.second - r.first,
+                                         cudaMemcpyHostToDevice, st) == cudaSuccess;
+        s->h2d_bytes += scan.cls.size();
+    } else {
+        std::vector<uint8_t> all((size_t)nx * ny, NODE_BULK);
+        for (size_t k = 0; k < scan.rows.size(); ++k)
+            std::copy_n(scan.cls.data() + k * nx, nx, all.data() + (size_t)scan.rows[k] * nx);
+        up = up && cudaMemcpy2DAsync(s->d_block, s->pitch, all.data(), nx, nx, ny, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+             cudaStreamSynchronize(st) == cudaSuccess;
+        s->h2d_bytes += all.size();
+    }
+    if (!host.empty())
+        up = up && cudaMemcpyAsync(s->d_block + o_nodes, host.data(), host.size(), cudaMemcpyHostToDevice, st) == cudaSuccess;
+    s->h2d_bytes += host.size();
+    // the geometry is on the device when the call returns (other streams may read it, and the host buffers
+    // end here); the zeroes are in order with the simulation's own work
+    up = up && cudaMemsetAsync(s->d_block + o_zero, 0, o_pop - o_zero, st) == cudaSuccess &&
+         cudaStreamSynchronize(st) == cudaSuccess;
+    for (size_t k = 0; up && k < nbuf; ++k) up = cudaMemsetAsync(s->buf[k], 0, pop, st) == cudaSuccess;
     if (!up) {
         free_sim(s);
         return set_error(LBM_ECUDA, "upload of geometry failed");
     }
 
-    InstDev& d = s->dev;
-    d.cls = s->d_cls;
-    d.links = s->d_links;
-    d.ticket = s->d_ticket;
-    d.err = s->d_err;
-    d.bnodes = s->d_bnodes;
-    d.nb = (int)s->link_nodes.size();
-    d.nbf = s->nbf;
     d.fconst = make_double2(s->fconst[0], s->fconst[1]);
     const bool mw = g.drive == LBM_DRIVE_WALL && g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
     d.fmov = mw ? make_double2(s->fmov[0], s->fmov[1]) : make_double2(0.0, 0.0);
@@ -965,20 +1097,6 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
         if (v) TRY_OR_FREE(use_variant(s, v));
     }
     TRY_OR_FREE(setup_tiles(s));
-    // force groups: by links for the two-buffer bounce-back step, by nodes (32 a group) otherwise
-    const bool by_links = g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
-    if (by_links) TRY_OR_FREE(setup_flinks(s));
-    s->link_groups = by_links ? force_groups(d.nfl, d.glen) : (s->nbf + 31) / 32;
-    d.ngroups = s->aa ? (s->nbf + 31) / 32 : s->link_groups;
-    // (two forces per group: the in-place even step records two steps)
-    const size_t np = 2 * (size_t)std::max(1, d.ngroups);
-    TRY_OR_FREE(dev_alloc(s, &s->d_partials, np));
-    if (cudaMemset(s->d_partials, 0, np * sizeof(double2)) != cudaSuccess) {
-        free_sim(s);
-        return set_error(LBM_ECUDA, "memset");
-    }
-    d.partials = s->d_partials;
-    TRY_OR_FREE(ensure_capacity(s, 1024));
     *out = s;
     return LBM_OK;
 }
@@ -1161,6 +1279,7 @@ int lbm_get_state(lbm_sim* s, double* out, size_t count) {
     if (!out || count != N * s->Q) return set_error(LBM_ERANGE, "need %zu values", N * s->Q);
     if (s->aa && (s->steps_done & 1))
         return set_error(LBM_ERANGE, "the in-place layout holds the state after an even number of steps only");
+    const std::vector<uint8_t>& lab = labels_of(s);
     std::vector<unsigned char> host(plane * s->Q * s->esize);
     CUDA_TRY(cudaMemcpy(host.data(), s->buf[s->cur], host.size(), cudaMemcpyDeviceToHost));
     float H[37] = {0};
@@ -1175,7 +1294,7 @@ int lbm_get_state(lbm_sim* s, double* out, size_t count) {
                 const double v = to_double(host.data(), s->geom.storage, (size_t)pi * plane + (size_t)y * s->pitch + x);
                 // with the stream offset the kernel forms h = stored + H in FP32; do the same here
                 const double h = s->stream_off ? (double)(float)(v + H[i]) : v;
-                out[(size_t)i * N + k] = s->labels[k] ? 0.0 : scale * h;
+                out[(size_t)i * N + k] = lab[k] ? 0.0 : scale * h;
             }
     }
     return rc;
@@ -1188,6 +1307,7 @@ int lbm_set_state(lbm_sim* s, const double* g, size_t count) {
     if (!g || count != N * s->Q) return set_error(LBM_ERANGE, "need %zu values", N * s->Q);
     if (s->aa && (s->steps_done & 1))
         return set_error(LBM_ERANGE, "the in-place layout takes a state after an even number of steps only");
+    const std::vector<uint8_t>& lab = labels_of(s);
     std::vector<unsigned char> host(plane * s->Q * s->esize, 0);
     float H[37] = {0};
     if (s->stream_off) stream_offset(s, s->U_stream, H, nullptr);
@@ -1196,7 +1316,7 @@ int lbm_set_state(lbm_sim* s, const double* g, size_t count) {
         for (int y = 0; y < s->ny; ++y)
             for (int x = 0; x < s->nx; ++x) {
                 const size_t k = (size_t)y * s->nx + x;
-                const double v = s->labels[k] ? 0.0 : g[(size_t)i * N + k] * inv - (double)H[i];
+                const double v = lab[k] ? 0.0 : g[(size_t)i * N + k] * inv - (double)H[i];
                 const int pi = s->aa ? s->lat.opp[i] : i;
                 from_double(host.data(), s->geom.storage, (size_t)pi * plane + (size_t)y * s->pitch + x, v);
             }
@@ -1208,8 +1328,9 @@ int lbm_set_state(lbm_sim* s, const double* g, size_t count) {
 int lbm_get_labels(lbm_sim* s, unsigned char* out, size_t count) {
     int rc = check_sim(s);
     if (rc) return rc;
-    if (!out || count != s->labels.size()) return set_error(LBM_ERANGE, "need %zu labels", s->labels.size());
-    std::memcpy(out, s->labels.data(), count);
+    const std::vector<uint8_t>& lab = labels_of(s);
+    if (!out || count != lab.size()) return set_error(LBM_ERANGE, "need %zu labels", lab.size());
+    std::memcpy(out, lab.data(), count);
     return LBM_OK;
 }
 
@@ -1233,7 +1354,7 @@ int lbm_tune(lbm_sim* s, int steps, lbm_tune_entry* out, int cap, int* n_out) {
     // a clone with the same geometry (as a label mask), parameters and storage
     lbm_geometry g = s->geom;
     g.kind = LBM_GEOM_MASK;
-    g.mask = s->labels.data();
+    g.mask = labels_of(s).data();
     lbm_sim* c = nullptr;
     if ((rc = lbm_create(s->Q, s->nx, s->ny, s->tau, s->omega, &g, &c))) return rc;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

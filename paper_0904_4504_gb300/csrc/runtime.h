@@ -25,25 +25,19 @@ size_t storage_size(int storage);
 int set_error(int code, const char* fmt, ...);
 void clear_error();
 const char* last_error();
-int build_labels(int Q, int nx, int ny, const lbm_geometry& g, std::vector<uint8_t>& lab);
 // A fluid node with blocked links: its offset in the unpadded grid (y nx + x) and link masks (bit i:
 // link i pulls from, or passes through, a solid node of the body, or of a static wall).
 struct LinkNode {
     size_t node;
     uint64_t body, wall;
 };
-void build_links(const HostLattice& H, int nx, int ny, const std::vector<uint8_t>& lab, std::vector<uint8_t>& cls,
-                 std::vector<LinkNode>& links, size_t& n_fluid);
-void constant_force(const HostLattice& H, const std::vector<LinkNode>& links, double rho0, double& fx, double& fy,
-                    double& mx, double& my);
-int body_tiles(int nx, int ny, int bx, int by, const std::vector<LinkNode>& links);
 double drive_value(int drive, double u0, double omega, long n);
 int fit_sincos(const double* fx, size_t stride, long n0, long n1, double omega, double coef[3]);
 
 // What another translation unit may read of a simulation: its layout, tile shape and the launch
 // parameters of its step kernel (device pointers to its geometry arrays included).
 struct SimView {
-    int device, Q, storage, collision, nx, ny, pitch, bx, by, nslots, drive;
+    int device, Q, storage, collision, nx, ny, pitch, bx, by, drive;
     int body_row0, body_row1;  // rows that hold nodes with body links
     int nlf;                   // force groups of the two-buffer bounce-back step (noalloc)
     double u0, omega;
@@ -61,6 +55,10 @@ struct SimView {
 SimView sim_view(const lbm_sim* s);
 // Make room for `steps` entries of force history (may allocate).
 int sim_reserve(lbm_sim* s, size_t steps);
+// Make the links by node that the tile kernels read (may allocate).
+int sim_tile_links(lbm_sim* s);
+// Tiles of the simulation's tile shape that hold body links.
+int sim_body_tiles(const lbm_sim* s);
 // Store plain scaled deviations (no uniform-stream offset); only before the first step.
 void sim_disable_stream_offset(lbm_sim* s);
 // Record that `steps` steps were run on the simulation's buffers by another launcher.

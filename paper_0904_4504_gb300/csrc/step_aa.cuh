@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(512) step_kernel_aa(const __grid_constant__ In
         ulonglong2 lk = make_ulonglong2(0ull, 0ull);
         if (k < P.nb) {
             at = P.bnodes[k];
-            lk = P.links[at.y * P.pitch + at.x];
+            lk = P.blinks[k];
         }
         pdl_wait_then_release();
         double2 F[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};

@@ -387,7 +387,7 @@ __device__ __forceinline__ void boundary_block(const InstDev& P, int b) {
     const int k = b * (blockDim.x * blockDim.y) + tid;
     const bool has = k < P.nb;
     const uint2 at = has ? P.bnodes[k] : make_uint2(0u, 0u);
-    const ulonglong2 lk = has ? P.links[at.y * P.pitch + at.x] : make_ulonglong2(0ull, 0ull);
+    const ulonglong2 lk = has ? P.blinks[k] : make_ulonglong2(0ull, 0ull);
     pdl_wait_then_release();
     const int lane = tid & 31, g = (k - lane) >> 5;
     if (!WALL && !has) return;

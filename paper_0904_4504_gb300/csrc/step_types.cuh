@@ -24,8 +24,8 @@ struct InstDev {
     const void* src;             // h at step n, [Q][ny][pitch]
     void* dst;                   // h at step n+1
     const uint8_t* cls;          // [ny][pitch] NodeClass
-    const ulonglong2* links;     // [ny][pitch]: .x bit i = link i blocked by the body (label 1),
-                                 //              .y bit i = blocked by a static wall (label 2)
+    const ulonglong2* links;     // [ny][pitch] (tile kernels): .x bit i = link i blocked by the body (label
+                                 // 1), .y bit i = blocked by a static wall (label 2)
     double2* partials;           // [ngroups] FP64 force partials of the groups (scratch)
     unsigned int* ticket;        // groups of the current step that have finished (scratch, 0 between
                                  // launches: the last one resets it)
@@ -39,7 +39,9 @@ struct InstDev {
     float mw_f[4], mw2_f[4];
     const uint2* bnodes;         // [nb] (x, y) of the fluid nodes with blocked links: the nodes with body
                                  // links first, then the others, each part in increasing node order
-    const void* flinks;          // body links for the force (FLinks)
+    const ulonglong2* blinks;    // [nb] their links, as in `links`
+    const void* flinks;          // body links for the force (flink_entries)
+    const void* list_pad;
     double2 fconst;              // geometry-only part of the force, -sum c_i 2 w_i rho0
     double2 fmov;                // moving-wall part of the force per unit drive, -sum c_i c_ix 2 w_i rho0 / theta
                                  // (body links, bounce-back, wall drive; 0 otherwise)
