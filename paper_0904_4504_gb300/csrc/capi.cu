@@ -528,6 +528,10 @@ struct lbm_sim {
     CUtensorMap maps[2];               // staged variants: load boxes of buffer k
     CUtensorMap store_maps[2];         // variants 13, 14: the tile's own box in buffer k
     InstDev dev{};
+
+    // Steps run in longer calls leave the sum of their forces to one launch every kForceSteps steps; with many
+    // groups (grids of a thousand nodes a side and more) the sum is no part of a step worth saving.
+    bool defers_forces() const { return !aa && dev.ngroups > 0 && dev.ngroups <= 1024; }
 };
 
 namespace {
@@ -979,8 +983,8 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     } while (0)
 
     // One block: node classes, then the uploaded lists (boundary nodes, their links, body links), then what
-    // starts at zero (group partials -- two forces per group: the in-place even step records two steps --,
-    // ticket, error word, history).  Populations of up to 64 MB join it; larger ones are allocated by
+    // starts at zero (ticket, error word, group partials -- of two steps, which the in-place even step
+    // records, or of the steps summed at once -- and history).  Populations of up to 64 MB join it; larger ones are allocated by
     // themselves.  (An allocation or its release costs about 30 us, 100 us and more above 256 MB; a grid
     // of 256^2 took ten of them.)
     auto up256 = [](size_t v) { return (v + 255) / 256 * 256; };
@@ -989,7 +993,7 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     const size_t o_nodes = up256(plane), o_links = up256(o_nodes + nb * sizeof(uint2));
     const size_t o_flinks = up256(o_links + nb * sizeof(ulonglong2));
     const size_t o_zero = up256(o_flinks + (by_links ? flinks_bytes(nfl) : 0));
-    const size_t np = 2 * (size_t)std::max(1, d.ngroups);
+    const size_t np = (size_t)std::max(1, d.ngroups) * (s->aa ? 2 : s->defers_forces() ? kForceSteps : 1);
     const size_t o_hist = up256(o_zero + 256 + np * sizeof(double2));
     s->cap = 1024;
     const size_t o_pop = up256(o_hist + s->cap * sizeof(double2));
@@ -1163,7 +1167,16 @@ int lbm_step(lbm_sim* s, long n) {
         }
         return LBM_OK;
     }
-    for (long k = 0; k < n; ++k) {
+    // a short call sums each step's force in the step; 8 steps are where one launch for all is worth it
+    const bool defer = s->defers_forces() && n >= 8;
+    unsigned int* const ticket = s->dev.ticket;
+    double2* const partials = s->dev.partials;
+    const long first = s->steps_done;
+    ForceSteps F;
+    F.n = 0;
+    F.scale = s->dev.wall_ds ? 1.0 : -2.0 * s->dev.s;
+    cudaError_t e = cudaSuccess;
+    for (long k = 0; k < n && e == cudaSuccess; ++k) {
         s->dev.src = s->buf[s->cur];
         s->dev.dst = s->buf[s->cur ^ 1];
         set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));
@@ -1175,13 +1188,26 @@ int lbm_step(lbm_sim* s, long n) {
             stream_offset_eo(s->dev.Hs, s->dev.He, s->dev.Ho);
         }
         s->dev.force_out = s->d_history + s->steps_done;
-        const cudaError_t e = s->tma_launch ? s->tma_launch(s->dev, s->maps[s->cur], s->store_maps[s->cur ^ 1], s->stream)
-                                            : s->launch(s->dev, block, s->stream);
-        if (e != cudaSuccess) return set_error(LBM_ECUDA, "step launch: %s", cudaGetErrorString(e));
+        if (defer) {
+            s->dev.ticket = nullptr;
+            s->dev.partials = partials + (size_t)F.n * s->dev.ngroups;
+            F.dv[F.n++] = s->dev.dv;
+        }
+        e = s->tma_launch ? s->tma_launch(s->dev, s->maps[s->cur], s->store_maps[s->cur ^ 1], s->stream)
+                          : s->launch(s->dev, block, s->stream);
+        s->dev.ticket = ticket;
+        s->dev.partials = partials;
+        if (e == cudaSuccess && defer && (F.n == kForceSteps || k + 1 == n)) {
+            F.force_out = s->d_history + first + (k + 1 - F.n);
+            e = launch_pdl(sum_forces, dim3((F.n + 3) / 4), dim3(128), 0, s->stream, s->dev, F);
+            F.n = 0;
+        }
+        if (e != cudaSuccess) break;
         s->cur ^= 1;
         ++s->steps_done;
         if (s->stream_off) s->U_stream += s->dev.dv;
     }
+    if (e != cudaSuccess) return set_error(LBM_ECUDA, "step launch: %s", cudaGetErrorString(e));
     return LBM_OK;
 }
 

@@ -154,22 +154,21 @@ __device__ __forceinline__ void aa_local(const InstDev& P, ST* A, int x, int y) 
 template <class L, class ST, int COLL, int PHASE>
 __global__ void __launch_bounds__(512) step_kernel_aa(const __grid_constant__ InstDev P) {
     ST* A = static_cast<ST*>(P.dst);
-    const int nbb = PHASE == 0 ? boundary_blocks(P.nb, blockDim.x * blockDim.y) : 0;
+    const int nbb = PHASE == 0 ? boundary_blocks(P.nb) : 0;
     if (PHASE == 0 && (int)blockIdx.x < nbb) {
-        const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-        const int lane = tid & 31;
-        const int k = blockIdx.x * (blockDim.x * blockDim.y) + tid;
+        const int lane = threadIdx.y * blockDim.x + threadIdx.x;
+        const int k = blockIdx.x * 32 + lane;
         uint2 at = make_uint2(0u, 0u);
         ulonglong2 lk = make_ulonglong2(0ull, 0ull);
-        if (k < P.nb) {
+        if (lane < 32 && k < P.nb) {
             at = P.bnodes[k];
             lk = P.blinks[k];
         }
         pdl_wait_then_release();
+        if (lane >= 32) return;
         double2 F[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
         if (k < P.nb) aa_pull_push<L, ST, COLL, true>(P, A, at.x, at.y, lk, F);
-        const int g = (k - lane) >> 5;
-        if (g < P.ngroups) group_force<2>(P, g, P.force_out, F, 1.0, lane);
+        if ((int)blockIdx.x < P.ngroups) group_force<2>(P, blockIdx.x, P.force_out, F, 1.0, lane);
         return;
     }
     const int tile = P.flip ? P.ntiles - 1 - (int)(blockIdx.x - nbb) : blockIdx.x - nbb;
@@ -187,7 +186,7 @@ __global__ void __launch_bounds__(512) step_kernel_aa(const __grid_constant__ In
 
 template <class L, class ST, int COLL, int PHASE>
 cudaError_t launch_step_aa(const InstDev& P, dim3 block, cudaStream_t stream) {
-    const int nbb = PHASE == 0 ? boundary_blocks(P.nb, block.x * block.y) : 0;
+    const int nbb = PHASE == 0 ? boundary_blocks(P.nb) : 0;
     return launch_pdl(step_kernel_aa<L, ST, COLL, PHASE>, dim3(P.ntiles + nbb), block, 0, stream, P);
 }
 

@@ -266,28 +266,41 @@ __device__ __forceinline__ double warp_sum2(double x, double y, int lane) {
     return v;
 }
 
-// One warp: the NF forces of the step from the group partials (force f of group g at g NF + f), times
-// scale, plus what depends on the geometry and the drive only.  Lanes 0-15 sum the x and lanes 16-31 the y
-// of every 16th group.
-template <int NF>
-__device__ __forceinline__ void force_sum(const InstDev& P, double2* force_out, double scale, int lane) {
-    __threadfence();
+// One warp: a step's force from its group partials (group g at g stride), times scale, plus what depends
+// on the geometry and the drive only.  Lanes 0-15 sum the x and lanes 16-31 the y of every 16th group.
+__device__ __forceinline__ void force_sum(const InstDev& P, const double2* partials, int stride, double dv,
+                                          double2* force_out, double scale, int lane) {
+    const double* part = reinterpret_cast<const double*>(partials) + (lane >> 4);
+    double v = 0.0;
+    for (int k = lane & 15; k < P.ngroups; k += 16) v = __dadd_rn(v, __ldcg(part + 2 * stride * (size_t)k));
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const double* part = reinterpret_cast<const double*>(P.partials + f) + (lane >> 4);
-        double v = 0.0;
-        for (int k = lane & 15; k < P.ngroups; k += 16) v = __dadd_rn(v, __ldcg(part + 2 * NF * (size_t)k));
-#pragma unroll
-        for (int o = 8; o; o >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, o, 16));
-        if ((lane & 15) == 0) {
-            const bool y = lane >> 4;
-            const double dv = f == 0 ? P.dv : P.dv2;
-            v = __fma_rn(scale, v, __fma_rn(dv, y ? P.fmov.y : P.fmov.x, y ? P.fconst.y : P.fconst.x));
-            if (!isfinite(v)) atomicOr(P.err, 1);
-            reinterpret_cast<double*>(force_out + f)[y] = v;
-        }
+    for (int o = 8; o; o >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, o, 16));
+    if ((lane & 15) == 0) {
+        const bool y = lane >> 4;
+        v = __fma_rn(scale, v, __fma_rn(dv, y ? P.fmov.y : P.fmov.x, y ? P.fconst.y : P.fconst.x));
+        if (!isfinite(v)) atomicOr(P.err, 1);
+        reinterpret_cast<double*>(force_out)[y] = v;
     }
-    if (lane == 0) *P.ticket = 0u;
+}
+
+// The forces of up to kForceSteps consecutive steps, whose kernels left their partials one after another
+// (step k at k ngroups) and no ticket: a warp each.  The wait for a step's last group and its sum
+// (fence, atomic, sum) then stay out of every step: 64^2 D2Q37 FP32 beam 4.1 -> 2.6 us a step, 256^2
+// 5.3 -> 3.9, together with boundary blocks of one warp.  The sums are the same, in the same order.
+constexpr int kForceSteps = 64;
+struct ForceSteps {
+    double dv[kForceSteps];
+    double2* force_out;
+    double scale;
+    int n;
+};
+
+static __global__ void __launch_bounds__(128) sum_forces(const __grid_constant__ InstDev P,
+                                                         const __grid_constant__ ForceSteps F) {
+    const int k = blockIdx.x * 4 + (threadIdx.x >> 5);
+    pdl_wait_then_release();
+    if (k < F.n)
+        force_sum(P, P.partials + (size_t)k * P.ngroups, 1, F.dv[k], F.force_out + k, F.scale, threadIdx.x & 31);
 }
 
 // One warp, force group g: the lanes' parts F into the group's partial; the last group of the step to
@@ -300,12 +313,18 @@ __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* fo
         const double v = warp_sum2(F[f].x, F[f].y, lane);
         if ((lane & 15) == 0) reinterpret_cast<double*>(P.partials + (size_t)g * NF + f)[lane >> 4] = v;
     }
+    if (!P.ticket) return false;  // summed for several steps at once (sum_forces)
     __threadfence();
     __syncwarp();
     unsigned t = 0;
     if (lane == 0) t = atomicAdd(P.ticket, 1u);
     const bool last = __shfl_sync(0xffffffffu, t, 0) == (unsigned)(P.ngroups - 1);
-    if (last) force_sum<NF>(P, force_out, scale, lane);
+    if (last) {
+        __threadfence();
+#pragma unroll
+        for (int f = 0; f < NF; ++f) force_sum(P, P.partials + f, NF, f == 0 ? P.dv : P.dv2, force_out + f, scale, lane);
+        if (lane == 0) *P.ticket = 0u;
+    }
     return last;
 }
 
@@ -372,25 +391,25 @@ __device__ __forceinline__ void force_block(const InstDev& P, int f) {
 // others compute bulk nodes only and need no links.  With wall rule and force inside the tiles, a
 // warp next to the body took every lane's links in turn, ten FP64 instructions each, and that chain was
 // the step of a small grid (256^2 D2Q37 FP32, 32 x 32 beam: 18.4 us a launch, the FP64 pipe of one SM
-// 89 % busy and the chip at an IPC of 1.03).  Per step, in back-to-back launches: 64^2 13.8 -> 4.1 us,
-// 256^2 15.0 -> 5.3, 512^2 19.3 -> 9.2, 1024^2 50.1 -> 47.5; 32 x 4096 plate 14.9 -> 5.8, with diffuse
-// walls (force still node by node) 19.2 -> 8.9.
+// 89 % busy and the chip at an IPC of 1.03).  Per step, in back-to-back launches: 64^2 13.8 -> 2.6 us,
+// 256^2 15.0 -> 3.9, 512^2 19.3 -> 9.2; 32 x 4096 plate 14.9 -> 5.2, with diffuse walls (force still node
+// by node) 19.2 -> 7.8.
 
-// Boundary blocks of a grid of blocks of `threads`.
-__host__ __device__ inline int boundary_blocks(int nb, int threads) { return (nb + threads - 1) / threads; }
+// Boundary blocks of a grid: one warp of listed nodes each (further warps leave), since their scattered
+// loads are bound by the SM's L1: four warps on one SM take four times as long as on four.
+__host__ __device__ inline int boundary_blocks(int nb) { return (nb + 31) / 32; }
 
-// The b-th boundary block: listed nodes b * threads + thread.  The list and the links (host-written) are
-// read before the wait for the previous step's grid.
+// The b-th boundary block: listed nodes 32 b + lane.  The list and the links (host-written) are read before
+// the wait for the previous step's grid.
 template <class L, class ST, int COLL, int WALL>
 __device__ __forceinline__ void boundary_block(const InstDev& P, int b) {
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int k = b * (blockDim.x * blockDim.y) + tid;
-    const bool has = k < P.nb;
+    const int lane = threadIdx.y * blockDim.x + threadIdx.x;
+    const int k = 32 * b + lane;
+    const bool has = lane < 32 && k < P.nb;
     const uint2 at = has ? P.bnodes[k] : make_uint2(0u, 0u);
     const ulonglong2 lk = has ? P.blinks[k] : make_ulonglong2(0ull, 0ull);
     pdl_wait_then_release();
-    const int lane = tid & 31, g = (k - lane) >> 5;
-    if (!WALL && !has) return;
+    if (lane >= 32 || (!WALL && !has)) return;
     double2 F[1] = {make_double2(0.0, 0.0)};
     typename StoreT<ST>::CT h[L::Q];
     gather_boundary<L, ST>(P, static_cast<const ST*>(P.src), at.x, at.y, lk.x | lk.y, h);
@@ -398,14 +417,14 @@ __device__ __forceinline__ void boundary_block(const InstDev& P, int b) {
     if (WALL) F[0] = ds_apply<L, ST, COLL>(P, lk, P.dv, P.dv_f, h);  // whole warps: votes
     else bb_apply<L, ST, COLL>(P, lk, h);
     if (has) collide_store<L, ST, COLL>(P, P.dst, at.x, at.y, P.dv, P.dv_f, h);
-    if (WALL && g < P.ngroups) group_force<1>(P, g, P.force_out, F, 1.0, lane);
+    if (WALL && b < P.ngroups) group_force<1>(P, b, P.force_out, F, 1.0, lane);
 }
 
 // Blocks of a grid before the bulk tiles: boundary blocks, then force blocks.  Returns true if this block
 // was one of them, else its tile.
 template <class L, class ST, int COLL, int WALL>
 __device__ __forceinline__ bool edge_block(const InstDev& P, int threads, int& tile) {
-    const int nbb = boundary_blocks(P.nb, threads), nfb = WALL ? 0 : force_blocks(P.ngroups, threads);
+    const int nbb = boundary_blocks(P.nb), nfb = WALL ? 0 : force_blocks(P.ngroups, threads);
     tile = (int)blockIdx.x - nbb - nfb;
     if (tile >= 0) {
         if (P.flip) tile = P.ntiles - 1 - tile;
@@ -418,7 +437,7 @@ __device__ __forceinline__ bool edge_block(const InstDev& P, int threads, int& t
 
 template <int WALL>
 inline dim3 edge_grid(const InstDev& P, int threads) {
-    return dim3(P.ntiles + boundary_blocks(P.nb, threads) + (WALL ? 0 : force_blocks(P.ngroups, threads)));
+    return dim3(P.ntiles + boundary_blocks(P.nb) + (WALL ? 0 : force_blocks(P.ngroups, threads)));
 }
 
 // Node (x, y) inside the grid, of class cls (already loaded), in a bulk block.  With 4- and 8-byte

@@ -86,7 +86,7 @@ __device__ __forceinline__ void pair_load(const InstDev& P, int x0, int y, PairW
 // grid's rows, so that a block's row is its block index and needs no division.
 constexpr int kPairGridRows = 32768;
 inline int pair_edge_rows(const InstDev& P, int ntx, int threads) {
-    const int n = boundary_blocks(P.nb, threads) + force_blocks(P.ngroups, threads);
+    const int n = boundary_blocks(P.nb) + force_blocks(P.ngroups, threads);
     return (n + ntx - 1) / ntx;
 }
 
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(BT, MINB) step_kernel_pair16(const __grid_cons
     using H = Half16<ST>;
     const int r = blockIdx.z * kPairGridRows + blockIdx.y;
     if (r < edge_rows) {
-        const int e = r * gridDim.x + blockIdx.x, nbb = boundary_blocks(P.nb, BT);
+        const int e = r * gridDim.x + blockIdx.x, nbb = boundary_blocks(P.nb);
         if (e < nbb) boundary_block<L, ST, COLL, 0>(P, e);
         else force_block<L, ST>(P, e - nbb);
         return;
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(BT, MINB) step_kernel_pair16s(const __grid_con
     __shared__ __align__(8) uint64_t bar;
     const int r = blockIdx.z * kPairGridRows + blockIdx.y;
     if (r < edge_rows) {
-        const int e = r * gridDim.x + blockIdx.x, nbb = boundary_blocks(P.nb, BT);
+        const int e = r * gridDim.x + blockIdx.x, nbb = boundary_blocks(P.nb);
         if (e < nbb) boundary_block<L, ST, COLL, 0>(P, e);
         else force_block<L, ST>(P, e - nbb);
         return;

@@ -82,3 +82,21 @@ def test_force_against_oracle(name):
                                                  seed=12)
     assert_state_close(Q, g_gpu, g_or, lab, L.LBM_STORE_F64, 6, g0)
     assert_force_close(F_gpu, F_or, Q, lab, L.LBM_STORE_F64, 6)
+
+
+@pytest.mark.parametrize("wall", [L.LBM_SCHEME_BOUNCEBACK, L.LBM_SCHEME_DIFFUSE], ids=["bounce", "diffuse"])
+@pytest.mark.parametrize("steps", [7, 8, 9, 64, 65, 131])
+def test_long_calls_give_the_forces_of_single_steps(steps, wall):
+    """Calls of several steps sum their forces at once, 64 steps at a time; one-step calls in each step."""
+    geom = L.make_geometry(kind=L.LBM_GEOM_BEAM, lx=13, ly=11, drive=L.LBM_DRIVE_WALL, u0=2e-3, eq_order=4,
+                           wall_scheme=wall)
+    histories = []
+    for chunk in (steps, 1):
+        h = L.lbm_create(37, 61, 47, 0.8, 0.05, geom)
+        try:
+            for _ in range(steps // chunk):
+                L.lbm_step(h, chunk)
+            histories.append(L.lbm_force_history(h))
+        finally:
+            L.lbm_destroy(h)
+    assert histories[0].shape == (steps, 2) and (histories[0] == histories[1]).all()
