@@ -1083,7 +1083,13 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     d.s_f = (float)d.s;
     d.inv_s_f = (float)d.inv_s;
     d.omega_c_f = (float)d.omega_c;
-    d.reg_a_f = (float)d.reg_a;
+    const bool q9 = lattice == LBM_D2Q9;
+    const double diag = (1.0 - 1.0 / tau) / (q9 ? reg_diag<D2Q9, float>() : reg_diag<D2Q37, float>());
+    const double cross = (1.0 - 1.0 / tau) / (q9 ? reg_cross<D2Q9, float>() : reg_cross<D2Q37, float>());
+    d.reg_f[0] = (float)diag;
+    d.reg_f[1] = (float)(diag - (double)d.reg_f[0]);
+    d.reg_f[2] = (float)cross;
+    d.reg_f[3] = (float)(cross - (double)d.reg_f[2]);
     d.src_k_f = (float)d.src_k;
     s->stream_off = es == 2 && g.drive == LBM_DRIVE_BODYFORCE;
     d.stream_off = s->stream_off ? 1 : 0;

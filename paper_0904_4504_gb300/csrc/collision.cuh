@@ -99,6 +99,66 @@ __device__ __forceinline__ V vmulk(double k, V b) {
     return vmuls<V>((typename Lane<V>::T)k, b);
 }
 
+// Sums over the weights as FP32 holds them (w_i, w_i c_i, .. rounded): what a collision and the next
+// step's moments multiply mass, momentum and the kept part of the stress by, were it not corrected --
+// 1 + 8e-9 and 1 + 1.5e-8 a step for mass and momentum in D2Q37, which adds up over a run.  The rest weight,
+// 1/theta and the regularization factors (InstDev::reg_f) make up for it, in two parts where one float
+// cannot hold them.
+template <class L, class T>
+__host__ __device__ constexpr double rest_weight() {  // 1 - sum of the other weights
+    double s = 1.0;
+    for (int k = 0; k < L::NP; ++k) s -= 2.0 * (double)(T)L::wp(k);
+    return s;
+}
+template <class L, class T>
+__host__ __device__ constexpr double inv_theta() {    // 1 / sum of w_i c_ix c_ix
+    double s = 0.0;
+    for (int k = 0; k < L::NP; ++k) s += 2.0 * (double)(T)(L::wp(k) * L::px(k)) * L::px(k);
+    return 1.0 / s;
+}
+// theta as the second moments see it: what p_xx holds of a constant, sum of w_i c_ix c_ix.
+template <class L, class T>
+__host__ __device__ constexpr double pressure() {
+    double s = 0.0;
+    for (int k = 0; k < L::NP; ++k) s += 2.0 * (double)(T)(L::wp(k) * L::px(k) * L::px(k));
+    return s;
+}
+// What the next step's P_xx and P_xy hold of r_xx and r_xy (exactly 2 theta^2 and theta^2).
+template <class L, class T>
+__host__ __device__ constexpr double reg_diag() {
+    double m = 0.0;
+    for (int k = 0; k < L::NP; ++k) {
+        const int x2 = L::px(k) * L::px(k);
+        m += 2.0 * (double)(T)(L::wp(k) * x2) * x2;
+    }
+    return m - pressure<L, T>() * pressure<L, T>();
+}
+template <class L, class T>
+__host__ __device__ constexpr double reg_cross() {
+    double m = 0.0;
+    for (int k = 0; k < L::NP; ++k) {
+        const int xy = L::px(k) * L::py(k);
+        m += 2.0 * (double)(T)(L::wp(k) * xy) * xy;
+    }
+    return m;
+}
+
+// k v for a constant k given to more digits than T holds.
+template <class V>
+__device__ __forceinline__ V vmulx(double k, V v) {
+    using T = typename Lane<V>::T;
+    if (sizeof(T) == 8) return vmulk(k, v);
+    const T hi = (T)k;
+    return vfmas<V>((T)(k - (double)hi), v, vmuls<V>(hi, v));
+}
+template <class V>
+__device__ __forceinline__ V vfmax(double k, V v, V c) {
+    using T = typename Lane<V>::T;
+    if (sizeof(T) == 8) return vfmak(k, v, c);
+    const T hi = (T)k;
+    return vfmas<V>((T)(k - (double)hi), v, vfmas<V>(hi, v, c));
+}
+
 // Eq. 16 on deviations: drho = sum g_i, j = sum g_i c_i, Pi' = sum g_i c_i c_i, in the units of
 // the populations (w_i divided out).  The pair tables list pairs in groups of two of one shell:
 // (p_x, p_y) and (p_x, -p_y), whose sums S, D and differences Jp, Jm of the pairs' sums and
@@ -113,7 +173,9 @@ struct Moments {
 template <class L, class V, class H>
 __device__ __forceinline__ Moments<V> moments(H&& h) {
     Moments<V> M;
-    M.m0 = vmulk(L::w0(), h(0));
+    using T = typename Lane<V>::T;
+    constexpr double w0 = sizeof(T) == 8 ? L::w0() : rest_weight<L, T>();
+    M.m0 = vmulx<V>(w0, h(0));
 #pragma unroll
     for (int k = 0; k < L::NP; k += 2) {
         const int m = L::px(k), n = L::py(k);
@@ -179,7 +241,8 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         jx = vfmak(0.5, F, jx);
     }
     const V ux = vmul(jx, irho), uy = vmul(M.jy, irho);
-    const V X = vmulk(1.0 / TH, ux), Y = vmulk(1.0 / TH, uy);
+    constexpr double ITH = sizeof(T) == 8 ? 1.0 / TH : inv_theta<L, T>();
+    const V X = vmulx<V>(ITH, ux), Y = vmulx<V>(ITH, uy);
     const V b = vfma(uy, Y, vmul(ux, X));
 
     // Eq. 15 (+ 4th order): g_i^eq / w_i = e0 + a^2 (e1 + a^2 e2) + a (o0 + o1 a^2), a = c_i.u/theta
@@ -201,12 +264,21 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
     V rxx, rxy, ryy, hf;
     if (COLL == COLL_REG) {
         // Eq. 19: Pi^ne = Pi - Pi^eq with Pi^eq = rho theta I + rho u u (exact on these lattices)
+        constexpr double THP = sizeof(T) == 8 ? TH : pressure<L, T>();
         const V rux = vmul(rho, ux), ruy = vmul(rho, uy);
-        const T A = kconst<T>(P.reg_a, P.reg_a_f);
-        rxx = vmuls<V>(A, vfma(vneg(rux), ux, vfmak(-TH, M.m0, M.pxx)));
-        rxy = vmuls<V>((T)2 * A, vfma(vneg(rux), uy, M.pxy));
-        ryy = vmuls<V>(A, vfma(vneg(ruy), uy, vfmak(-TH, M.m0, M.pyy)));
-        e0 = vfmak(-TH, vadd(rxx, ryy), e0);
+        const V Pxx = vfma(vneg(rux), ux, vfmax<V>(-THP, M.m0, M.pxx));
+        const V Pxy = vfma(vneg(rux), uy, M.pxy);
+        const V Pyy = vfma(vneg(ruy), uy, vfmax<V>(-THP, M.m0, M.pyy));
+        if constexpr (sizeof(T) == 8) {
+            rxx = vmuls<V>(P.reg_a, Pxx);
+            rxy = vmuls<V>(2.0 * P.reg_a, Pxy);
+            ryy = vmuls<V>(P.reg_a, Pyy);
+        } else {
+            rxx = vfmas<V>(P.reg_f[1], Pxx, vmuls<V>(P.reg_f[0], Pxx));
+            rxy = vfmas<V>(P.reg_f[3], Pxy, vmuls<V>(P.reg_f[2], Pxy));
+            ryy = vfmas<V>(P.reg_f[1], Pyy, vmuls<V>(P.reg_f[0], Pyy));
+        }
+        e0 = vfmax<V>(-THP, vadd(rxx, ryy), e0);
         if (P.body_force) e0 = vfma(vneg(kf), ux, e0);
         hf = vmulk(0.5 / TH, F);   // first-order part: kept J^ne = -F/2 plus the source
     }

@@ -69,7 +69,9 @@ struct InstDev {
     double mw_k;                 // 2 rho0 / (theta s): moving-wall term per unit c_i.U_w
     // FP32 copies of the constants above (and of dv), so that FP32 arithmetic converts nothing per
     // node: double -> float conversions run on the FP64 pipe, which is slow on this GPU
-    float dv_f, rho0_f, s_f, inv_s_f, omega_c_f, reg_a_f, src_k_f, dv2_f;
+    float dv_f, rho0_f, s_f, inv_s_f, omega_c_f, reg_pad, src_k_f, dv2_f;
+    // FP32 regularization factors of P_xx, P_yy and of P_xy, each as the sum of two floats (collision.cuh)
+    float reg_f[4];
     // 16-bit body-frame runs store h_i - H_i(n), with H_i(n) the (scaled) equilibrium deviation of
     // the uniform stream U(n) = sum_{k<n} g(k + 1/2) that the body force sets up; far from the body
     // the stored values are then small and so are their rounding errors.  The stream is along x, so
