@@ -383,7 +383,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         // four-nodes-per-thread kernel (30); else the plain kernel
         const int want = b->variant >= 0 ? b->variant
                          : half ? (b->Q != 37 ? 30 : b->collision == LBM_COLL_REGULARIZED ? 32 : 27)
-                         : (b->Q == 37 && b->storage == LBM_STORE_F32) ? 2 : 0;
+                         : b->storage == LBM_STORE_F32 ? (b->Q == 37 ? 2 : 30) : 0;
         if (want == 0 || lbm_set_variant(sim, want) != LBM_OK) rc = lbm_set_tile(sim, b->bx, b->by);
     }
     if (rc) return undo(rc);

@@ -67,7 +67,7 @@ static TmaStepLaunchFn find_tma_launcher(int Q, int storage, int coll, int varia
 }
 
 // Tile of a staged variant (see lbm_set_variant); false for other variants.
-static bool variant_tile(int variant, int* bx, int* by) {
+static bool variant_tile(int variant, int storage, int* bx, int* by) {
     switch (variant) {
         case 1:
         case 2:
@@ -85,7 +85,7 @@ static bool variant_tile(int variant, int* bx, int* by) {
         case 27: *bx = 64; *by = 3; return true;
         case 28: *bx = 128; *by = 3; return true;
         case 20: *bx = 64; *by = 4; return true;
-        case 30: *bx = 128; *by = 4; return true;
+        case 30: *bx = storage == ST_F32 ? 64 : 128; *by = 4; return true;
         case 31: *bx = 64; *by = 1; return true;
         case 32: *bx = 128; *by = 2; return true;
         case 21: *bx = 64; *by = 2; return true;
@@ -694,7 +694,7 @@ int use_variant(lbm_sim* s, int variant) {
                                                     : nullptr)
                                        : find_occ_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
         if (!f) return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
-        variant_tile(variant, &s->bx, &s->by);
+        variant_tile(variant, s->geom.storage, &s->bx, &s->by);
         s->variant = variant;
         s->tma_launch = nullptr;
         s->launch = f;
@@ -702,7 +702,7 @@ int use_variant(lbm_sim* s, int variant) {
     }
     int bx, by, bw, pad, rc;
     TmaStepLaunchFn fn = find_tma_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
-    if (!fn || !variant_tile(variant, &bx, &by))
+    if (!fn || !variant_tile(variant, s->geom.storage, &bx, &by))
         return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
     tma_box(s->Q, s->geom.storage, bx, &bw, &pad);
     for (int k = 0; k < 2; ++k) {
@@ -1096,11 +1096,13 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     // default kernel: the fastest measured single-instance form -- for D2Q37 the plain kernel with
     // an occupancy floor on the default 32 x 4 tile (variant 1 for FP32, 2 for 16-bit storage), for
     // the regularized collision of 16-bit storage two nodes per thread (31; 32, staged, where the two
-    // buffers hold over 200 MB; step_q37v.cuh has the measurements), for 16-bit D2Q9 the
-    // four-nodes-per-thread kernel on 128 x 4 tiles (variant 30)
+    // buffers hold over 200 MB; step_q37v.cuh has the measurements), for FP32 and 16-bit D2Q9 several
+    // nodes per thread (30) but on small grids, where fewer nodes per thread mean more warps (FP32: 2048^2
+    // 44.7 us against 55.4, 1024^2 9.6 / 12.0, 512^2 3.9 / 3.7, 128^2 2.2 / 1.8; FP16: 512^2 4.1 / 4.2, 128^2
+    // 3.1 / 1.8)
     if (!s->aa && g.wall_scheme == LBM_SCHEME_BOUNCEBACK) {
         int v = 0;
-        if (lattice == LBM_D2Q9) v = es == 2 ? 30 : 0;
+        if (lattice == LBM_D2Q9) v = es <= 4 && (size_t)nx * ny > ((size_t)1 << (es == 4 ? 18 : 17)) ? 30 : 0;
         else if (es == 4) v = 1;
         else if (es == 2)
             v = g.collision != LBM_COLL_REGULARIZED || nx < 48 ? 2 : 2 * plane * H.Q * es > (size_t)200000000 ? 32 : 31;
@@ -1372,15 +1374,16 @@ int lbm_tune(lbm_sim* s, int steps, lbm_tune_entry* out, int cap, int* n_out) {
     if (steps < 1 || !n_out || (cap > 0 && !out)) return set_error(LBM_EINVAL, "need steps >= 1 and an output");
     // candidates: plain kernel tiles, then every staged variant built for this storage type
     const int tiles[][2] = {{32, 4}, {32, 8}, {64, 2}, {64, 4}, {128, 1}, {32, 2}};
-    const int variants[] = {1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27, 31, 32};
+    const int variants[] = {1, 2, 3, 4, 10, 11, 12, 13, 18, 20, 23, 24, 25, 26, 27, 30, 31, 32};
     std::vector<lbm_tune_entry> cand;
     for (auto& t : tiles) cand.push_back(lbm_tune_entry{0, t[0], t[1], 0.0});
     for (int v : variants)
         if (!s->aa && s->geom.wall_scheme == LBM_SCHEME_BOUNCEBACK &&
             (find_tma_launcher(s->Q, s->geom.storage, s->geom.collision, v) ||
-             find_occ_launcher(s->Q, s->geom.storage, s->geom.collision, v))) {
+             find_occ_launcher(s->Q, s->geom.storage, s->geom.collision, v) ||
+             (s->Q == 9 && find_q9v_launcher(s->geom.storage, s->geom.collision, v)))) {
             int bx = 0, by = 0;
-            variant_tile(v, &bx, &by);
+            variant_tile(v, s->geom.storage, &bx, &by);
             cand.push_back(lbm_tune_entry{v, bx, by, 0.0});
         }
     // a clone with the same geometry (as a label mask), parameters and storage

@@ -55,20 +55,18 @@ PbKernel find_pbatch_q9(int storage, int coll, int variant) {
     }
 }
 
-// The four-nodes-per-thread kernel of 16-bit storage (variant 30, 128 x 4 tiles; step_q9v.cuh).
-// The kernel is latency bound, so the occupancy floor is set above what the registers alone
-// give: the regularized collision at 8 blocks per SM (64 registers, 8 B spilled; measured 0.62 /
-// 0.73 of the copy peak at 2048^2 / 4096^2 against 0.56 / 0.63 at its unspilled 6 blocks, 0.61 /
-// 0.72 at 9 and 0.53 / 0.62 at 10), plain BGK at 7 (0.57 against 0.55 at 6 and 8).  (Two rows per
-// thread with both rows' loads issued first, 128 x 8 tiles, measured 0.54-0.64 against 0.56-0.63
-// on the same box: not built.)
+// The kernel of several nodes per thread (variant 30; step_q9v.cuh): 128 x 4 tiles with 16-bit storage,
+// 64 x 4 with FP32.  At least 8 blocks of 128 threads per SM, 7 for plain BGK with 16-bit storage (9 and 10
+// measured 0 to 12 % slower with 16-bit storage, 10 % slower on a 512^2 FP32 grid; 5 and 6 no better).
 void* find_q9v_launcher(int storage, int coll, int variant) {
     if (variant != 30) return nullptr;
     switch (storage * 2 + coll) {
-        case ST_BF16 * 2 + COLL_BGK: return (void*)&launch_step_q9v<__nv_bfloat16, COLL_BGK, 1, 7>;
-        case ST_BF16 * 2 + COLL_REG: return (void*)&launch_step_q9v<__nv_bfloat16, COLL_REG, 1, 8>;
-        case ST_F16 * 2 + COLL_BGK: return (void*)&launch_step_q9v<__half, COLL_BGK, 1, 7>;
-        case ST_F16 * 2 + COLL_REG: return (void*)&launch_step_q9v<__half, COLL_REG, 1, 8>;
+        case ST_F32 * 2 + COLL_BGK: return (void*)&launch_step_q9v<float, COLL_BGK, 8>;
+        case ST_F32 * 2 + COLL_REG: return (void*)&launch_step_q9v<float, COLL_REG, 8>;
+        case ST_BF16 * 2 + COLL_BGK: return (void*)&launch_step_q9v<__nv_bfloat16, COLL_BGK, 7>;
+        case ST_BF16 * 2 + COLL_REG: return (void*)&launch_step_q9v<__nv_bfloat16, COLL_REG, 8>;
+        case ST_F16 * 2 + COLL_BGK: return (void*)&launch_step_q9v<__half, COLL_BGK, 7>;
+        case ST_F16 * 2 + COLL_REG: return (void*)&launch_step_q9v<__half, COLL_REG, 8>;
         default: return nullptr;
     }
 }
