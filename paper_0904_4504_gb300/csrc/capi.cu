@@ -1077,6 +1077,7 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     d.inv_s = 1.0 / d.s;
     d.omega_c = 1.0 / tau;
     d.reg_a = (1.0 - 1.0 / tau) / (2.0 * H.theta * H.theta);
+    d.reg_a2 = 2.0 * d.reg_a;
     d.src_k = (1.0 - 0.5 / tau) / H.theta;
     d.mw_k = 2.0 * g.rho0 / (H.theta * d.s);
     d.rho0_f = (float)d.rho0;

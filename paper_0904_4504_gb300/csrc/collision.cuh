@@ -10,8 +10,9 @@
 // whose coefficients depend on the node only.  They are expanded in monomials, so that the axis parts
 // are evaluated once per |c_x| and |c_y| and shared by the shells, and the four velocities
 // +-(m, n), +-(m, -n) of a shell cost 14 operations together.  (Polynomials in a = c.u / theta,
-// evaluated velocity by velocity, take 410 FP64 operations a node, this form about 310.  FP64 storage is
-// bound by them: 725 -> 593 us a step of the 1024^2 D2Q37 box, 51 -> 43 us of a 512^2 D2Q9 one.)
+// evaluated velocity by velocity, take 410 FP64 operations a node, this form 291, and 284 without a body
+// force.  FP64 storage is bound by them: 725 -> 579 us a step of the 1024^2 D2Q37 box, 51 -> 38 us of a 512^2
+// D2Q9 plate, plain BGK 53 -> 40 with 74 operations.)
 #pragma once
 
 #include "step_types.cuh"
@@ -116,21 +117,24 @@ __host__ __device__ constexpr double inv_theta() {    // 1 / sum of w_i c_ix c_i
     for (int k = 0; k < L::NP; ++k) s += 2.0 * (double)(T)(L::wp(k) * L::px(k)) * L::px(k);
     return 1.0 / s;
 }
+// Weight of pair k in p_xx as the moments apply it (diagonal shells in two parts).
+template <class L, class T>
+__host__ __device__ constexpr double weight_xx(int k) {
+    const int x2 = L::px(k) * L::px(k);
+    return x2 && L::py(k) ? (double)(T)L::wp(k) + (double)(T)(L::wp(k) * (x2 - 1)) : (double)(T)(L::wp(k) * x2);
+}
 // theta as the second moments see it: what p_xx holds of a constant, sum of w_i c_ix c_ix.
 template <class L, class T>
 __host__ __device__ constexpr double pressure() {
     double s = 0.0;
-    for (int k = 0; k < L::NP; ++k) s += 2.0 * (double)(T)(L::wp(k) * L::px(k) * L::px(k));
+    for (int k = 0; k < L::NP; ++k) s += 2.0 * weight_xx<L, T>(k);
     return s;
 }
 // What the next step's P_xx and P_xy hold of r_xx and r_xy (exactly 2 theta^2 and theta^2).
 template <class L, class T>
 __host__ __device__ constexpr double reg_diag() {
     double m = 0.0;
-    for (int k = 0; k < L::NP; ++k) {
-        const int x2 = L::px(k) * L::px(k);
-        m += 2.0 * (double)(T)(L::wp(k) * x2) * x2;
-    }
+    for (int k = 0; k < L::NP; ++k) m += 2.0 * weight_xx<L, T>(k) * (L::px(k) * L::px(k));
     return m - pressure<L, T>() * pressure<L, T>();
 }
 template <class L, class T>
@@ -162,8 +166,8 @@ __device__ __forceinline__ V vfmax(double k, V v, V c) {
 // Eq. 16 on deviations: drho = sum g_i, j = sum g_i c_i, Pi' = sum g_i c_i c_i, in the units of
 // the populations (w_i divided out).  The pair tables list pairs in groups of two of one shell:
 // (p_x, p_y) and (p_x, -p_y), whose sums S, D and differences Jp, Jm of the pairs' sums and
-// differences give the six moments with one multiply-add each, or (m, 0) and (0, m), taken pair by
-// pair.
+// differences go into the moments, or (m, 0) and (0, m), taken pair by pair.  A diagonal shell's w S goes
+// once into a sum that m0, pxx and pyy share.
 template <class V>
 struct Moments {
     V m0, jx, jy, pxx, pxy, pyy;
@@ -172,35 +176,59 @@ struct Moments {
 // (h(i): the population that arrived along direction i.)
 template <class L, class V, class H>
 __device__ __forceinline__ Moments<V> moments(H&& h) {
-    Moments<V> M;
     using T = typename Lane<V>::T;
-    constexpr double w0 = sizeof(T) == 8 ? L::w0() : rest_weight<L, T>();
-    M.m0 = vmulx<V>(w0, h(0));
+    static_assert(L::NP % 2 == 0 && L::py(0) == 0 && L::py(2) != 0 && L::py(2) == -L::py(3),
+                  "the pair tables start with the axis pairs (1, 0), (0, 1) and the diagonal shell");
+    Moments<V> M;
+    // what the diagonal shells give to m0, pxx and pyy alike, and what they give to pxx and pyy beyond it
+    V all, xx, yy;
+    bool first_xx = true;
 #pragma unroll
-    for (int k = 0; k < L::NP; k += 2) {
+    for (int k = 2; k < L::NP; k += 2) {
         const int m = L::px(k), n = L::py(k);
+        if (n == 0) continue;
         const double w = L::wp(k);
         const V a1 = h(1 + 2 * k), b1 = h(2 + 2 * k), a2 = h(3 + 2 * k), b2 = h(4 + 2 * k);
         const V sp1 = vadd(a1, b1), dm1 = vsub(a1, b1), sp2 = vadd(a2, b2), dm2 = vsub(a2, b2);
-        if (n == 0) {
-            // (m, 0) and (0, m); the first group starts the sums
-            M.m0 = vfmak(w, sp2, vfmak(w, sp1, M.m0));
-            M.jx = k == 0 ? vmulk(w * m, dm1) : vfmak(w * m, dm1, M.jx);
-            M.jy = k == 0 ? vmulk(w * m, dm2) : vfmak(w * m, dm2, M.jy);
-            M.pxx = k == 0 ? vmulk(w * m * m, sp1) : vfmak(w * m * m, sp1, M.pxx);
-            M.pyy = k == 0 ? vmulk(w * m * m, sp2) : vfmak(w * m * m, sp2, M.pyy);
+        const V S = vadd(sp1, sp2), D = vsub(sp1, sp2), Jp = vadd(dm1, dm2), Jm = vsub(dm1, dm2);
+        if (k == 2) {
+            all = vmulk(w, S);
+            M.jx = vmulk(w * m, Jp);
+            M.jy = vmulk(w * n, Jm);
+            M.pxy = vmulk(w * m * n, D);
         } else {
-            const V S = vadd(sp1, sp2), D = vsub(sp1, sp2), Jp = vadd(dm1, dm2), Jm = vsub(dm1, dm2);
-            M.m0 = vfmak(w, S, M.m0);
+            all = vfmak(w, S, all);
             M.jx = vfmak(w * m, Jp, M.jx);
             M.jy = vfmak(w * n, Jm, M.jy);
-            M.pxx = vfmak(w * m * m, S, M.pxx);
-            M.pxy = k == 2 ? vmulk(w * m * n, D) : vfmak(w * m * n, D, M.pxy);
-            M.pyy = vfmak(w * n * n, S, M.pyy);
+            M.pxy = vfmak(w * m * n, D, M.pxy);
+        }
+        if (m > 1 && n > 1) {  // the (2, 2) shell comes first of those with more than `all`
+            xx = yy = vmulk(w * (m * m - 1), S);
+            first_xx = false;
+        } else if (m > 1) {
+            xx = vfmak(w * (m * m - 1), S, xx);
+        } else if (n > 1) {
+            yy = vfmak(w * (n * n - 1), S, yy);
         }
     }
-    static_assert(L::NP % 2 == 0 && L::py(0) == 0 && L::py(2) != 0 && L::py(2) == -L::py(3),
-                  "the pair tables start with the axis pairs (1, 0), (0, 1) and the diagonal shell");
+    M.m0 = all;
+    M.pxx = first_xx ? all : vadd(all, xx);
+    M.pyy = first_xx ? all : vadd(all, yy);
+#pragma unroll
+    for (int k = 0; k < L::NP; k += 2) {
+        const int m = L::px(k);
+        if (L::py(k) != 0) continue;
+        const double w = L::wp(k);
+        const V a1 = h(1 + 2 * k), b1 = h(2 + 2 * k), a2 = h(3 + 2 * k), b2 = h(4 + 2 * k);
+        const V sp1 = vadd(a1, b1), dm1 = vsub(a1, b1), sp2 = vadd(a2, b2), dm2 = vsub(a2, b2);
+        M.m0 = vfmak(w, sp2, vfmak(w, sp1, M.m0));
+        M.jx = vfmak(w * m, dm1, M.jx);
+        M.jy = vfmak(w * m, dm2, M.jy);
+        M.pxx = vfmak(w * m * m, sp1, M.pxx);
+        M.pyy = vfmak(w * m * m, sp2, M.pyy);
+    }
+    constexpr double w0 = sizeof(T) == 8 ? L::w0() : rest_weight<L, T>();
+    M.m0 = vfmax<V>(w0, h(0), M.m0);
     return M;
 }
 
@@ -217,11 +245,14 @@ struct Coef {
 // Coefficients from the moments (storage units, relative to the stream offset with 16-bit storage and
 // the offset on): Eqs. 15 and 19 and the Guo-type source.  With 16-bit storage the moments are scaled
 // by s on the way in and the coefficients by 1/s on the way out.
-template <class L, class ST, int COLL, class V>
+// BODY: whether there is a body force (0, 1), or -1 to ask the launch parameters.  (FP64 asks once per node, in
+// collide_emit: an FP64 instruction predicated off takes as long as one that runs.)
+template <class L, class ST, int COLL, class V, int BODY = -1>
 __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, float dv_f, Moments<V> M) {
     using T = typename Lane<V>::T;
     constexpr bool SCALED = sizeof(ST) == 2;
     constexpr bool H4 = L::R == 3;  // the lattice carries the fourth-order equilibrium
+    const bool body = BODY < 0 ? P.body_force != 0 : BODY == 1;
     Coef<V> C;
     if (SCALED) {
         if (COLL == COLL_REG && P.stream_off) {
@@ -236,7 +267,7 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
     const V rho = vadds(M.m0, kconst<T>(P.rho0, P.rho0_f));
     const V irho = vrcp(rho);
     V jx = M.jx, F = vset<V>((T)0);
-    if (P.body_force) {
+    if (body) {
         F = vmuls<V>(kconst<T>(dv, dv_f), rho);
         jx = vfmak(0.5, F, jx);
     }
@@ -260,7 +291,7 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         }
     }
     // Guo-type source: even part kf (a c_x - u_x), odd part c_x times kf (plain BGK) or F/(2 theta)
-    const V kf = P.body_force ? vmuls<V>(kconst<T>(P.src_k, P.src_k_f), F) : vset<V>((T)0);
+    const V kf = body ? vmuls<V>(kconst<T>(P.src_k, P.src_k_f), F) : vset<V>((T)0);
     V rxx, rxy, ryy, hf;
     if (COLL == COLL_REG) {
         // Eq. 19: Pi^ne = Pi - Pi^eq with Pi^eq = rho theta I + rho u u (exact on these lattices)
@@ -271,7 +302,7 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         const V Pyy = vfma(vneg(ruy), uy, vfmax<V>(-THP, M.m0, M.pyy));
         if constexpr (sizeof(T) == 8) {
             rxx = vmuls<V>(P.reg_a, Pxx);
-            rxy = vmuls<V>(2.0 * P.reg_a, Pxy);
+            rxy = vmuls<V>(P.reg_a2, Pxy);
             ryy = vmuls<V>(P.reg_a, Pyy);
         } else {
             rxx = vfmas<V>(P.reg_f[1], Pxx, vmuls<V>(P.reg_f[0], Pxx));
@@ -279,7 +310,7 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
             ryy = vfmas<V>(P.reg_f[1], Pyy, vmuls<V>(P.reg_f[0], Pyy));
         }
         e0 = vfmax<V>(-THP, vadd(rxx, ryy), e0);
-        if (P.body_force) e0 = vfma(vneg(kf), ux, e0);
+        if (body) e0 = vfma(vneg(kf), ux, e0);
         hf = vmulk(0.5 / TH, F);   // first-order part: kept J^ne = -F/2 plus the source
     }
     if (SCALED) {
@@ -302,8 +333,8 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         C.q20 = vfma(eX, X, rxx);
         C.q11 = vfma(eX2, Y, rxy);
         C.q02 = vfma(eY, Y, ryy);
-        C.l10 = vfma(o0, X, hf);
-        if (P.body_force) {
+        C.l10 = BODY == 0 ? vmul(o0, X) : vfma(o0, X, hf);
+        if (body) {
             C.q20 = vfma(C.kf, X, C.q20);
             C.q11 = vfma(C.kf, Y, C.q11);
         }
@@ -312,9 +343,11 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         C.q11 = vmul(eX2, Y);
         C.q02 = vmul(eY, Y);
         C.l10 = vmul(o0, X);
-        C.kfu = vmul(vneg(C.kf), ux);
-        C.kfx = vmul(C.kf, X);
-        C.kfy = vmul(C.kf, Y);
+        if (BODY != 0) {
+            C.kfu = vmul(vneg(C.kf), ux);
+            C.kfx = vmul(C.kf, X);
+            C.kfy = vmul(C.kf, Y);
+        }
     }
     C.l01 = vmul(o0, Y);
     if (H4) {
@@ -338,14 +371,14 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
 // to the stream offset of the stored state when it is on: He and Ho of |c_x| leave the even and odd
 // parts).  Plain BGK reads the pulled populations h (absolute ones), the regularized collision does
 // not.
-template <class L, class ST, int COLL, class V, class H, class Emit>
-__device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C, H&& h, Emit&& emit) {
+template <class L, class ST, int COLL, class V, bool SOURCE, class H, class Emit>
+__device__ __forceinline__ void emit_outputs_s(const InstDev& P, const Coef<V>& C, H&& h, Emit&& emit) {
     using T = typename Lane<V>::T;
     constexpr int R = L::R;
     constexpr bool H4 = R == 3;
     constexpr bool SCALED = sizeof(ST) == 2, REG = COLL == COLL_REG;
     const T om = kconst<T>(P.omega_c, P.omega_c_f);
-    const bool source = !REG && (P.body_force || (SCALED && P.stream_off));  // launch-uniform
+    constexpr bool source = !REG && SOURCE;
     V EA[R + 1], EB[R + 1], OX[R + 1], OY[R + 1], U[R + 1];
     V Sa[R + 1], So[R + 1];  // plain BGK: source parts per |c_x|, less the stored state's stream offset
 #pragma unroll
@@ -424,6 +457,19 @@ __device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C,
             out(i + 3, vsub(Em, Om), m, sm, So[m], -1);
         }
     }
+}
+
+// The same; plain BGK adds its source where the launch has one (a branch, not predicated operations).
+template <class L, class ST, int COLL, class V, int BODY = -1, class H, class Emit>
+__device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C, H&& h, Emit&& emit) {
+    if constexpr (COLL == COLL_REG || BODY == 0)
+        emit_outputs_s<L, ST, COLL, V, false>(P, C, h, emit);
+    else if constexpr (BODY == 1)
+        emit_outputs_s<L, ST, COLL, V, true>(P, C, h, emit);
+    else if (P.body_force || (sizeof(ST) == 2 && P.stream_off))
+        emit_outputs_s<L, ST, COLL, V, true>(P, C, h, emit);
+    else
+        emit_outputs_s<L, ST, COLL, V, false>(P, C, h, emit);
 }
 
 }  // namespace lbm

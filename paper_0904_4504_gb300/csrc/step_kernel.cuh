@@ -202,8 +202,15 @@ __device__ __forceinline__ void add_offset(const InstDev& P, unsigned long long 
 template <class L, class ST, int COLL, class V, class Emit>
 __device__ __forceinline__ void collide_emit(const InstDev& P, double dv, float dv_f, const V (&h)[L::Q], Emit&& emit) {
     const auto at = [&](int i) { return h[i]; };
-    const Coef<V> C = coefficients<L, ST, COLL, V>(P, dv, dv_f, moments<L, V>(at));
-    emit_outputs<L, ST, COLL, V>(P, C, at, emit);
+    const Moments<V> M = moments<L, V>(at);
+    if constexpr (sizeof(ST) == 8) {
+        if (P.body_force)
+            emit_outputs<L, ST, COLL, V, 1>(P, coefficients<L, ST, COLL, V, 1>(P, dv, dv_f, M), at, emit);
+        else
+            emit_outputs<L, ST, COLL, V, 0>(P, coefficients<L, ST, COLL, V, 0>(P, dv, dv_f, M), at, emit);
+    } else {
+        emit_outputs<L, ST, COLL, V>(P, coefficients<L, ST, COLL, V>(P, dv, dv_f, M), at, emit);
+    }
 }
 
 // The same, stored at the node's place (element offset y pitch + x).

@@ -64,7 +64,7 @@ struct InstDev {
     double rho0;
     double s, inv_s;             // storage scale
     double omega_c;              // 1/tau
-    double reg_a;                // (1 - 1/tau) / (2 theta^2)
+    double reg_a, reg_a2;        // (1 - 1/tau) / (2 theta^2), and twice that
     double src_k;                // (1 - 1/(2 tau)) / theta
     double mw_k;                 // 2 rho0 / (theta s): moving-wall term per unit c_i.U_w
     // FP32 copies of the constants above (and of dv), so that FP32 arithmetic converts nothing per
