@@ -477,13 +477,13 @@ void lbm_server_destroy(lbm_server* server);
  * The work is enqueued on `stream` (a cudaStream_t; 0 is the default stream) and the call returns
  * before it runs.
  *
- * Scratch: the kernel's force partials and its reduction counter live in one static
- * device array of the library (LBM_NOALLOC_MAX_SLOTS * 256 + 256 bytes), held by every GPU that
- * loads the library until the process exits.  A geometry with more than LBM_NOALLOC_MAX_SLOTS
- * tiles holding body links is rejected with LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer).
- * All calls in the process share that array: calls whose work overlaps on the GPU (two streams,
- * or two host threads) race and give wrong forces; serialize them.  The counter is cleared at
- * the start of every call, so a call that never completed does not affect the next one.
+ * Scratch: the kernel's force partials live in one static device array of the library
+ * (LBM_NOALLOC_MAX_SLOTS * 256 + 256 bytes), held by every GPU that loads the library until the process
+ * exits.  A geometry with more than LBM_NOALLOC_MAX_SLOTS tiles holding body links is rejected with
+ * LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer).  All calls in the process share that array: calls
+ * whose work overlaps on the GPU (two streams, or two host threads) race and give wrong forces;
+ * serialize them.  Nothing is carried from one call to the next, so a call that never completed does not
+ * affect the next one.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress) with
  * that device current; make that first call before any stream capture (a lookup that fails is
  * not remembered: the next call tries again).

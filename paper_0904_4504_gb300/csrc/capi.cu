@@ -138,6 +138,11 @@ static void* find_launcher(int Q, int storage, int coll) {
     return nullptr;
 }
 
+StepLaunchFn find_direct_launcher(int Q, int storage, int coll, int variant) {
+    if (variant != 30) return find_occ_launcher(Q, storage, coll, variant);
+    return Q == 9 ? reinterpret_cast<StepLaunchFn>(find_q9v_launcher(storage, coll, variant)) : nullptr;
+}
+
 StepLaunchFn find_occ_launcher(int Q, int storage, int coll, int variant) {
     if (Q != 37 || !(variant >= 1 && variant <= 4 || variant == 31) || !q37_table(storage)) return nullptr;
     return reinterpret_cast<StepLaunchFn>(q37_table(storage)->occ(coll, variant));
@@ -689,10 +694,7 @@ void stream_offset_eo(const float* H7, float* He, float* Ho) {
 // Switch to a kernel variant other than 0 (two-buffer layout, bounce-back walls).
 int use_variant(lbm_sim* s, int variant) {
     if ((variant >= 1 && variant <= 4) || variant == 30 || variant == 31) {
-        StepLaunchFn f = variant == 30 ? (s->Q == 9 ? reinterpret_cast<StepLaunchFn>(find_q9v_launcher(
-                                                          s->geom.storage, s->geom.collision, variant))
-                                                    : nullptr)
-                                       : find_occ_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
+        StepLaunchFn f = find_direct_launcher(s->Q, s->geom.storage, s->geom.collision, variant);
         if (!f) return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
         variant_tile(variant, s->geom.storage, &s->bx, &s->by);
         s->variant = variant;

@@ -6,11 +6,13 @@
 // is already fully reserved, or a loop with a fixed memory budget where an allocation that can fail
 // or stall is not acceptable.  lbm_step itself may allocate (it grows the force history), so these
 // callers step the lattice through this entry point instead: the populations and the force live in
-// buffers the caller owns, and the only other memory the step kernel needs -- its force
-// partials and the ticket of their reduction -- lives in one file-scope device array below,
-// loaded with the library and held by every GPU that uses it until the process exits.
+// buffers the caller owns, and the only other memory the step kernel needs -- its force partials --
+// lives in one file-scope device array below, loaded with the library and held by every GPU that uses it
+// until the process exits.
 //
-// The kernel is the library's step kernel itself; only the scratch pointers differ.
+// The kernel is the simulation's own step kernel, where it reads the populations directly and the
+// caller's buffers are aligned for it, else the plain one; a second launch sums the force (sum_forces), so
+// that there is no counter to clear before the step.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -21,10 +23,10 @@
 
 namespace {
 
-// Scratch: the group partials of the force (16 B each), then the ticket counter and the non-finite
-// flag.  With bounce-back walls a step has at most kMaxForceGroups groups; with diffuse walls one per 32
-// nodes with body links, and a geometry is accepted with up to LBM_NOALLOC_MAX_SLOTS tiles holding such
-// nodes, 512 in a tile at most.  Shared by every call in the process on a given device.
+// Scratch: the group partials of the force (16 B each), then the non-finite flag.  With bounce-back walls a
+// step has at most kMaxForceGroups groups; with diffuse walls one per 32 nodes with body links, and a
+// geometry is accepted with up to LBM_NOALLOC_MAX_SLOTS tiles holding such nodes, 512 in a tile at most.
+// Shared by every call in the process on a given device.
 constexpr size_t kPartialBytes = (size_t)LBM_NOALLOC_MAX_SLOTS * 16 * sizeof(double2);
 constexpr size_t kScratchBytes = kPartialBytes + 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -79,7 +81,14 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     const cudaError_t arc = scratch_address(v.device, &base);
     if (arc != cudaSuccess || !base)
         return set_error(LBM_ECUDA, "cudaGetSymbolAddress of the step scratch: %s", cudaGetErrorString(arc));
-    StepLaunchFn fn = find_step_launcher(v.Q, v.storage, v.collision, v.inst.wall_ds);
+    // the simulation's kernel if it reads the populations directly: 30 with 8-byte loads, 31 with 4-byte
+    // ones (for 32, its staged form, 31)
+    StepLaunchFn fn = nullptr;
+    const size_t misalign = reinterpret_cast<size_t>(g_in) | reinterpret_cast<size_t>(g_out);
+    const int variant = v.variant == 32 ? 31 : v.variant;
+    const bool fits = variant == 30 ? misalign % 8 == 0 : variant == 31 ? misalign % 4 == 0 : true;
+    if (variant != 0 && fits && !v.aa) fn = find_direct_launcher(v.Q, v.storage, v.collision, variant);
+    if (!fn) fn = find_step_launcher(v.Q, v.storage, v.collision, v.inst.wall_ds);
     if (!fn) return set_error(LBM_EINVAL, "no kernel for this simulation");
 
     unsigned char* b = static_cast<unsigned char*>(base);
@@ -87,8 +96,8 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     P.src = g_in;
     P.dst = g_out;
     P.partials = reinterpret_cast<double2*>(b);
-    P.ticket = reinterpret_cast<unsigned int*>(b + kPartialBytes);
-    P.err = reinterpret_cast<int*>(b + kPartialBytes + 128);
+    P.ticket = nullptr;
+    P.err = reinterpret_cast<int*>(b + kPartialBytes);
     P.force_out = reinterpret_cast<double2*>(force_out);
     P.ngroups = v.nlf;
     P.flip = (int)(n & 1);
@@ -96,11 +105,16 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     P.stream_off = 0;  // caller buffers hold plain scaled deviations: no offsets
     for (int m = 0; m < 4; ++m) P.He[m] = P.Ho[m] = 0.f;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the ticket must start at zero (a completed call leaves it at zero; this also covers a call
-    // that never completed); the partials are always written before they are read
-    cudaError_t e = cudaMemsetAsync(b + kPartialBytes, 0, 256, st);
-    if (e == cudaSuccess) e = fn(P, dim3(v.bx, v.by), st);
-    if (e == cudaSuccess && v.nlf == 0) e = cudaMemsetAsync(force_out, 0, 2 * sizeof(double), st);
+    cudaError_t e = fn(P, dim3(v.bx, v.by), st);
+    if (e == cudaSuccess && P.ngroups > 0) {
+        ForceSteps F;
+        F.dv[0] = P.dv;
+        F.force_out = P.force_out;
+        F.scale = v.inst.wall_ds ? 1.0 : -2.0 * P.s;
+        F.n = 1;
+        e = launch_pdl(sum_forces, dim3(1), dim3(128), 0, st, P, F);
+    }
+    if (e == cudaSuccess && P.ngroups == 0) e = cudaMemsetAsync(force_out, 0, 2 * sizeof(double), st);
     if (cur != v.device) cudaSetDevice(cur);
     if (e != cudaSuccess) return set_error(LBM_ECUDA, "lbm_step_noalloc: %s", cudaGetErrorString(e));
     return LBM_OK;

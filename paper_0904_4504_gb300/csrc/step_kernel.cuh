@@ -529,5 +529,7 @@ StepLaunchFn find_step_launcher(int Q, int storage, int coll, int wall = 0);
 // Plain step with an occupancy floor: variant 1 = 6 blocks of 128 per SM, 2 = 7; 3, 4 = 7 blocks with
 // 2 or 4 nodes per thread (nullptr if not built).
 StepLaunchFn find_occ_launcher(int Q, int storage, int coll, int variant);
+// The direct kernel of a variant (1-4, 30, 31), nullptr if not built.
+StepLaunchFn find_direct_launcher(int Q, int storage, int coll, int variant);
 
 }  // namespace lbm
