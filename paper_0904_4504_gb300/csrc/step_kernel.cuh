@@ -483,18 +483,26 @@ __global__ void __launch_bounds__(512) step_kernel(const __grid_constant__ InstD
 
 using StepLaunchFn = cudaError_t (*)(const InstDev& P, dim3 block, cudaStream_t stream);
 
-template <class L, class ST, int COLL, int WALL = 0>
-cudaError_t launch_step(const InstDev& P, dim3 block, cudaStream_t stream) {
-    return launch_pdl(step_kernel<L, ST, COLL, WALL>, edge_grid<WALL>(P, block.x * block.y), block, 0, stream, P);
-}
-
 // The plain step on 32 x 4 tiles with an occupancy floor: at least MINB blocks of 128 threads per
 // SM, so the compiler keeps the kernel within 65536 / (128 MINB) registers per thread.  The plain
 // kernel waits on its global loads; more resident warps hide more of that latency.
-template <class L, class ST, int COLL, int MINB>
+template <class L, class ST, int COLL, int MINB, int WALL = 0>
 __global__ void __launch_bounds__(128, MINB) step_kernel_occ(const __grid_constant__ InstDev P) {
     int tile;
-    if (!edge_block<L, ST, COLL, 0>(P, 128, tile)) bulk_tile<L, ST, COLL>(P, tile);
+    if (!edge_block<L, ST, COLL, WALL>(P, 128, tile)) bulk_tile<L, ST, COLL>(P, tile);
+}
+
+// Diffuse walls: the boundary blocks' wall rule takes 128 registers, which would leave the bulk blocks at 16
+// warps per SM; on tiles of 128 nodes FP32 D2Q37 is held to six blocks (the rule spills, the bulk not)
+// where the bulk is what counts: 1024^2 52.1 -> 45.5 us a step, but 512^2 FP16 12.6 -> 14.0 and 32 x 4096 7.8
+// -> 9.0, so from 4096 tiles on.
+template <class L, class ST, int COLL, int WALL = 0>
+cudaError_t launch_step(const InstDev& P, dim3 block, cudaStream_t stream) {
+    if constexpr (WALL == 1 && L::Q == 37 && sizeof(ST) < 8) {
+        if (block.x * block.y == 128 && P.ntiles >= 4096)
+            return launch_pdl(step_kernel_occ<L, ST, COLL, 6, 1>, edge_grid<1>(P, 128), block, 0, stream, P);
+    }
+    return launch_pdl(step_kernel<L, ST, COLL, WALL>, edge_grid<WALL>(P, block.x * block.y), block, 0, stream, P);
 }
 
 template <class L, class ST, int COLL, int MINB>
