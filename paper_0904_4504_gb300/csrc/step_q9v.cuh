@@ -5,9 +5,8 @@
 // per-thread kernels spend most of their instructions on addressing, per-element loads, stores and
 // conversions.  Here each thread owns N x-neighbouring nodes (x0 .. x0 + N - 1, x0 a multiple of N, so
 // 8-byte aligned in every row of every plane): per direction it loads the N stored values of its source
-// row with one 8-byte load, takes the value shifted in by c_x = +1 or -1 from the neighbouring lane (warp
-// shuffle) or, at a warp's ends and the periodic seam, with one single load, evaluates the collision of
-// two nodes at a time (V2), and stores the N outputs of each direction with one 8-byte store.  A warp
+// row with one 8-byte load and the value shifted in by c_x = +1 or -1 with a single one, evaluates the
+// collision of two nodes at a time (V2), and stores the N outputs of each direction with one 8-byte store.  A warp
 // covers 32 N nodes of one row, a block 32 N x 4.  Nodes with blocked links are left to the boundary
 // blocks.
 #pragma once
@@ -23,10 +22,6 @@ template <class ST> struct Vec8 {
     using One = unsigned short;  // one stored value
     uint2 v;
     __device__ __forceinline__ void load(const ST* p) { v = *reinterpret_cast<const uint2*>(p); }
-    __device__ __forceinline__ unsigned first() const { return v.x; }   // words holding the first and the last
-    __device__ __forceinline__ unsigned last() const { return v.y; }
-    static __device__ __forceinline__ One from_first(unsigned w) { return (One)(w & 0xffffu); }
-    static __device__ __forceinline__ One from_last(unsigned w) { return (One)(w >> 16); }
     static __device__ __forceinline__ float value(One o) { return H::lo((unsigned)o); }
     __device__ __forceinline__ float get(int e) const {
         return e == 0 ? H::lo(v.x) : e == 1 ? H::hi(v.x) : e == 2 ? H::lo(v.y) : H::hi(v.y);
@@ -47,10 +42,6 @@ template <> struct Vec8<float> {
     using One = float;
     float2 v;
     __device__ __forceinline__ void load(const float* p) { v = *reinterpret_cast<const float2*>(p); }
-    __device__ __forceinline__ unsigned first() const { return __float_as_uint(v.x); }
-    __device__ __forceinline__ unsigned last() const { return __float_as_uint(v.y); }
-    static __device__ __forceinline__ One from_first(unsigned w) { return __uint_as_float(w); }
-    static __device__ __forceinline__ One from_last(unsigned w) { return __uint_as_float(w); }
     static __device__ __forceinline__ float value(One o) { return o; }
     __device__ __forceinline__ float get(int e) const { return e == 0 ? v.x : v.y; }
     __device__ __forceinline__ void set(int, One o) { v.y = o; }
@@ -67,46 +58,34 @@ struct Q9Row {
     typename Vec8<ST>::One sh[9];
 };
 
-// Loads of the row y of a thread's nodes (warp-uniform y: the shuffles need the whole warp; `any`: this
-// thread owns a node inside the grid).
+// Loads of the row y of a thread's nodes.  The value shifted in is a load of its own, from the line the
+// neighbouring lane reads anyway: no lane depends on another's load, and the seam is only another address.
 template <class ST>
-__device__ __forceinline__ void q9v_load(const InstDev& P, int x0, int y, int lane, bool any, Q9Row<ST>& R) {
+__device__ __forceinline__ void q9v_load(const InstDev& P, int x0, int y, Q9Row<ST>& R) {
     using L = D2Q9;
     using W = Vec8<ST>;
     using One = typename W::One;
     constexpr int N = W::N;
-    const ST* __restrict__ src = static_cast<const ST*>(P.src);
-    const unsigned plane = (unsigned)P.plane;
-    const int nx = P.nx, ny = P.ny, pitch = P.pitch;
-    int ys[3];  // source row of c_y = -1, 0, +1
+    const int nx = P.nx, ny = P.ny;
+    const unsigned long long plane = (unsigned)P.plane;
+    const int xl = x0 == 0 ? nx - 1 : x0 - 1;   // neighbour columns (periodic)
+    const int xr = x0 + N >= nx ? x0 + N - nx : x0 + N;
+    const bool ragged = x0 + N > nx;            // the row ends inside this vector
+    const One* row[3];                          // source row of c_y = -1, 0, +1
 #pragma unroll
     for (int d = -1; d <= 1; ++d) {
         int r = y - d;
         r += r < 0 ? ny : 0;
         r -= r >= ny ? ny : 0;
-        ys[d + 1] = r;
+        row[d + 1] = static_cast<const One*>(P.src) + (unsigned)(r * P.pitch);
     }
-    const int xl = x0 == 0 ? nx - 1 : x0 - 1;   // left neighbour column (periodic)
-    const int xr = x0 + N >= nx ? x0 + N - nx : x0 + N;
-    const bool edge_l = lane == 0 || x0 == 0;
-    const bool edge_r = lane == 31 || x0 + N >= nx;
-    const bool ragged = any && x0 + N > nx;     // the row ends inside this vector
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        const int cx = cx_of<L>(i), cy = cy_of<L>(i);
-        const unsigned rowoff = (unsigned)(i * plane + ys[cy + 1] * pitch);
-        const One* r = reinterpret_cast<const One*>(src) + rowoff;
-        R.w[i].v = {};
-        if (any) R.w[i].load(src + rowoff + x0);
-        R.sh[i] = One{};
-        if (cx == 1) {
-            R.sh[i] = W::from_last(__shfl_up_sync(0xffffffffu, R.w[i].last(), 1));
-            if (edge_l && any) R.sh[i] = r[xl];
-        } else if (cx == -1) {
-            R.sh[i] = W::from_first(__shfl_down_sync(0xffffffffu, R.w[i].first(), 1));
-            if (edge_r && any && !ragged) R.sh[i] = r[xr];
-            if (ragged) R.w[i].set(nx - x0, r[0]);  // the element after the row's last node is column 0
-        }
+        const int cx = cx_of<L>(i);
+        const One* r = row[cy_of<L>(i) + 1];
+        R.w[i].load(reinterpret_cast<const ST*>(r + x0 + plane * (unsigned)i));
+        R.sh[i] = cx == 1 ? (r + xl)[plane * (unsigned)i] : cx == -1 ? (r + xr)[plane * (unsigned)i] : One{};
+        if (cx == -1 && ragged) R.w[i].set(nx - x0, r[plane * (unsigned)i]);  // the element after the last node is column 0
     }
 }
 
@@ -117,8 +96,8 @@ __device__ __forceinline__ void q9v_compute(const InstDev& P, int x0, int y, uns
     using L = D2Q9;
     using W = Vec8<ST>;
     constexpr int Q = 9, N = W::N;
-    const unsigned plane = (unsigned)P.plane;
-    ST* __restrict__ dst = static_cast<ST*>(P.dst) + (size_t)y * P.pitch + x0;
+    const unsigned long long plane = (unsigned)P.plane;
+    ST* __restrict__ dst = static_cast<ST*>(P.dst) + (unsigned)(y * P.pitch + x0);
     W o[Q];
     // value of direction i pulled to node j of this thread
     auto pulled = [&](int i, int j) -> float {
@@ -135,13 +114,13 @@ __device__ __forceinline__ void q9v_compute(const InstDev& P, int x0, int y, uns
     }
     if (cls == 0u) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) o[i].store(dst + (size_t)i * plane);
+        for (int i = 0; i < Q; ++i) o[i].store(dst + plane * (unsigned)i);
     } else {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
 #pragma unroll
             for (int j = 0; j < N; ++j)
-                if (((cls >> (8 * j)) & 0xffu) == NODE_BULK) o[i].store1(dst + (size_t)i * plane, j);
+                if (((cls >> (8 * j)) & 0xffu) == NODE_BULK) o[i].store1(dst + plane * (unsigned)i, j);
         }
     }
 }
@@ -162,9 +141,9 @@ __global__ void __launch_bounds__(128, MINB) step_kernel_q9v(const __grid_consta
         cls = N == 4 ? *reinterpret_cast<const unsigned*>(c) : (unsigned)*reinterpret_cast<const unsigned short*>(c);
     }
     pdl_wait_then_release();
-    if (y >= P.ny) return;  // warp-uniform
+    if (y >= P.ny || x0 >= P.nx) return;
     Q9Row<ST> R;
-    q9v_load<ST>(P, x0, y, lane, x0 < P.nx, R);
+    q9v_load<ST>(P, x0, y, R);
     if (cls != solid) q9v_compute<ST, COLL>(P, x0, y, cls, R);
 }
 
