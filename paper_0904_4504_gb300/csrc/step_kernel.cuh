@@ -415,6 +415,7 @@ __device__ __forceinline__ void boundary_block(const InstDev& P, int b) {
     const bool has = lane < 32 && k < P.nb;
     const uint2 at = has ? P.bnodes[k] : make_uint2(0u, 0u);
     const ulonglong2 lk = has ? P.blinks[k] : make_ulonglong2(0ull, 0ull);
+    prepare_collision<ST>();
     pdl_wait_then_release();
     if (lane >= 32 || (!WALL && !has)) return;
     double2 F[1] = {make_double2(0.0, 0.0)};
@@ -470,6 +471,7 @@ __device__ __forceinline__ void bulk_tile(const InstDev& P, int tile) {
     const int y = (tile / P.ntx) * blockDim.y + threadIdx.y;
     const bool inside = x < P.nx && y < P.ny;
     const int cls = inside ? (int)P.cls[y * P.pitch + x] : (int)NODE_SOLID;
+    prepare_collision<ST>();
     pdl_wait_then_release();
     if (inside) bulk_node<L, ST, COLL>(P, x, y, cls);
 }
