@@ -11,10 +11,12 @@
 // until the process exits.
 //
 // The kernel is the simulation's own step kernel, where it reads the populations directly and the
-// caller's buffers are aligned for it, else the plain one; a second launch sums the force (sum_forces), so
-// that there is no counter to clear before the step.
+// caller's buffers are aligned for it, else the plain one.  Each call takes the next of a ring of tickets, and
+// the last force group of a call clears its own and the one after it: no launch before the step, and a call
+// that never completed leaves nothing to the next.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "lbm.h"
@@ -23,12 +25,13 @@
 
 namespace {
 
-// Scratch: the group partials of the force (16 B each), then the non-finite flag.  With bounce-back walls a
+// Scratch: the group partials of the force (16 B each), then the non-finite flag and the tickets.  With bounce-back walls a
 // step has at most kMaxForceGroups groups; with diffuse walls one per 32 nodes with body links, and a
 // geometry is accepted with up to LBM_NOALLOC_MAX_SLOTS tiles holding such nodes, 512 in a tile at most.
 // Shared by every call in the process on a given device.
 constexpr size_t kPartialBytes = (size_t)LBM_NOALLOC_MAX_SLOTS * 16 * sizeof(double2);
-constexpr size_t kScratchBytes = kPartialBytes + 256;
+constexpr int kTickets = 56;
+constexpr size_t kScratchBytes = kPartialBytes + 256;  // flag at 0, tickets from 32
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
@@ -96,7 +99,11 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     P.src = g_in;
     P.dst = g_out;
     P.partials = reinterpret_cast<double2*>(b);
-    P.ticket = nullptr;
+    static std::atomic<unsigned> calls{0};
+    const unsigned call = calls.fetch_add(1u);
+    unsigned int* tickets = reinterpret_cast<unsigned int*>(b + kPartialBytes + 32);
+    P.ticket = tickets + call % kTickets;
+    P.ticket_next = tickets + (call + 1) % kTickets;
     P.err = reinterpret_cast<int*>(b + kPartialBytes);
     P.force_out = reinterpret_cast<double2*>(force_out);
     P.ngroups = v.nlf;
@@ -106,14 +113,6 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     for (int m = 0; m < 4; ++m) P.He[m] = P.Ho[m] = 0.f;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = fn(P, dim3(v.bx, v.by), st);
-    if (e == cudaSuccess && P.ngroups > 0) {
-        ForceSteps F;
-        F.dv[0] = P.dv;
-        F.force_out = P.force_out;
-        F.scale = v.inst.wall_ds ? 1.0 : -2.0 * P.s;
-        F.n = 1;
-        e = launch_pdl(sum_forces, dim3(1), dim3(128), 0, st, P, F);
-    }
     if (e == cudaSuccess && P.ngroups == 0) e = cudaMemsetAsync(force_out, 0, 2 * sizeof(double), st);
     if (cur != v.device) cudaSetDevice(cur);
     if (e != cudaSuccess) return set_error(LBM_ECUDA, "lbm_step_noalloc: %s", cudaGetErrorString(e));

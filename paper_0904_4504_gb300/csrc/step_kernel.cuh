@@ -330,7 +330,10 @@ __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* fo
         __threadfence();
 #pragma unroll
         for (int f = 0; f < NF; ++f) force_sum(P, P.partials + f, NF, f == 0 ? P.dv : P.dv2, force_out + f, scale, lane);
-        if (lane == 0) *P.ticket = 0u;
+        if (lane == 0) {
+            *P.ticket = 0u;
+            if (P.ticket_next) *P.ticket_next = 0u;
+        }
     }
     return last;
 }
