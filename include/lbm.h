@@ -271,8 +271,10 @@ typedef struct lbm_batch lbm_batch; /* opaque; owned by the library */
  *                         streams, so that instances of different sizes overlap (the default);
  *   LBM_BATCH_PERSISTENT  one launch per run of the persistent kernel over all instances' tiles
  *                         for K steps (per-band step counters, no grid barrier), replayed through
- *                         a CUDA graph: staged 64 x 3 tiles (the shape of variant 27) with 16-bit
- *                         storage, plain 32 x 4 tiles otherwise (lbm_batch_set_variant). */
+ *                         a CUDA graph: plain 64 x 8 tiles, two nodes per thread, for regularized
+ *                         D2Q37 with 16-bit storage, staged 64 x 3 tiles (the shape of variant 27)
+ *                         otherwise with 16-bit storage, plain 32 x 4 tiles else
+ *                         (lbm_batch_set_variant). */
 enum { LBM_BATCH_STREAMS = 0, LBM_BATCH_PERSISTENT = 1 };
 
 /* One instance: the arguments of lbm_create plus the number of steps to run. */
@@ -334,9 +336,9 @@ int lbm_batch_set_mode(lbm_batch* batch, int mode);
  * variant 2 with FP32; for D2Q9 with FP32 or 16-bit storage variant 30; else the plain kernel on 32 x 4 tiles).  An
  * instance whose layout or wall scheme the variant does not support falls back to the plain
  * kernel.  In the persistent mode (before the first lbm_batch_add) it picks the tile code the
- * persistent kernel runs: 27 staged 64 x 3 tiles, 28 staged 128 x 3 (D2Q37), 2 plain 32 x 4
- * (D2Q37 FP32/16-bit), 0 plain 32 x 4 (the others), -1 the default of the class (27 with 16-bit
- * storage, else 2 or 0); a number the class does not build is LBM_EINVAL there.  LBM_EINVAL for a
+ * persistent kernel runs: 27 staged 64 x 3 tiles, 28 staged 128 x 3 (D2Q37), 31 plain 64 x 8, two
+ * nodes per thread (regularized D2Q37, 16-bit), 2 plain 32 x 4 (D2Q37 FP32/16-bit), 0 plain 32 x 4
+ * (the others), -1 the default of the class (31 where built, else 27 with 16-bit storage, else 2 or 0); a number the class does not build is LBM_EINVAL there.  LBM_EINVAL for a
  * number below -1. */
 int lbm_batch_set_variant(lbm_batch* batch, int variant);
 
@@ -360,7 +362,7 @@ int lbm_batch_info(lbm_batch* batch, lbm_batch_info_t* out);
  * clones of `descs` (as many as the batch's budget holds) in this batch's mode for 2 + steps batch
  * steps, the last `steps` timed.  Candidates: in the streams mode the step-kernel variants built for
  * the class (variant; segment 0); in the persistent mode the tile codes it runs for the class
- * (variants 27, 28, 2, 0) times strip lengths 4, 8, 12.  Needs device memory for the clones. */
+ * (variants 31, 27, 28, 2, 0) times strip lengths 4, 8, 12.  Needs device memory for the clones. */
 typedef struct {
     int variant;               /* lbm_batch_set_variant number                                   */
     int segment;               /* persistent mode: tile rows per strip (lbm_batch_set_segment)   */

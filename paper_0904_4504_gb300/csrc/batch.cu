@@ -171,13 +171,13 @@ int rebuild(lbm_batch* b) {
         I.start = s.start;
         I.nsteps = s.nsteps;
         I.bx = v.bx;
-        I.by = v.by;
-        I.nty = (v.ny + v.by - 1) / v.by;
+        I.by = b->by;
+        I.nty = (v.ny + b->by - 1) / b->by;
         const int ntx = v.inst.ntx, S = b->seg_tiles;
         I.band = S;
         I.nseg = ntx;
-        I.fb0 = v.inst.ngroups > 0 ? v.body_row0 / (S * v.by) : 1;
-        I.fb1 = v.inst.ngroups > 0 ? v.body_row1 / (S * v.by) : 0;
+        I.fb0 = v.inst.ngroups > 0 ? v.body_row0 / (S * b->by) : 1;
+        I.fb1 = v.inst.ngroups > 0 ? v.body_row1 / (S * b->by) : 0;
         if (!slot_running(b, s)) continue;
         // force items first, then the strips: the columns of a band follow each other, so that they run
         // side by side
@@ -256,10 +256,13 @@ int launch(lbm_batch* b, int grid, long long step0, int nsteps) {
     return LBM_OK;
 }
 
-// The persistent kernel's default variant for the batch's class: staged 64 x 3 tiles (27) with
-// 16-bit storage, plain 32 x 4 tiles otherwise (2 for D2Q37 FP32, else 0).
+// The persistent kernel's default variant for the batch's class: two nodes per thread (31) for regularized
+// D2Q37 with 16-bit storage (16 FP16 instances of 256 to 1024 a side 206 us a step, staged 64 x 3 tiles 242;
+// 64 of them 872, 955; 16 of 128^2 87, 121), staged 64 x 3 tiles (27) for the others with 16-bit storage, plain
+// 32 x 4 tiles otherwise (2 for D2Q37 FP32, else 0).
 int default_pvariant(const lbm_batch* b) {
-    if (b->storage == LBM_STORE_BF16 || b->storage == LBM_STORE_F16) return 27;
+    if (b->storage == LBM_STORE_BF16 || b->storage == LBM_STORE_F16)
+        return b->Q == 37 && b->collision == LBM_COLL_REGULARIZED ? 31 : 27;
     return (b->Q == 37 && b->storage != LBM_STORE_F64) ? 2 : 0;
 }
 
@@ -397,7 +400,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         // per-step constants, tile counters (0: no step done) and the force ring (entry j free,
         // as if the step j - kRing had left it)
         const SimView v = sim_view(sim);
-        const size_t pb = pb_layout(d->nsteps, (v.ny + v.by - 1) / v.by, v.inst.ngroups, &s);
+        const size_t pb = pb_layout(d->nsteps, (v.ny + b->by - 1) / b->by, v.inst.ngroups, &s);
         std::vector<unsigned char> host(pb, 0);
         sim_step_constants(sim, d->nsteps, reinterpret_cast<StepConst*>(host.data()));
         int* fin = reinterpret_cast<int*>(host.data() + s.off_fin);
@@ -623,12 +626,12 @@ int lbm_batch_tune(lbm_batch* b, const lbm_instance_desc* descs, int n, int step
     if (!descs || n < 1 || steps < 1 || !n_out || (cap > 0 && !out))
         return set_error(LBM_EINVAL, "need instance descriptions, steps >= 1 and an output");
     // candidates: streams mode, the step kernels of the class; persistent mode, its tile paths
-    // (staged 27 and 28, plain 2 and 0) times the strip lengths
+    // (two nodes per thread 31, staged 27 and 28, plain 2 and 0) times the strip lengths
     std::vector<lbm_batch_tune_entry> cand;
     if (b->mode == LBM_BATCH_STREAMS) {
         for (int v : {0, 1, 2, 10, 20, 26, 27, 28, 30, 31, 32}) cand.push_back(lbm_batch_tune_entry{v, 0, 0.0});
     } else {
-        for (int v : {27, 28, 2, 0})
+        for (int v : {31, 27, 28, 2, 0})
             if (find_pbatch_kernel(b->Q, b->storage, b->collision, v).func)
                 for (int sg : {4, 8, 12}) cand.push_back(lbm_batch_tune_entry{v, sg, 0.0});
     }

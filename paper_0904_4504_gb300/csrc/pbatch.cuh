@@ -25,7 +25,8 @@
 // steps of one instance can be in flight at once.
 //
 // The tile code is that of the single-instance kernels (staged TMA tiles of BX x NR nodes, one
-// thread per column, or plain tiles of 32 x 4 nodes with global loads), so every instance is
+// thread per column; plain tiles of 32 x 4 nodes with global loads; or, regularized D2Q37 with 16-bit
+// storage, plain tiles of 64 x 8 nodes with two nodes per thread), so every instance is
 // computed exactly as lbm_step computes it with the same tile shape.  The populations other blocks
 // of the launch wrote are read after an acquire of their band counters: by TMA (after a proxy
 // fence) or by plain weak loads, never through the read-only path.
@@ -34,7 +35,7 @@
 #include <cuda.h>
 #include <stddef.h>
 
-#include "step_tma.cuh"
+#include "step_q37v.cuh"
 
 namespace lbm {
 
@@ -75,7 +76,13 @@ struct alignas(64) PInst {
 
 constexpr int kForceItemGroups = 4;  // force groups per warp of a force item
 
-enum PbPath { PB_STAGED = 0, PB_PLAIN = 1 };
+// PB_PAIR: plain, two nodes per thread; each of four warps takes every fourth row of its 64 x 8 tile.  Bound
+// by the strips' load latency: 16 warps of 57 loads each, 128 registers, and the bulk of a step's items is long
+// enough that the item's prologue (about 3 us of 90) does not show.  16 FP16 instances of 256 to 1024 a side
+// 205 us a step (0.75 of the copy bandwidth; staged one node per thread 235 to 245), 64 of them 868 (950).  Not
+// faster: 64 x 4 tiles at 20 warps of 96 registers 208 and 881, 128-node rows 252 and 924, staged 128 x 2
+// pairs 366 and 1057 (blocks too short-lived between waits).
+enum PbPath { PB_STAGED = 0, PB_PLAIN = 1, PB_PAIR = 2 };
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
     int v;
@@ -163,11 +170,19 @@ struct PbArgs {
     long long limit;              // clock cycles a wait may take
 };
 
+// A boundary node, out of line: its registers do not weigh on the pairs' code.
+template <class L, class ST, int COLL>
+__device__ __noinline__ void pb_boundary(const InstDev& P, int x, int y) {
+    typename StoreT<ST>::CT h[L::Q];
+    gather_global<L, ST, true>(P, static_cast<const ST*>(P.src), x, y, h);
+    tile_node<L, ST, COLL, true>(P, P.src, P.dst, x, y, NODE_BOUNDARY, P.dv, P.dv_f, h);
+}
+
 template <class L, class ST, int COLL, int PATH, int BX, int NR, int MINB>
 struct PbShape {
     static constexpr int THREADS = PATH == PB_STAGED ? BX : 128;
-    static constexpr int TX = PATH == PB_STAGED ? BX : 32;   // tile in nodes
-    static constexpr int TY = PATH == PB_STAGED ? NR : 4;
+    static constexpr int TX = PATH == PB_STAGED ? BX : PATH == PB_PAIR ? 64 : 32;   // tile in nodes
+    static constexpr int TY = PATH == PB_PLAIN ? 4 : NR;
     using G = TmaGeom<L, ST, 1, BX, NR>;
     static constexpr int SMEM = PATH == PB_STAGED ? G::SMEM : 0;
 };
@@ -307,16 +322,32 @@ __global__ void __launch_bounds__(PbShape<L, ST, COLL, PATH, BX, NR, MINB>::THRE
                         gather_global<L, ST, true>(P, static_cast<const ST*>(P.src), x, y, h);
                     tile_node<L, ST, COLL, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h);
                 }
+            } else if constexpr (PATH == PB_PAIR) {
+                const int x = tx * 64 + 2 * threadIdx.x;
+#pragma unroll 1
+                for (int r = 0; r < NR; r += 4) {
+                    const int y = ty * NR + r + threadIdx.y;
+                    if (x >= P.nx || y >= P.ny) break;
+                    // the pulls of any node inside the grid are in bounds: they do not wait for the class
+                    const unsigned c = *reinterpret_cast<const unsigned short*>(P.cls + y * P.pitch + x);
+                    PairWords<L> W;
+                    pair_load<L, ST, true>(P, x, y, W);
+                    if (pair_bulk(c)) pair_compute<L, ST, COLL>(P, x, y, c, W);
+                    // boundary nodes one by one
+                    if (c & (NODE_BOUNDARY << 8 | NODE_BOUNDARY)) {
+#pragma unroll 1
+                        for (int e = 0; e < 2; ++e)
+                            if (((c >> (8 * e)) & 0xffu) == NODE_BOUNDARY) pb_boundary<L, ST, COLL>(P, x + e, y);
+                    }
+                }
             } else {
                 const int x = tx * 32 + threadIdx.x;
                 const int y = ty * 4 + threadIdx.y;
                 if (x < P.nx && y < P.ny) {
                     const int c = (int)P.cls[y * P.pitch + x];
-                    if (c != NODE_SOLID) {
-                        typename StoreT<ST>::CT h[L::Q];
-                        gather_global<L, ST, true>(P, static_cast<const ST*>(P.src), x, y, h);
-                        tile_node<L, ST, COLL, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h);
-                    }
+                    typename StoreT<ST>::CT h[L::Q];
+                    gather_global<L, ST, true>(P, static_cast<const ST*>(P.src), x, y, h);
+                    if (c != NODE_SOLID) tile_node<L, ST, COLL, true>(P, P.src, P.dst, x, y, c, P.dv, P.dv_f, h);
                 }
             }
             if (PATH == PB_STAGED) __syncthreads();  // the stage is free for the next tile
@@ -354,8 +385,8 @@ PbKernel pbatch_kernel_info() {
 
 // The persistent kernel of a (lattice, storage, collision) class, by the variant whose tile code it
 // runs (lbm_set_variant numbers): 27 = staged 64 x 3 tiles, 28 = staged 128 x 3 tiles (D2Q37),
-// 2 = plain 32 x 4 tiles (D2Q37, 4- and 2-byte storage), 0 = plain 32 x 4 tiles (the others);
-// func is null if not built.
+// 31 = plain 64 x 8 tiles, two nodes per thread (D2Q37, 16-bit storage, regularized), 2 = plain 32 x 4
+// tiles (D2Q37, 4- and 2-byte storage), 0 = plain 32 x 4 tiles (the others); func is null if not built.
 PbKernel find_pbatch_kernel(int Q, int storage, int coll, int variant);
 
 }  // namespace lbm

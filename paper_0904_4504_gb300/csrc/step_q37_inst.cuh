@@ -28,6 +28,8 @@ PbKernel q37_pbatch_c(int variant) {
             return pbatch_kernel_info<D2Q37, ST, COLL, PB_STAGED, 64, 3, sizeof(ST) == 2 ? 11 : 6>();
         if (variant == 28) return pbatch_kernel_info<D2Q37, ST, COLL, PB_STAGED, 128, 3, sizeof(ST) == 2 ? 6 : 3>();
         if (variant == 2) return pbatch_kernel_info<D2Q37, ST, COLL, PB_PLAIN, 32, 4, 6>();
+        if constexpr (sizeof(ST) == 2 && COLL == COLL_REG)
+            if (variant == 31) return pbatch_kernel_info<D2Q37, ST, COLL, PB_PAIR, 64, 8, 4>();
     } else {
         if (variant == 0) return pbatch_kernel_info<D2Q37, ST, COLL, PB_PLAIN, 32, 4, 3>();
     }

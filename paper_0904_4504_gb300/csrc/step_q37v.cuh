@@ -35,9 +35,25 @@ __device__ __forceinline__ V2 pair_value(const PairWords<L>& W, int i) {
     return cx_of<L>(i) & 1 ? V2{H::hi(W.a[i]), H::lo(W.b[i])} : V2{H::lo(W.a[i]), H::hi(W.a[i])};
 }
 
+// Plain loads, or (COH) weak loads that never take the read-only path (see StoreT::ldc).
+template <bool COH>
+__device__ __forceinline__ unsigned load_word(const unsigned* p) {
+    if (!COH) return *p;
+    unsigned v;
+    asm volatile("ld.global.ca.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+template <bool COH>
+__device__ __forceinline__ unsigned load_half(const unsigned short* p) {
+    if (!COH) return *p;
+    unsigned short v;
+    asm volatile("ld.global.ca.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
 // Away from the seam the words lie at compile-time offsets from the node's place in the source row, one
 // widening multiply-add per direction; threads within the reach of the seam read value by value.
-template <class L, class ST>
+template <class L, class ST, bool COH = false>
 __device__ __forceinline__ void pair_load(const InstDev& P, int x0, int y, PairWords<L>& W) {
     constexpr int R = L::R;
     const unsigned char* __restrict__ src = static_cast<const unsigned char*>(P.src);
@@ -59,8 +75,8 @@ __device__ __forceinline__ void pair_load(const InstDev& P, int x0, int y, PairW
             const int cx = cx_of<L>(i);
             const unsigned* w = reinterpret_cast<const unsigned*>(row[cy_of<L>(i) + R] + (unsigned long long)plane2 * (unsigned)i);
             // odd c_x: the first node's element x0 - cx is the upper half of the word before it
-            W.a[i] = cx & 1 ? w[(-cx - 1) / 2] : w[-cx / 2];
-            W.b[i] = cx & 1 ? w[(-cx + 1) / 2] : 0u;
+            W.a[i] = load_word<COH>(w + (cx & 1 ? (-cx - 1) / 2 : -cx / 2));
+            W.b[i] = cx & 1 ? load_word<COH>(w + (-cx + 1) / 2) : 0u;
         }
     } else {
         unsigned xs[2 * R + 2];  // columns x0 - R .. x0 + R + 1, periodic
@@ -75,10 +91,57 @@ __device__ __forceinline__ void pair_load(const InstDev& P, int x0, int y, PairW
         for (int i = 0; i < L::Q; ++i) {
             const int cx = cx_of<L>(i);
             const unsigned short* r = reinterpret_cast<const unsigned short*>(row[cy_of<L>(i) + R] + (unsigned long long)plane2 * (unsigned)i);
-            const unsigned v0 = r[xs[R - cx]], v1 = r[xs[R - cx + 1]];
+            const unsigned v0 = load_half<COH>(r + xs[R - cx]), v1 = load_half<COH>(r + xs[R - cx + 1]);
             W.a[i] = cx & 1 ? v0 << 16 : v0 | v1 << 16;
             W.b[i] = v1;
         }
+    }
+}
+
+// Collision and store of a pair of row y from its words; cls: the two classes, a byte each (bulk nodes only).
+template <class L, class ST, int COLL>
+__device__ __forceinline__ void pair_compute(const InstDev& P, int x0, int y, unsigned cls, const PairWords<L>& W) {
+    using H = Half16<ST>;
+    const bool off = COLL == COLL_BGK && P.stream_off;
+    const auto at = [&](int i) {
+        const V2 v = pair_value<L, ST>(W, i);
+        return off ? vadds(v, off_l<L>(P, i)) : v;
+    };
+    const Coef<V2> C = coefficients<L, ST, COLL, V2>(P, P.dv, P.dv_f, moments<L, V2>(at));
+    unsigned char* __restrict__ dst = static_cast<unsigned char*>(P.dst) + 2ull * (unsigned)(y * P.pitch + x0);
+    const unsigned plane2 = 2u * (unsigned)P.plane;
+    if (cls == 0u) {
+        // (no memory clobber before the last store: where P lies in shared memory -- the persistent batch kernel --
+        // its constants would be read again after each, 903 us a step of 64 instances instead of 881)
+        emit_outputs<L, ST, COLL, V2>(P, C, at, [&](int i, V2 v) {
+            asm volatile("st.global.b32 [%0], %1;" ::"l"(dst + (unsigned long long)plane2 * (unsigned)i), "r"(H::pack(v.x, v.y)));
+        });
+        asm volatile("" ::: "memory");
+    } else {
+        // one of the two is a bulk node: its half of each word
+        const bool first = (cls & 0xffu) == NODE_BULK;
+        emit_outputs<L, ST, COLL, V2>(P, C, at, [&](int i, V2 v) {
+            const unsigned w = H::pack(v.x, v.y);
+            unsigned short* p = reinterpret_cast<unsigned short*>(dst + (unsigned long long)plane2 * (unsigned)i);
+            if (first) *p = (unsigned short)w;
+            else p[1] = (unsigned short)(w >> 16);
+        });
+    }
+}
+
+// Whether a pair holds a bulk node.
+__device__ __forceinline__ bool pair_bulk(unsigned cls) { return (cls & 0xffu) == NODE_BULK || cls >> 8 == NODE_BULK; }
+
+// The words of a pair from a staged tile of box width G::BW: row j, columns 2 tx, 2 tx + 1 of the tile.
+template <class G, class L>
+__device__ __forceinline__ void pair_stage(const unsigned char* stage, int tx, int j, PairWords<L>& W) {
+    const unsigned char* base = stage + 2 * (j * G::BW + G::PAD) + 4 * tx;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const int cx = cx_of<L>(i);
+        const unsigned* w = reinterpret_cast<const unsigned*>(base + i * G::SLOT);
+        W.a[i] = cx & 1 ? w[(-cx - 1) / 2] : w[-cx / 2];
+        W.b[i] = cx & 1 ? w[(-cx + 1) / 2] : 0u;
     }
 }
 
@@ -92,7 +155,6 @@ inline int pair_edge_rows(const InstDev& P, int ntx, int threads) {
 
 template <class L, class ST, int COLL, int BT, int MINB>
 __global__ void __launch_bounds__(BT, MINB) step_kernel_pair16(const __grid_constant__ InstDev P, int edge_rows) {
-    using H = Half16<ST>;
     const int r = blockIdx.z * kPairGridRows + blockIdx.y;
     if (r < edge_rows) {
         const int e = r * gridDim.x + blockIdx.x, nbb = boundary_blocks(P.nb);
@@ -111,30 +173,7 @@ __global__ void __launch_bounds__(BT, MINB) step_kernel_pair16(const __grid_cons
     // the pulls of any node inside the grid are in bounds: they do not wait for the class
     PairWords<L> W;
     pair_load<L, ST>(P, x0, y, W);
-    const bool b0 = (cls & 0xffu) == NODE_BULK, b1 = (cls >> 8) == NODE_BULK;
-    if (!b0 && !b1) return;
-    const bool off = COLL == COLL_BGK && P.stream_off;
-    const auto at = [&](int i) {
-        const V2 v = pair_value<L, ST>(W, i);
-        return off ? vadds(v, off_l<L>(P, i)) : v;
-    };
-    const Coef<V2> C = coefficients<L, ST, COLL, V2>(P, P.dv, P.dv_f, moments<L, V2>(at));
-    unsigned char* __restrict__ dst = static_cast<unsigned char*>(P.dst) + 2ull * (unsigned)(y * P.pitch + x0);
-    const unsigned plane2 = 2u * (unsigned)P.plane;
-    if (cls == 0u) {
-        emit_outputs<L, ST, COLL, V2>(P, C, at, [&](int i, V2 v) {
-            asm volatile("st.global.b32 [%0], %1;" ::"l"(dst + (unsigned long long)plane2 * (unsigned)i), "r"(H::pack(v.x, v.y))
-                         : "memory");
-        });
-    } else {
-        // one of the two is a bulk node: its half of each word
-        emit_outputs<L, ST, COLL, V2>(P, C, at, [&](int i, V2 v) {
-            const unsigned w = H::pack(v.x, v.y);
-            unsigned short* p = reinterpret_cast<unsigned short*>(dst + (unsigned long long)plane2 * (unsigned)i);
-            if (b0) *p = (unsigned short)w;
-            else p[1] = (unsigned short)(w >> 16);
-        });
-    }
+    if (pair_bulk(cls)) pair_compute<L, ST, COLL>(P, x0, y, cls, W);
 }
 
 template <class L, class ST, int COLL, int BT, int MINB>
@@ -159,7 +198,6 @@ cudaError_t launch_step_pair16(const InstDev& P, dim3, cudaStream_t stream) {
 template <class L, class ST, int COLL, int BT, int NR, int MINB>
 __global__ void __launch_bounds__(BT, MINB) step_kernel_pair16s(const __grid_constant__ InstDev P,
                                                                 const __grid_constant__ CUtensorMap map, int edge_rows) {
-    using H = Half16<ST>;
     using G = TmaGeom<L, ST, 1, 2 * BT, NR>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
@@ -206,48 +244,16 @@ __global__ void __launch_bounds__(BT, MINB) step_kernel_pair16s(const __grid_con
             return;
         }
     }
-    const unsigned plane2 = 2u * (unsigned)P.plane;
 #pragma unroll 1
     for (int j = 0; j < NR; ++j) {
         const unsigned c = cls[0];
 #pragma unroll
         for (int q = 0; q + 1 < NR; ++q) cls[q] = cls[q + 1];
-        const bool b0 = (c & 0xffu) == NODE_BULK, b1 = (c >> 8) == NODE_BULK;
-        if (!b0 && !b1) continue;
-        const int y = y0 + j;
+        if (!pair_bulk(c)) continue;
         PairWords<L> W;
-        if (interior) {
-            const unsigned char* base = smem + 2 * (j * G::BW + G::PAD) + 4 * threadIdx.x;
-#pragma unroll
-            for (int i = 0; i < L::Q; ++i) {
-                const int cx = cx_of<L>(i);
-                const unsigned* w = reinterpret_cast<const unsigned*>(base + i * G::SLOT);
-                W.a[i] = cx & 1 ? w[(-cx - 1) / 2] : w[-cx / 2];
-                W.b[i] = cx & 1 ? w[(-cx + 1) / 2] : 0u;
-            }
-        } else {
-            pair_load<L, ST>(P, x0, y, W);
-        }
-        const bool off = COLL == COLL_BGK && P.stream_off;
-        const auto at = [&](int i) {
-            const V2 v = pair_value<L, ST>(W, i);
-            return off ? vadds(v, off_l<L>(P, i)) : v;
-        };
-        const Coef<V2> C = coefficients<L, ST, COLL, V2>(P, P.dv, P.dv_f, moments<L, V2>(at));
-        unsigned char* __restrict__ dst = static_cast<unsigned char*>(P.dst) + 2ull * (unsigned)(y * P.pitch + x0);
-        if (c == 0u) {
-            emit_outputs<L, ST, COLL, V2>(P, C, at, [&](int i, V2 v) {
-                asm volatile("st.global.b32 [%0], %1;" ::"l"(dst + (unsigned long long)plane2 * (unsigned)i), "r"(H::pack(v.x, v.y))
-                             : "memory");
-            });
-        } else {
-            emit_outputs<L, ST, COLL, V2>(P, C, at, [&](int i, V2 v) {
-                const unsigned w = H::pack(v.x, v.y);
-                unsigned short* p = reinterpret_cast<unsigned short*>(dst + (unsigned long long)plane2 * (unsigned)i);
-                if (b0) *p = (unsigned short)w;
-                else p[1] = (unsigned short)(w >> 16);
-            });
-        }
+        if (interior) pair_stage<G, L>(smem, threadIdx.x, j, W);
+        else pair_load<L, ST>(P, x0, y0 + j, W);
+        pair_compute<L, ST, COLL>(P, x0, y0 + j, c, W);
     }
 }
 
