@@ -356,7 +356,9 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
     if (b->mode == LBM_BATCH_PERSISTENT && !b->kernel.func && (rc = choose_kernel(b, -1))) return rc;
     HostLattice H;
     host_lattice(d->lattice, H);
-    const size_t bytes = footprint(H, d->nx, d->ny, d->geom.storage, d->geom.layout, d->nsteps, b->bx, b->by);
+    // (the pairs' tall tiles are counted as the staged ones of the class, so that a budget admits the same mix)
+    const int rows = b->mode == LBM_BATCH_PERSISTENT && b->pvariant == 31 ? 3 : b->by;
+    const size_t bytes = footprint(H, d->nx, d->ny, d->geom.storage, d->geom.layout, d->nsteps, b->bx, rows);
     if (b->used + bytes > b->budget)
         return set_error(LBM_ENOMEM, "instance needs %zu bytes, %zu of the %zu-byte budget are free", bytes,
                          b->budget - b->used, b->budget);
