@@ -667,7 +667,7 @@ def run_ours(args):
             extras["batched_mixed_precision_persistent"] = dict(
                 keep(p16, "value", "unit", "steps", "ms_per_step", "roofline", "clocks", "gpu_launches", "config"),
                 workload="sweep64-f16 in the persistent mode: one launch per 64 steps of the persistent kernel "
-                         "(staged 64 x 3 tiles, work items of one tile column x 8 tile rows) through a CUDA graph",
+                         "(tiles and strip length as tuned) through a CUDA graph",
                 speedup_vs_plain_fp32=round(p16["value"] / value, 4))
             if prec is not None:
                 extras["precision_study"] = prec
