@@ -6,7 +6,7 @@
 // of 2.8 of 4).  Here a thread owns the nodes (x0, x0 + 1), x0 even: a direction with even c_x has both
 // values in one aligned word of its source row, one with odd c_x the upper half of one word and the lower
 // half of the next; the collision runs on both nodes at once (V2, packed FP32 operations); an output is
-// one conversion and one 4-byte store for both: 510 instructions a node (regularized collision; plain
+// one conversion and one 4-byte store for both: about 510 instructions a node (regularized collision; plain
 // BGK needs the populations again for its outputs, 168 registers, and gains nothing).
 //
 // Two forms.  Direct (variant 31): the 57 loads of a thread are independent and all in flight at once; 96
