@@ -343,7 +343,9 @@ __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* fo
 // FP64 multiply-adds a link.  FP64 is slow here (an instruction holds its sub-partition's unit for 64
 // cycles whatever its active lanes), so a warp takes 32 links at a time, whoever their nodes are, and
 // the factors and the moving-wall term (geometry only) come in once per step.  `wait` runs between the
-// loads of the list and those of the populations.
+// loads of the list and those of the populations.  Lanes past the end of the list load no population: any
+// place but a body link's may hold NaN or infinities (solid nodes are never written), which a weight of 0
+// would not keep out of the sum.
 template <class L, class ST, bool COH = false, class Wait>
 __device__ __forceinline__ bool link_force(const InstDev& P, const void* src_v, int g, double2* force_out, int lane,
                                            Wait&& wait) {
@@ -355,19 +357,23 @@ __device__ __forceinline__ bool link_force(const InstDev& P, const void* src_v, 
     double2 F[1] = {make_double2(0.0, 0.0)};
     const long long first = (long long)g * 32 * P.glen + lane;
     for (int j0 = 0; j0 < P.glen; j0 += 4) {
+        bool has[4];
         uint2 e[4];
         double2 cw[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const long long k = first + 32ll * (j0 + j);
-            const bool has = j0 + j < P.glen && k < P.nfl;
-            e[j] = has ? list[k] : make_uint2(0u, 3u << 8);
-            cw[j] = has ? weights[e[j].y & 0xffu] : make_double2(0.0, 0.0);
+            has[j] = j0 + j < P.glen && k < P.nfl;
+            e[j] = has[j] ? list[k] : make_uint2(0u, 3u << 8);
+            cw[j] = has[j] ? weights[e[j].y & 0xffu] : make_double2(0.0, 0.0);
         }
         if (j0 == 0) wait();
         typename S::CT own[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) own[j] = COH ? S::ldc(src + e[j].x) : S::ld(src + e[j].x);
+        for (int j = 0; j < 4; ++j) {
+            own[j] = 0;
+            if (has[j]) own[j] = COH ? S::ldc(src + e[j].x) : S::ld(src + e[j].x);
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             // offset of the opposite direction: index 3 - c_x
