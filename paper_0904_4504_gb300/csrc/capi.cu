@@ -631,18 +631,25 @@ void fill_flinks(const lbm_sim* s, const std::vector<size_t>& count, unsigned ch
     }
 }
 
-// Make room for the force history of `need` steps.
+// Make room for the force history of `need` steps.  Everything goes through the simulation's stream: its steps
+// are ordered with that stream only, and a clear on the default stream could wait behind other work there and
+// come after them.
 int ensure_capacity(lbm_sim* s, size_t need) {
     if (need <= s->cap) return LBM_OK;
     size_t cap = std::max<size_t>(std::max<size_t>(need, 2 * s->cap), 1024);
     double2* hist = nullptr;
     CUDA_TRY(cudaMalloc((void**)&hist, cap * sizeof(double2)));
-    CUDA_TRY(cudaStreamSynchronize(s->stream));
-    CUDA_TRY(cudaMemset(hist, 0, cap * sizeof(double2)));
     // an in-place even step has already written the force of the step after it
-    const size_t keep = std::min(s->cap, (size_t)s->steps_done + (s->aa ? 1 : 0));
-    if (s->d_history && keep > 0)
-        CUDA_TRY(cudaMemcpy(hist, s->d_history, keep * sizeof(double2), cudaMemcpyDeviceToDevice));
+    const size_t keep = s->d_history ? std::min(s->cap, (size_t)s->steps_done + (s->aa ? 1 : 0)) : 0;
+    cudaError_t e = cudaMemsetAsync(hist + keep, 0, (cap - keep) * sizeof(double2), s->stream);
+    if (e == cudaSuccess && keep > 0)
+        e = cudaMemcpyAsync(hist, s->d_history, keep * sizeof(double2), cudaMemcpyDeviceToDevice, s->stream);
+    // the old history may be freed, and the next steps may run on another stream
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) {
+        cudaFree(hist);
+        return set_error(LBM_ECUDA, "force history of %zu steps: %s", need, cudaGetErrorString(e));
+    }
     if (s->own_history) cudaFree(s->d_history);
     s->device_bytes += (cap - (s->own_history ? s->cap : 0)) * sizeof(double2);
     s->d_history = hist;
