@@ -319,8 +319,8 @@ int lbm_batch_create(int lattice, int storage, int collision, size_t device_budg
     b->own_stream = true;
     if (cudaMalloc((void**)&b->d_queue, sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc((void**)&b->d_err, sizeof(int)) != cudaSuccess ||
-        cudaMemset(b->d_queue, 0, sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMemset(b->d_err, 0, sizeof(int)) != cudaSuccess)
+        cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned long long), b->stream) != cudaSuccess ||
+        cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream) != cudaSuccess)
         return fail(set_error(LBM_ENOMEM, "batch work counter"));
     for (int k = 0; k < kSubStreams; ++k)
         if (cudaStreamCreateWithFlags(&b->sub[k], cudaStreamNonBlocking) != cudaSuccess ||
@@ -408,7 +408,10 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         int* fin = reinterpret_cast<int*>(host.data() + s.off_fin);
         for (int j = 0; j < kRing; ++j) fin[j] = j - kRing + 1;
         if (cudaMalloc((void**)&s.d_pb, pb) != cudaSuccess) return undo(set_error(LBM_ENOMEM, "batch step table"));
-        if (cudaMemcpy(s.d_pb, host.data(), pb, cudaMemcpyHostToDevice) != cudaSuccess) {
+        // (a stream that this mode does not use otherwise: a copy on the default stream may still be on its way
+        // when the call returns, and one on the batch's stream would wait for a run in flight)
+        if (cudaMemcpyAsync(s.d_pb, host.data(), pb, cudaMemcpyHostToDevice, b->sub[0]) != cudaSuccess ||
+            cudaStreamSynchronize(b->sub[0]) != cudaSuccess) {
             cudaFree(s.d_pb);
             return undo(set_error(LBM_ECUDA, "batch step table upload"));
         }

@@ -1365,7 +1365,9 @@ int lbm_set_state(lbm_sim* s, const double* g, size_t count) {
                 from_double(host.data(), s->geom.storage, (size_t)pi * plane + (size_t)y * s->pitch + x, v);
             }
     }
-    CUDA_TRY(cudaMemcpy(s->buf[s->cur], host.data(), host.size(), cudaMemcpyHostToDevice));
+    // on the stream of the steps: a copy on the default stream may still be on its way when the call returns
+    CUDA_TRY(cudaMemcpyAsync(s->buf[s->cur], host.data(), host.size(), cudaMemcpyHostToDevice, s->stream));
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
     return LBM_OK;
 }
 

@@ -38,3 +38,43 @@ def test_history_that_grows(layout, calls):
             L.lbm_destroy(sim)
     assert got[0].shape == (sum(calls), 2) and (np.abs(got[0]).max(1) > 0).all()
     assert (got[0] == got[1]).all()
+
+
+def test_persistent_batch():
+    """Counters and step tables of a batch that is created, filled and run behind queued work."""
+    got = []
+    for busy in (False, True):
+        torch.cuda.synchronize()
+        _busy(busy)
+        batch = L.lbm_batch_create(37, L.LBM_STORE_F32, L.LBM_COLL_REGULARIZED)
+        try:
+            L.lbm_batch_set_mode(batch, L.LBM_BATCH_PERSISTENT)
+            slots = [L.lbm_batch_add(batch, L.make_instance(37, n, 41, 0.8, 0.05, 1100, kind=L.LBM_GEOM_BEAM, lx=7, ly=9,
+                                                            drive=L.LBM_DRIVE_WALL, u0=2e-3, eq_order=4)) for n in (45, 70)]
+            _busy(busy)
+            L.lbm_batch_run(batch, 1100)
+            L.lbm_batch_synchronize(batch)
+            got.append([L.lbm_force_history(L.lbm_batch_instance(batch, s)) for s in slots])
+        finally:
+            torch.cuda.synchronize()
+            L.lbm_batch_destroy(batch)
+    for idle, queued in zip(*got):
+        assert (np.abs(idle).max(1) > 0).all() and (idle == queued).all()
+
+
+def test_set_state():
+    rng = np.random.default_rng(3)
+    got = []
+    g = rng.uniform(-1e-4, 1e-4, (37, 47, 61))
+    for busy in (False, True):
+        sim = L.lbm_create(37, 61, 47, 0.8, 0.05, _geom(L.LBM_LAYOUT_AB))
+        try:
+            _busy(busy)
+            L.lbm_set_state(sim, g)
+            _busy(busy)
+            L.lbm_step(sim, 4)
+            got.append((L.lbm_get_state(sim), L.lbm_force_history(sim)))
+        finally:
+            torch.cuda.synchronize()
+            L.lbm_destroy(sim)
+    assert (got[0][0] == got[1][0]).all() and (got[0][1] == got[1][1]).all()
