@@ -484,8 +484,9 @@ void lbm_server_destroy(lbm_server* server);
  * exits.  A geometry with more than LBM_NOALLOC_MAX_SLOTS tiles holding body links is rejected with
  * LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer).  All calls in the process share that array: calls
  * whose work overlaps on the GPU (two streams, or two host threads) race and give wrong forces;
- * serialize them.  Nothing is carried from one call to the next, so a call that never completed does not
- * affect the next one.
+ * serialize them.  Nothing is carried from one call to the next, so a call that never completed, or that
+ * overlapped another, does not affect the calls after it.  While the stream is being captured, a clear of one
+ * word of the scratch is recorded before the step.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress) with
  * that device current; make that first call before any stream capture (a lookup that fails is
  * not remembered: the next call tries again).

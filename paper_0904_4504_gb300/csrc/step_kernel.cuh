@@ -310,6 +310,18 @@ static __global__ void __launch_bounds__(128) sum_forces(const __grid_constant__
         force_sum(P, P.partials + (size_t)k * P.ngroups, 1, F.dv[k], F.force_out + k, F.scale, threadIdx.x & 31);
 }
 
+// One lane: how many groups of the step have taken a ticket before this one.  Where calls share the ticket
+// (P.call, their increasing numbers) it holds the number of the newest call above kTicketBits bits of count: the
+// first group of a call raises it to the call's own, whatever an earlier call has left there.
+constexpr int kTicketBits = 20;
+__device__ __forceinline__ unsigned long long take_ticket(const InstDev& P) {
+    if (!P.call) return atomicAdd(P.ticket, 1u);
+    unsigned long long* word = reinterpret_cast<unsigned long long*>(P.ticket);
+    const unsigned long long first = P.call << kTicketBits;
+    atomicMax(word, first);
+    return atomicAdd(word, 1ull) - first;
+}
+
 // One warp, force group g: the lanes' parts F into the group's partial; the last group of the step to
 // finish sums them all (and returns true).
 template <int NF>
@@ -323,17 +335,14 @@ __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* fo
     if (!P.ticket) return false;  // summed for several steps at once (sum_forces)
     __threadfence();
     __syncwarp();
-    unsigned t = 0;
-    if (lane == 0) t = atomicAdd(P.ticket, 1u);
-    const bool last = __shfl_sync(0xffffffffu, t, 0) == (unsigned)(P.ngroups - 1);
+    bool last = false;
+    if (lane == 0) last = take_ticket(P) == (unsigned long long)(P.ngroups - 1);
+    last = __shfl_sync(0xffffffffu, last, 0);
     if (last) {
         __threadfence();
 #pragma unroll
         for (int f = 0; f < NF; ++f) force_sum(P, P.partials + f, NF, f == 0 ? P.dv : P.dv2, force_out + f, scale, lane);
-        if (lane == 0) {
-            *P.ticket = 0u;
-            if (P.ticket_next) *P.ticket_next = 0u;
-        }
+        if (lane == 0 && !P.call) *P.ticket = 0u;
     }
     return last;
 }
