@@ -482,8 +482,8 @@ void lbm_server_destroy(lbm_server* server);
  * Scratch: the kernel's force partials live in one static device array of the library
  * (LBM_NOALLOC_MAX_SLOTS * 256 + 256 bytes), held by every GPU that loads the library until the process
  * exits.  A geometry with more than LBM_NOALLOC_MAX_SLOTS tiles holding body links is rejected with
- * LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer).  All calls in the process share that array: calls
- * whose work overlaps on the GPU (two streams, or two host threads) race and give wrong forces;
+ * LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer; the variants 30 with FP32, 31 and 32 count tiles of
+ * 32 x 4 nodes).  All calls in the process share that array: calls whose work overlaps on the GPU (two streams, or two host threads) race and give wrong forces;
  * serialize them.  Nothing is carried from one call to the next, so a call that never completed, or that
  * overlapped another, does not affect the calls after it.  While the stream is being captured, a clear of one
  * word of the scratch is recorded before the step.

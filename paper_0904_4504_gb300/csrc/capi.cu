@@ -430,16 +430,16 @@ void constant_force(const HostLattice& H, const std::vector<size_t>& count, doub
 
 // Tiles of bx x by nodes that hold body links.
 static int body_tiles(int nx, int bx, int by, const std::vector<LinkNode>& links) {
-    const int ntx = (nx + bx - 1) / bx;
-    std::vector<uint8_t> row(ntx, 0);  // of the current row of tiles (links are in node order)
-    int n = 0, at = -1;
+    std::vector<uint8_t> row((nx + bx - 1) / bx, 0);  // of the current row of tiles (links are in node order)
+    int n = 0, y = 0;
+    size_t first = 0;                                  // first node of row y
     for (const LinkNode& ln : links) {
         if (!ln.body) continue;
-        const int tx = (int)(ln.node % (size_t)nx) / bx, ty = (int)(ln.node / (size_t)nx) / by;
-        if (ty != at) std::fill(row.begin(), row.end(), 0);
-        at = ty;
-        n += !row[tx];
-        row[tx] = 1;
+        for (; ln.node - first >= (size_t)nx; first += nx)
+            if (++y % by == 0) std::fill(row.begin(), row.end(), 0);
+        uint8_t& seen = row[(unsigned)(ln.node - first) / (unsigned)bx];
+        n += !seen;
+        seen = 1;
     }
     return n;
 }
@@ -520,7 +520,7 @@ struct lbm_sim {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int bx = 32, by = 4, ntx = 0, ntiles = 0;
-    mutable int body_tiles = -1, body_tiles_bx = 0, body_tiles_by = 0;  // sim_body_tiles
+    int slots = 0, slots_bx = 0, slots_by = 0;  // count_slots
     int plain_bx = 32, plain_by = 4;   // tile of the plain kernel (lbm_set_tile)
     int variant = 0;                   // 0 plain kernel, else a staged variant (lbm_set_variant)
     bool stream_off = false;           // 16-bit body frame: store h - H(U(n)), see InstDev
@@ -601,12 +601,26 @@ int ensure_links(lbm_sim* s) {
     return LBM_OK;
 }
 
+// Tiles with body links, which lbm_step_noalloc accepts up to LBM_NOALLOC_MAX_SLOTS of: tiles of the
+// simulation's shape, but of 32 x 4 nodes for the kernels of neighbouring nodes that lbm_create chooses by itself
+// (30 with FP32, 31, 32), so that its choice decides nothing.  Counted only where the nodes with body links are
+// more than that, here and not in the step.
+void count_slots(lbm_sim* s) {
+    const bool own = s->variant != 31 && s->variant != 32 && !(s->variant == 30 && s->geom.storage == LBM_STORE_F32);
+    const int bx = own ? s->bx : 32, by = own ? s->by : 4;
+    if (s->nbf <= LBM_NOALLOC_MAX_SLOTS || (bx == s->slots_bx && by == s->slots_by)) return;
+    s->slots = body_tiles(s->nx, bx, by, s->link_nodes);
+    s->slots_bx = bx;
+    s->slots_by = by;
+}
+
 // Tiles of the current tile shape.
 int setup_tiles(lbm_sim* s) {
     s->ntx = (s->nx + s->bx - 1) / s->bx;
     s->ntiles = s->ntx * ((s->ny + s->by - 1) / s->by);
     s->dev.ntx = s->ntx;
     s->dev.ntiles = s->ntiles;
+    count_slots(s);
     return LBM_OK;
 }
 
@@ -752,6 +766,7 @@ SimView sim_view(const lbm_sim* s) {
     v.bx = s->bx;
     v.by = s->by;
     v.nlf = s->link_groups;
+    v.slots = s->slots;
     v.body_row0 = s->body_row0;
     v.body_row1 = s->body_row1;
     v.drive = s->geom.drive;
@@ -775,15 +790,6 @@ SimView sim_view(const lbm_sim* s) {
 int sim_reserve(lbm_sim* s, size_t steps) { return ensure_capacity(s, steps); }
 
 int sim_tile_links(lbm_sim* s) { return ensure_links(s); }
-
-int sim_body_tiles(const lbm_sim* s) {
-    if (s->body_tiles < 0 || s->body_tiles_bx != s->bx || s->body_tiles_by != s->by) {
-        s->body_tiles = body_tiles(s->nx, s->bx, s->by, s->link_nodes);
-        s->body_tiles_bx = s->bx;
-        s->body_tiles_by = s->by;
-    }
-    return s->body_tiles;
-}
 
 void sim_disable_stream_offset(lbm_sim* s) {
     if (s->steps_done == 0) s->stream_off = false;

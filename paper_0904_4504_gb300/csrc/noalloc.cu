@@ -72,12 +72,11 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     if (g_in == g_out) return set_error(LBM_EINVAL, "g_in and g_out must be different buffers");
     if (n < 0) return set_error(LBM_EINVAL, "negative step index");
     const SimView v = sim_view(sim);
-    const int tiles = sim_body_tiles(sim);
-    if (tiles > LBM_NOALLOC_MAX_SLOTS)
+    if (v.slots > LBM_NOALLOC_MAX_SLOTS)
         return set_error(LBM_ERANGE,
                          "lbm_step_noalloc: the geometry has %d tiles with body links, more than the %d its static "
                          "scratch holds; use lbm_step, or a larger tile (lbm_set_tile)",
-                         tiles, LBM_NOALLOC_MAX_SLOTS);
+                         v.slots, LBM_NOALLOC_MAX_SLOTS);
     if (v.device < 0 || v.device >= kMaxDevices) return set_error(LBM_EINVAL, "device %d out of range", v.device);
     int cur = -1;
     if (cudaGetDevice(&cur) != cudaSuccess) return set_error(LBM_ECUDA, "cudaGetDevice failed");

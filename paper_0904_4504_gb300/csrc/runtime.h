@@ -40,6 +40,7 @@ struct SimView {
     int device, Q, storage, collision, nx, ny, pitch, bx, by, drive;
     int body_row0, body_row1;  // rows that hold nodes with body links
     int nlf;                   // force groups of the two-buffer bounce-back step (noalloc)
+    int slots;                 // tiles with body links as lbm_step_noalloc counts them (0: not more than it accepts)
     double u0, omega;
     InstDev inst;
     void* buf[2];
@@ -57,8 +58,6 @@ SimView sim_view(const lbm_sim* s);
 int sim_reserve(lbm_sim* s, size_t steps);
 // Make the links by node that the tile kernels read (may allocate).
 int sim_tile_links(lbm_sim* s);
-// Tiles of the simulation's tile shape that hold body links.
-int sim_body_tiles(const lbm_sim* s);
 // Store plain scaled deviations (no uniform-stream offset); only before the first step.
 void sim_disable_stream_offset(lbm_sim* s);
 // Record that `steps` steps were run on the simulation's buffers by another launcher.
