@@ -133,10 +133,11 @@ size_t pb_layout(long long nsteps, int nty, int ring_len, Slot* s) {
     return off;
 }
 
-// Device bytes of one instance (populations, geometry arrays, force history, and in the persistent
-// mode its step table, tile counters and force ring; the tile shape bx x by; the force scratch of an
-// instance is bounded by its tiles).
-size_t footprint(const HostLattice& H, int nx, int ny, int storage, int layout, long nsteps, int bx, int by) {
+// What a budget admits an instance by, from its sizes: populations, node classes and link masks by node, force
+// history, step table, and a share for lists and force scratch that goes by its tiles of bx x by nodes.  It covers
+// all but bodies whose lists are long for their grid (masks full of holes, wide and flat plates); for those the
+// instance's own need counts.
+size_t estimate(const HostLattice& H, int nx, int ny, int storage, int layout, long nsteps, int bx, int by) {
     const size_t es = storage_size(storage);
     const size_t align = 128 / es;
     const size_t pitch = (nx + align - 1) / align * align;
@@ -146,6 +147,34 @@ size_t footprint(const HostLattice& H, int nx, int ny, int storage, int layout, 
     const size_t nbuf = layout == LBM_LAYOUT_AA ? 1 : 2;
     return nbuf * plane * H.Q * es + plane * (1 + sizeof(ulonglong2)) + tiles * (sizeof(int) + 2 * sizeof(double2)) +
            hist * sizeof(double2) + pb_layout(nsteps, (int)tiles, (int)tiles, nullptr) + 4096;
+}
+
+// What an instance whose simulation holds `sim` bytes and `groups` force groups can come to hold: the link masks by
+// node too, where kernels that read them can be chosen, and the persistent mode's table, counters and force ring
+// (tiles of `by` rows).
+size_t need(size_t sim, const lbm_instance_desc& d, int groups, int by) {
+    const size_t align = 128 / storage_size(d.geom.storage), pitch = (d.nx + align - 1) / align * align;
+    const bool tiles = d.geom.wall_scheme == LBM_SCHEME_BOUNCEBACK && d.geom.layout == LBM_LAYOUT_AB;
+    return sim + (tiles ? (size_t)d.ny * pitch * sizeof(ulonglong2) : 0) +
+           pb_layout(d.nsteps, (d.ny + by - 1) / by, groups, nullptr);
+}
+
+// The question lbm_batch_add asks of an instance's creation (CreatePlan::admit).
+struct Admission {
+    const lbm_batch* b;
+    const lbm_instance_desc* d;
+    size_t bytes;    // what the instance counts: in, the estimate; out, at least its need
+};
+
+int over_budget(const lbm_batch* b, size_t bytes) {
+    return set_error(LBM_ENOMEM, "instance needs %zu bytes, %zu of the %zu-byte budget are free", bytes,
+                     b->budget - b->used, b->budget);
+}
+
+int admit_instance(void* context, size_t sim, int groups) {
+    Admission& a = *static_cast<Admission*>(context);
+    a.bytes = std::max(a.bytes, need(sim, *a.d, groups, a.b->by));
+    return a.b->used + a.bytes > a.b->budget ? over_budget(a.b, a.bytes) : LBM_OK;
 }
 
 // Rebuild the per-instance launch table and the strip list of the unfinished instances.
@@ -338,7 +367,18 @@ int lbm_batch_footprint(const lbm_instance_desc* d, size_t* bytes) {
     if (!host_lattice(d->lattice, H)) return set_error(LBM_EINVAL, "unknown lattice %d", d->lattice);
     if (!storage_size(d->geom.storage)) return set_error(LBM_EINVAL, "bad storage type");
     if (d->nx < 1 || d->ny < 1 || d->nsteps < 0) return set_error(LBM_EINVAL, "bad size");
-    *bytes = footprint(H, d->nx, d->ny, d->geom.storage, d->geom.layout, d->nsteps, 32, 4);
+    *bytes = estimate(H, d->nx, d->ny, d->geom.storage, d->geom.layout, d->nsteps, 32, 4);
+    // (sizes and geometries that lbm_batch_add refuses have no lists)
+    const size_t plane = (size_t)d->ny * (d->nx + 128);
+    if (d->nx < 2 * H.R + 1 || d->ny < 2 * H.R + 1 || H.Q * plane >= (1ull << 32)) return LBM_OK;
+    if (check_geometry(H, d->nx, d->ny, d->geom) != LBM_OK) {
+        clear_error();
+        return LBM_OK;
+    }
+    const SolidLists lists = solid_lists(H, d->nx, d->ny, d->geom);
+    const SimLayout at = sim_layout(H, d->nx, d->ny, d->geom, lists, std::max<size_t>(1024, (size_t)d->nsteps + 1), false);
+    const int groups = std::max((int)(lists.nbf + 31) / 32, force_groups((int)lists.nfl, force_group_len((int)lists.nfl)));
+    *bytes = std::max(*bytes, need(at.bytes() + (at.together ? 0 : at.nbuf * at.pop), *d, groups, 3));
     return LBM_OK;
 }
 
@@ -358,12 +398,12 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
     host_lattice(d->lattice, H);
     // (the pairs' tall tiles are counted as the staged ones of the class, so that a budget admits the same mix)
     const int rows = b->mode == LBM_BATCH_PERSISTENT && b->pvariant == 31 ? 3 : b->by;
-    const size_t bytes = footprint(H, d->nx, d->ny, d->geom.storage, d->geom.layout, d->nsteps, b->bx, rows);
-    if (b->used + bytes > b->budget)
-        return set_error(LBM_ENOMEM, "instance needs %zu bytes, %zu of the %zu-byte budget are free", bytes,
-                         b->budget - b->used, b->budget);
+    Admission asked{b, d, estimate(H, d->nx, d->ny, d->geom.storage, d->geom.layout, d->nsteps, b->bx, rows)};
+    if (b->used + asked.bytes > b->budget) return over_budget(b, asked.bytes);
+    // (+1: an in-place even step also writes the force of the step after it)
+    const CreatePlan plan{(size_t)d->nsteps + 1, admit_instance, &asked};
     lbm_sim* sim = nullptr;
-    rc = lbm_create(d->lattice, d->nx, d->ny, d->tau, d->omega, &d->geom, &sim);
+    rc = sim_create(d->lattice, d->nx, d->ny, d->tau, d->omega, &d->geom, &plan, &sim);
     if (rc) return rc;
     auto undo = [&](int code) {
         lbm_destroy(sim);
@@ -393,8 +433,6 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
     }
     if (rc) return undo(rc);
     clear_error();
-    // (+1: an in-place even step also writes the force of the step after it)
-    if ((rc = sim_reserve(sim, (size_t)d->nsteps + 1))) return undo(rc);
     if ((rc = lbm_set_stream(sim, b->mode == LBM_BATCH_STREAMS ? b->sub[id % kSubStreams] : b->stream)))
         return undo(rc);
     Slot s;
@@ -419,10 +457,10 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
     s.sim = sim;
     s.start = b->gstep;
     s.nsteps = d->nsteps;
-    s.bytes = bytes;
+    s.bytes = asked.bytes;
     if (id == (int)b->slots.size()) b->slots.push_back(s);
     else b->slots[id] = s;
-    b->used += bytes;
+    b->used += asked.bytes;
     b->dirty = true;
     *slot = id;
     return LBM_OK;

@@ -536,7 +536,8 @@ struct lbm_sim {
 
     // Steps run in longer calls leave the sum of their forces to one launch every kForceSteps steps; with many
     // groups (grids of a thousand nodes a side and more) the sum is no part of a step worth saving.
-    bool defers_forces() const { return !aa && dev.ngroups > 0 && dev.ngroups <= 1024; }
+    bool may_defer = true;             // (a batch runs its instances step by step)
+    bool defers_forces() const { return lbm::defers_forces(may_defer, aa, dev.ngroups); }
 };
 
 namespace {
@@ -624,9 +625,7 @@ int setup_tiles(lbm_sim* s) {
     return LBM_OK;
 }
 
-// Bytes of the list of the body's links (InstDev::flinks), and the list, sorted by direction, then node.
-size_t flinks_bytes(size_t n) { return kFLinkTable + n * sizeof(uint2); }
-
+// The body's links (InstDev::flinks), sorted by direction, then node.
 void fill_flinks(const lbm_sim* s, const std::vector<size_t>& count, unsigned char* host) {
     const size_t plane = (size_t)s->ny * s->pitch;
     double2* cw = reinterpret_cast<double2*>(host);
@@ -787,7 +786,53 @@ SimView sim_view(const lbm_sim* s) {
     return v;
 }
 
-int sim_reserve(lbm_sim* s, size_t steps) { return ensure_capacity(s, steps); }
+SimLayout sim_layout(const HostLattice& H, int nx, int ny, const lbm_geometry& g, const SolidLists& n, size_t history,
+                     bool may_defer) {
+    const auto up256 = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t es = storage_size(g.storage), align = 128 / es, plane = (nx + align - 1) / align * align * ny;
+    const bool aa = g.layout == LBM_LAYOUT_AA, by_links = g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
+    const int groups = aa || !by_links ? (int)((n.nbf + 31) / 32) : force_groups((int)n.nfl, force_group_len((int)n.nfl));
+    SimLayout at;
+    at.pop = up256(plane * H.Q * es);
+    at.nbuf = aa ? 1 : 2;
+    at.together = at.nbuf * at.pop <= (size_t)64 << 20;
+    at.nodes = up256(plane);
+    at.links = up256(at.nodes + n.nb * sizeof(uint2));
+    at.flinks = up256(at.links + n.nb * sizeof(ulonglong2));
+    at.zero = up256(at.flinks + (by_links ? kFLinkTable + n.nfl * sizeof(uint2) : 0));
+    const size_t partials = (size_t)std::max(1, groups) * (aa ? 2 : defers_forces(may_defer, aa, groups) ? kForceSteps : 1);
+    at.history = up256(at.zero + 256 + partials * sizeof(double2));
+    at.pops = up256(at.history + history * sizeof(double2));
+    return at;
+}
+
+// Counted, for masks; for a plate and a beam from their sides, as an upper bound: a direction's links around a
+// rectangle are what each of its gcd(|c_x|, |c_y|) steps shifts out of it.
+SolidLists solid_lists(const HostLattice& H, int nx, int ny, const lbm_geometry& g) {
+    SolidLists n{0, 0, 0};
+    const bool by_links = g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
+    if (g.kind == LBM_GEOM_PLATE) {
+        n.nb = (size_t)nx * std::min(2 * H.R, ny - 2 * H.R);
+        n.nbf = (size_t)nx * std::min(H.R, ny - 2 * H.R);
+        for (int i = 1; by_links && i < H.Q; ++i) n.nfl += (size_t)nx * std::max(0, H.c[i][1]);
+    } else if (g.kind == LBM_GEOM_BEAM) {
+        const size_t lx = g.lx, ly = g.ly;
+        n.nb = n.nbf = (lx + 2 * H.R) * (ly + 2 * H.R) - lx * ly;
+        for (int i = 1; by_links && i < H.Q; ++i) {
+            const int cx = std::abs(H.c[i][0]), cy = std::abs(H.c[i][1]), k = gcd_int(cx, cy);
+            n.nfl += k * std::min(lx * ly, cx / k * ly + cy / k * lx - (size_t)(cx / k) * (cy / k));
+        }
+    } else if (g.kind == LBM_GEOM_MASK) {
+        GeomScan scan;
+        scan_geometry(H, nx, ny, g, scan);
+        n.nb = scan.links.size();
+        for (const LinkNode& ln : scan.links) {
+            n.nbf += ln.body != 0;
+            n.nfl += by_links ? __builtin_popcountll(ln.body) : 0;
+        }
+    }
+    return n;
+}
 
 int sim_tile_links(lbm_sim* s) { return ensure_links(s); }
 
@@ -887,6 +932,13 @@ int lbm_params_from_tau_omega(int lattice, double tau_omega, double delta_min, i
 }
 
 int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_geometry* geom, lbm_sim** out) {
+    return sim_create(lattice, nx, ny, tau, omega, geom, nullptr, out);
+}
+
+}  // extern "C"
+
+int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const lbm_geometry* geom,
+                    const CreatePlan* plan, lbm_sim** out) {
     clear_error();
     if (!out) return set_error(LBM_EINVAL, "null output handle");
     *out = nullptr;
@@ -970,17 +1022,25 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     constant_force(H, link_count, g.rho0, s->fconst[0], s->fconst[1], s->fmov[0], s->fmov[1]);
 
     InstDev& d = s->dev;
-    const size_t nb = s->link_nodes.size();
     const bool by_links = g.wall_scheme == LBM_SCHEME_BOUNCEBACK;
-    size_t nfl = 0;
-    for (size_t n : link_count) nfl += by_links ? n : 0;
-    // force groups: by links for the two-buffer bounce-back step, by nodes (32 a group) otherwise
-    d.nb = (int)nb;
+    SolidLists lists{s->link_nodes.size(), (size_t)s->nbf, 0};
+    for (size_t n : link_count) lists.nfl += by_links ? n : 0;
+    // force groups: by links for the two-buffer bounce-back step, by nodes (32 a group) otherwise.  (Along one
+    // direction and its opposite at most 2 min(fluid, solid) links, or 2 fluid where a link passes over other
+    // nodes, are blocked: 18 links a node of the grid in D2Q37, 4 in D2Q9, below 2^31 with Q plane < 2^32.)
+    d.nb = (int)lists.nb;
     d.nbf = s->nbf;
-    d.nfl = (int)nfl;
-    d.glen = force_group_len((int)nfl);
+    d.nfl = (int)lists.nfl;
+    d.glen = force_group_len(d.nfl);
     s->link_groups = by_links ? force_groups(d.nfl, d.glen) : (s->nbf + 31) / 32;
     d.ngroups = s->aa ? (s->nbf + 31) / 32 : s->link_groups;
+    if (plan) s->may_defer = false;
+    s->cap = std::max<size_t>(1024, plan ? plan->history : 0);
+    const SimLayout at = sim_layout(H, nx, ny, g, lists, s->cap, s->may_defer);
+    if (plan && (rc = plan->admit(plan->context, at.bytes() + (at.together ? 0 : at.nbuf * at.pop), d.ngroups))) {
+        delete s;
+        return rc;
+    }
 
     if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) {
         delete s;
@@ -997,48 +1057,32 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
         }                       \
     } while (0)
 
-    // One block: node classes, then the uploaded lists (boundary nodes, their links, body links), then what
-    // starts at zero (ticket, error word, group partials -- of two steps, which the in-place even step
-    // records, or of the steps summed at once -- and history).  Populations of up to 64 MB join it; larger ones are allocated by
-    // themselves.  (An allocation or its release costs about 30 us, 100 us and more above 256 MB; a grid
-    // of 256^2 took ten of them.)
-    auto up256 = [](size_t v) { return (v + 255) / 256 * 256; };
-    const size_t pop = up256(plane * H.Q * es), nbuf = s->aa ? 1 : 2;
-    const bool together = nbuf * pop <= (size_t)64 << 20;
-    const size_t o_nodes = up256(plane), o_links = up256(o_nodes + nb * sizeof(uint2));
-    const size_t o_flinks = up256(o_links + nb * sizeof(ulonglong2));
-    const size_t o_zero = up256(o_flinks + (by_links ? flinks_bytes(nfl) : 0));
-    const size_t np = (size_t)std::max(1, d.ngroups) * (s->aa ? 2 : s->defers_forces() ? kForceSteps : 1);
-    const size_t o_hist = up256(o_zero + 256 + np * sizeof(double2));
-    s->cap = 1024;
-    const size_t o_pop = up256(o_hist + s->cap * sizeof(double2));
-    const size_t block = o_pop + (together ? nbuf * pop : 0);
-    TRY_OR_FREE(dev_alloc(s, &s->d_block, block));
-    for (size_t k = 0; k < nbuf; ++k) {
-        if (together) s->buf[k] = s->d_block + o_pop + k * pop;
-        else TRY_OR_FREE(dev_alloc(s, (unsigned char**)&s->buf[k], pop));
-        s->own_buf = !together;
+    TRY_OR_FREE(dev_alloc(s, &s->d_block, at.bytes()));
+    for (size_t k = 0; k < at.nbuf; ++k) {
+        if (at.together) s->buf[k] = s->d_block + at.pops + k * at.pop;
+        else TRY_OR_FREE(dev_alloc(s, (unsigned char**)&s->buf[k], at.pop));
+        s->own_buf = !at.together;
     }
     d.cls = s->d_block;
-    d.bnodes = reinterpret_cast<const uint2*>(s->d_block + o_nodes);
-    d.blinks = reinterpret_cast<const ulonglong2*>(s->d_block + o_links);
-    d.flinks = s->d_block + o_flinks;
-    d.ticket = reinterpret_cast<unsigned int*>(s->d_block + o_zero);
-    d.err = s->d_err = reinterpret_cast<int*>(s->d_block + o_zero + 128);
-    d.partials = reinterpret_cast<double2*>(s->d_block + o_zero + 256);
-    s->d_history = reinterpret_cast<double2*>(s->d_block + o_hist);
+    d.bnodes = reinterpret_cast<const uint2*>(s->d_block + at.nodes);
+    d.blinks = reinterpret_cast<const ulonglong2*>(s->d_block + at.links);
+    d.flinks = s->d_block + at.flinks;
+    d.ticket = reinterpret_cast<unsigned int*>(s->d_block + at.zero);
+    d.err = s->d_err = reinterpret_cast<int*>(s->d_block + at.zero + 128);
+    d.partials = reinterpret_cast<double2*>(s->d_block + at.zero + 256);
+    s->d_history = reinterpret_cast<double2*>(s->d_block + at.history);
 
     // lists of boundary nodes, body nodes first, and of body links
-    std::vector<unsigned char> host(o_zero - o_nodes, 0);
+    std::vector<unsigned char> host(at.zero - at.nodes, 0);
     uint2* nodes = reinterpret_cast<uint2*>(host.data());
-    ulonglong2* links = reinterpret_cast<ulonglong2*>(host.data() + (o_links - o_nodes));
+    ulonglong2* links = reinterpret_cast<ulonglong2*>(host.data() + (at.links - at.nodes));
     size_t body_place = 0, wall_place = (size_t)s->nbf;
     for (const LinkNode& ln : s->link_nodes) {
         const size_t k = ln.body ? body_place++ : wall_place++;
         nodes[k] = make_uint2((unsigned)(ln.node % (size_t)nx), (unsigned)(ln.node / (size_t)nx));
         links[k] = make_ulonglong2(ln.body, ln.wall);
     }
-    if (by_links) fill_flinks(s, link_count, host.data() + (o_flinks - o_nodes));
+    if (by_links) fill_flinks(s, link_count, host.data() + (at.flinks - at.nodes));
 
     // node classes: bulk, the padding solid, then the visited rows, run by run (many runs: all rows at once)
     cudaStream_t st = s->stream;
@@ -1064,13 +1108,13 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
         s->h2d_bytes += all.size();
     }
     if (!host.empty())
-        up = up && cudaMemcpyAsync(s->d_block + o_nodes, host.data(), host.size(), cudaMemcpyHostToDevice, st) == cudaSuccess;
+        up = up && cudaMemcpyAsync(s->d_block + at.nodes, host.data(), host.size(), cudaMemcpyHostToDevice, st) == cudaSuccess;
     s->h2d_bytes += host.size();
     // the geometry is on the device when the call returns (other streams may read it, and the host buffers
     // end here); the zeroes are in order with the simulation's own work
-    up = up && cudaMemsetAsync(s->d_block + o_zero, 0, o_pop - o_zero, st) == cudaSuccess &&
+    up = up && cudaMemsetAsync(s->d_block + at.zero, 0, at.pops - at.zero, st) == cudaSuccess &&
          cudaStreamSynchronize(st) == cudaSuccess;
-    for (size_t k = 0; up && k < nbuf; ++k) up = cudaMemsetAsync(s->buf[k], 0, pop, st) == cudaSuccess;
+    for (size_t k = 0; up && k < at.nbuf; ++k) up = cudaMemsetAsync(s->buf[k], 0, at.pop, st) == cudaSuccess;
     if (!up) {
         free_sim(s);
         return set_error(LBM_ECUDA, "upload of geometry failed");
@@ -1128,6 +1172,8 @@ int lbm_create(int lattice, int nx, int ny, double tau, double omega, const lbm_
     *out = s;
     return LBM_OK;
 }
+
+extern "C" {
 
 int lbm_set_tile(lbm_sim* s, int block_x, int block_y) {
     int rc = check_sim(s);

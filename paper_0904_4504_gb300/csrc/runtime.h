@@ -54,8 +54,43 @@ struct SimView {
     const CUtensorMap* maps;  // staged variants: load boxes of buf[0], buf[1]
 };
 SimView sim_view(const lbm_sim* s);
-// Make room for `steps` entries of force history (may allocate).
-int sim_reserve(lbm_sim* s, size_t steps);
+
+// What a geometry's device lists hold: boundary nodes, those of them with body links, and body links (bounce-back
+// walls only); of a checked geometry.
+struct SolidLists {
+    size_t nb, nbf, nfl;
+};
+SolidLists solid_lists(const HostLattice& H, int nx, int ny, const lbm_geometry& g);
+int check_geometry(const HostLattice& H, int nx, int ny, const lbm_geometry& g);
+
+// Whether the sums of the forces of a long call's steps are left to one launch every kForceSteps steps; with many
+// groups (grids of a thousand nodes a side and more) the sum is no part of a step worth saving.
+inline bool defers_forces(bool may_defer, bool aa, int groups) { return may_defer && !aa && groups > 0 && groups <= 1024; }
+
+// Device memory of a simulation, by offsets in one block: node classes, then the uploaded lists (boundary nodes,
+// their links, body links), then what starts at zero (ticket, error word, group partials -- of two steps, which
+// the in-place even step records, or of the steps summed at once -- and history).  Populations of up to 64 MB join
+// it; larger ones are allocated by themselves.  (An allocation or its release costs about 30 us, 100 us and
+// more above 256 MB; a grid of 256^2 took ten of them.)
+struct SimLayout {
+    size_t nodes, links, flinks, zero, history, pops;
+    size_t pop, nbuf;              // bytes of a population buffer, and buffers
+    bool together;
+    size_t bytes() const { return pops + (together ? nbuf * pop : 0); }  // of the block
+};
+SimLayout sim_layout(const HostLattice& H, int nx, int ny, const lbm_geometry& g, const SolidLists& n, size_t history,
+                     bool may_defer);
+
+// lbm_create for a batch: the force history holds `history` steps at once, forces are not deferred, and
+// admit(context, device bytes, force groups) is asked before anything is allocated (a code it returns is passed on).
+struct CreatePlan {
+    size_t history;
+    int (*admit)(void* context, size_t bytes, int groups);
+    void* context;
+};
+int sim_create(int lattice, int nx, int ny, double tau, double omega, const lbm_geometry* geom, const CreatePlan* plan,
+               lbm_sim** out);
+
 // Make the links by node that the tile kernels read (may allocate).
 int sim_tile_links(lbm_sim* s);
 // Store plain scaled deviations (no uniform-stream offset); only before the first step.

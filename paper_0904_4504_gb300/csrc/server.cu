@@ -258,8 +258,9 @@ int lbm_server_create(size_t device_budget_bytes, int steps_per_round, lbm_serve
 
 int lbm_server_submit(lbm_server* s, const lbm_request* req, long long* id) {
     if (!s || !req || !id) return set_error(LBM_EINVAL, "null argument");
-    const lbm_instance_desc& d = req->desc;
+    lbm_instance_desc d = req->desc;
     if (d.nsteps < 1) return set_error(LBM_EINVAL, "nsteps must be >= 1");
+    if (d.geom.kind == LBM_GEOM_MASK) d.geom.mask = nullptr;  // not served (below): its labels are not read
     size_t bytes = 0;
     int rc = lbm_batch_footprint(&d, &bytes);
     if (rc) return rc;
