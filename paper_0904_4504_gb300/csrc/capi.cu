@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "deferred.h"
 #include "lbm.h"
 #include "runtime.h"
 #include "pbatch.cuh"
@@ -536,6 +537,7 @@ struct lbm_sim {
 
     // Steps run in longer calls leave the sum of their forces to one launch every kForceSteps steps; with many
     // groups (grids of a thousand nodes a side and more) the sum is no part of a step worth saving.
+    int lost_forces = 0;               // steps that ran and whose forces could not be summed
     bool may_defer = true;             // (a batch runs its instances step by step)
     bool defers_forces() const { return lbm::defers_forces(may_defer, aa, dev.ngroups); }
 };
@@ -1241,12 +1243,9 @@ int lbm_step(lbm_sim* s, long n) {
     const bool defer = s->defers_forces() && n >= 8;
     unsigned int* const ticket = s->dev.ticket;
     double2* const partials = s->dev.partials;
-    const long first = s->steps_done;
     ForceSteps F;
-    F.n = 0;
     F.scale = s->dev.wall_ds ? 1.0 : -2.0 * s->dev.s;
-    cudaError_t e = cudaSuccess;
-    for (long k = 0; k < n && e == cudaSuccess; ++k) {
+    const auto step = [&](long, int held) {
         s->dev.src = s->buf[s->cur];
         s->dev.dst = s->buf[s->cur ^ 1];
         set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));
@@ -1260,24 +1259,29 @@ int lbm_step(lbm_sim* s, long n) {
         s->dev.force_out = s->d_history + s->steps_done;
         if (defer) {
             s->dev.ticket = nullptr;
-            s->dev.partials = partials + (size_t)F.n * s->dev.ngroups;
-            F.dv[F.n++] = s->dev.dv;
+            s->dev.partials = partials + (size_t)held * s->dev.ngroups;
+            F.dv[held] = s->dev.dv;
         }
-        e = s->tma_launch ? s->tma_launch(s->dev, s->maps[s->cur], s->store_maps[s->cur ^ 1], s->stream)
-                          : s->launch(s->dev, block, s->stream);
+        const cudaError_t e = s->tma_launch ? s->tma_launch(s->dev, s->maps[s->cur], s->store_maps[s->cur ^ 1], s->stream)
+                                            : s->launch(s->dev, block, s->stream);
         s->dev.ticket = ticket;
         s->dev.partials = partials;
-        if (e == cudaSuccess && defer && (F.n == kForceSteps || k + 1 == n)) {
-            F.force_out = s->d_history + first + (k + 1 - F.n);
-            e = launch_pdl(sum_forces, dim3((F.n + 3) / 4), dim3(128), 0, s->stream, s->dev, F);
-            F.n = 0;
-        }
-        if (e != cudaSuccess) break;
+        if (e != cudaSuccess) return (int)e;
         s->cur ^= 1;
         ++s->steps_done;
         if (s->stream_off) s->U_stream += s->dev.dv;
-    }
-    if (e != cudaSuccess) return set_error(LBM_ECUDA, "step launch: %s", cudaGetErrorString(e));
+        return 0;
+    };
+    const auto sum = [&](int held) {
+        if (!defer) return 0;
+        F.n = held;
+        F.force_out = s->d_history + s->steps_done - held;
+        return (int)launch_pdl(sum_forces, dim3((held + 3) / 4), dim3(128), 0, s->stream, s->dev, F);
+    };
+    int lost = 0;
+    rc = run_deferred(n, kForceSteps, step, sum, &lost);
+    s->lost_forces += lost;
+    if (rc) return set_error(LBM_ECUDA, "step launch: %s", cudaGetErrorString((cudaError_t)rc));
     return LBM_OK;
 }
 
@@ -1298,6 +1302,8 @@ int lbm_force_history(lbm_sim* s, double* out_xy, size_t cap_steps, size_t* n_st
     if (n_steps) *n_steps = (size_t)s->steps_done;
     const size_t n = std::min(cap_steps, (size_t)s->steps_done);
     if (n && !out_xy) return set_error(LBM_EINVAL, "null output buffer");
+    if (s->lost_forces)
+        return set_error(LBM_ECUDA, "the forces of %d steps of a call that failed were not summed", s->lost_forces);
     if (n) CUDA_TRY(cudaMemcpy(out_xy, s->d_history, n * sizeof(double2), cudaMemcpyDeviceToHost));
     s->d2h_bytes += n * sizeof(double2);
     return rc;
