@@ -729,14 +729,19 @@ int use_variant(lbm_sim* s, int variant) {
     if (!fn || !variant_tile(variant, s->geom.storage, &bx, &by))
         return set_error(LBM_EINVAL, "variant %d is not built for this lattice/storage/collision", variant);
     tma_box(s->Q, s->geom.storage, bx, &bw, &pad);
-    for (int k = 0; k < 2; ++k) {
-        if ((rc = encode_map(&s->maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bw, by)))
-            return rc;
-        if ((rc = encode_map(&s->store_maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bx, by)))
-            return rc;
-    }
     // (32 leaves the boundary nodes to their own blocks; the others' tiles read their links)
     if (variant != 32 && (rc = ensure_links(s))) return rc;
+    // everything that can fail comes before the first change: a staged kernel with the boxes of another would wait
+    // for bytes that never come
+    CUtensorMap maps[2], store_maps[2];
+    for (int k = 0; k < 2; ++k) {
+        if ((rc = encode_map(&maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bw, by)))
+            return rc;
+        if ((rc = encode_map(&store_maps[k], s->buf[k], s->geom.storage, s->nx, s->ny, s->Q, s->pitch, bx, by)))
+            return rc;
+    }
+    std::copy_n(maps, 2, s->maps);
+    std::copy_n(store_maps, 2, s->store_maps);
     s->bx = bx;
     s->by = by;
     s->variant = variant;
