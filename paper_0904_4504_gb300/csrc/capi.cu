@@ -497,7 +497,7 @@ struct lbm_sim {
     lbm_geometry geom{};
     HostLattice lat{};
     size_t esize = 0;
-    std::vector<uint8_t> labels;       // LBM_GEOM_MASK: a copy; else filled when first asked for (labels_of)
+    std::vector<uint8_t> labels;       // LBM_GEOM_MASK: a copy; else kept by the first call that needs them (labels_of)
     std::vector<LinkNode> link_nodes;  // boundary nodes and their link masks
     size_t n_fluid = 0, n_boundary = 0;
     double fconst[2] = {0, 0}, fmov[2] = {0, 0};
@@ -576,11 +576,23 @@ void free_sim(lbm_sim* s) {
     delete s;
 }
 
-// The labels the simulation runs with.
+// The labels the simulation runs with: into a caller's buffer (which allocates nothing), and kept.
+void fill_labels(const lbm_sim* s, unsigned char* out) {
+    if (!s->labels.empty()) {
+        std::copy(s->labels.begin(), s->labels.end(), out);
+        return;
+    }
+    for (int y = 0; y < s->ny; ++y) {
+        unsigned char* row = out + (size_t)y * s->nx;
+        if (!label_row(s->lat, s->nx, s->ny, s->geom, y, row)) std::fill_n(row, s->nx, (unsigned char)0);
+    }
+}
+
 const std::vector<uint8_t>& labels_of(lbm_sim* s) {
     if (s->labels.empty()) {
-        s->labels.assign((size_t)s->nx * s->ny, 0);
-        for (int y = 0; y < s->ny; ++y) label_row(s->lat, s->nx, s->ny, s->geom, y, s->labels.data() + (size_t)y * s->nx);
+        std::vector<uint8_t> lab((size_t)s->nx * s->ny);
+        fill_labels(s, lab.data());
+        s->labels.swap(lab);
     }
     return s->labels;
 }
@@ -1437,9 +1449,9 @@ int lbm_set_state(lbm_sim* s, const double* g, size_t count) {
 int lbm_get_labels(lbm_sim* s, unsigned char* out, size_t count) {
     int rc = check_sim(s);
     if (rc) return rc;
-    const std::vector<uint8_t>& lab = labels_of(s);
-    if (!out || count != lab.size()) return set_error(LBM_ERANGE, "need %zu labels", lab.size());
-    std::memcpy(out, lab.data(), count);
+    const size_t N = (size_t)s->nx * s->ny;
+    if (!out || count != N) return set_error(LBM_ERANGE, "need %zu labels", N);
+    fill_labels(s, out);
     return LBM_OK;
 }
 
