@@ -1157,6 +1157,7 @@ int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const
     d.reg_a = (1.0 - 1.0 / tau) / (2.0 * H.theta * H.theta);
     d.reg_a2 = 2.0 * d.reg_a;
     d.src_k = (1.0 - 0.5 / tau) / H.theta;
+    d.src_t = d.src_k / d.omega_c;
     d.mw_k = 2.0 * g.rho0 / (H.theta * d.s);
     d.rho0_f = (float)d.rho0;
     d.s_f = (float)d.s;
@@ -1170,6 +1171,9 @@ int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const
     d.reg_f[2] = (float)cross;
     d.reg_f[3] = (float)(cross - (double)d.reg_f[2]);
     d.src_k_f = (float)d.src_k;
+    const double src_t = d.src_k / (double)d.omega_c_f;  // (the rounded 1/tau times it is the source)
+    d.src_t_f[0] = (float)src_t;
+    d.src_t_f[1] = (float)(src_t - (double)d.src_t_f[0]);
     s->stream_off = es == 2 && g.drive == LBM_DRIVE_BODYFORCE;
     d.stream_off = s->stream_off ? 1 : 0;
     // default kernel: the fastest measured single-instance form -- for D2Q37 the plain kernel with
@@ -1237,7 +1241,6 @@ int lbm_step(lbm_sim* s, long n) {
             // the drive of the next step, then that of this one
             set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done + 1));
             s->dev.dv2 = s->dev.dv;
-            s->dev.dv2_f = s->dev.dv_f;
             std::copy_n(s->dev.mw, 4, s->dev.mw2);
             std::copy_n(s->dev.mw_f, 4, s->dev.mw2_f);
             set_drive(s->dev, drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done));

@@ -110,6 +110,9 @@ template <>
 __device__ __forceinline__ double vadds<double>(double b, double k) { return __fma_rn(b, opaque(1.0), opaque(k)); }
 template <>
 __device__ __forceinline__ V2 vadds<V2>(V2 b, float k) { return V2{__fadd_rn(b.x, k), __fadd_rn(b.y, k)}; }
+// A launch constant in every lane, as an operand in registers.
+template <class V> __device__ __forceinline__ V vconst(typename Lane<V>::T k) { return vset<V>(k); }
+template <> __device__ __forceinline__ double vconst<double>(double k) { return opaque(k); }
 // The same for compile-time constants (after inlining): a factor of 1 or -1 is an add or a subtract.
 template <class V>
 __device__ __forceinline__ V vfmak(double k, V b, V c) {
@@ -262,7 +265,6 @@ struct Coef {
     V q40, q31, q22, q13, q04;      // fourth order; q31, q13 and q22 less their factors 4, 4 and 6
     V l10, l01;                     // odd part, first order
     V c30, c21, c12, c03;           // third order; c21 and c12 less their factor 3
-    V kf, kfu, kfx, kfy;            // plain BGK: the source, odd (c_x kf) and even (kfu, c_x^2 kfx, c_x c_y kfy)
 };
 
 // Coefficients from the moments (storage units, relative to the stream offset with 16-bit storage and
@@ -313,9 +315,18 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
             o1 = vmulk(1.0 / 6.0, rho);
         }
     }
-    // Guo-type source: even part kf (a c_x - u_x), odd part c_x times kf (plain BGK) or F/(2 theta)
-    const V kf = body ? vmuls<V>(kconst<T>(P.src_k, P.src_k_f), F) : vset<V>((T)0);
-    V rxx, rxy, ryy, hf;
+    // Guo-type source: even part kf (a c_x - u_x), odd part c_x times hf, kf (plain BGK) or F/(2 theta).  It goes
+    // into the coefficients; for plain BGK, whose outputs are h + (E + O - h) / tau, it is tau times the source.
+    // (Added to each output instead it took two operations a direction and the registers of its parts: 16
+    // instances of 256^2 D2Q37 FP64 788 us a step against 555, 12 of D2Q9 FP16 56.5 against 50.4.)
+    V kf = vset<V>((T)0);
+    if (body) {
+        if constexpr (COLL == COLL_REG) kf = vmuls<V>(kconst<T>(P.src_k, P.src_k_f), F);
+        else if constexpr (sizeof(T) == 8) kf = vmuls<V>(P.src_t, F);
+        else kf = vfmas<V>(P.src_t_f[1], F, vmuls<V>(P.src_t_f[0], F));
+    }
+    if (body && COLL == COLL_BGK) e0 = vfma(vneg(kf), ux, e0);
+    V rxx, rxy, ryy, hf = kf, kx = kf;
     if (COLL == COLL_REG) {
         // Eq. 19: Pi^ne = Pi - Pi^eq with Pi^eq = rho theta I + rho u u (exact on these lattices)
         constexpr double THP = sizeof(T) == 8 ? TH : pressure<L, T>();
@@ -343,11 +354,9 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         if (H4) { e2 = vmuls<V>(is, e2); o1 = vmuls<V>(is, o1); }
         if (COLL == COLL_REG) {
             rxx = vmuls<V>(is, rxx); rxy = vmuls<V>(is, rxy); ryy = vmuls<V>(is, ryy);
-            hf = vmuls<V>(is, hf);
         }
-        C.kf = vmuls<V>(is, kf);
-    } else {
-        C.kf = kf;
+        hf = vmuls<V>(is, hf);
+        kx = vmuls<V>(is, kf);
     }
     // monomials
     C.c0 = e0;
@@ -356,21 +365,15 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
         C.q20 = vfma(eX, X, rxx);
         C.q11 = vfma(eX2, Y, rxy);
         C.q02 = vfma(eY, Y, ryy);
-        C.l10 = BODY == 0 ? vmul(o0, X) : vfma(o0, X, hf);
-        if (body) {
-            C.q20 = vfma(C.kf, X, C.q20);
-            C.q11 = vfma(C.kf, Y, C.q11);
-        }
     } else {
         C.q20 = vmul(eX, X);
         C.q11 = vmul(eX2, Y);
         C.q02 = vmul(eY, Y);
-        C.l10 = vmul(o0, X);
-        if (BODY != 0) {
-            C.kfu = vmul(vneg(C.kf), ux);
-            C.kfx = vmul(C.kf, X);
-            C.kfy = vmul(C.kf, Y);
-        }
+    }
+    C.l10 = BODY == 0 ? vmul(o0, X) : vfma(o0, X, hf);
+    if (body) {
+        C.q20 = vfma(kx, X, C.q20);
+        C.q11 = vfma(kx, Y, C.q11);
     }
     C.l01 = vmul(o0, Y);
     if (H4) {
@@ -390,32 +393,20 @@ __device__ __forceinline__ Coef<V> coefficients(const InstDev& P, double dv, flo
     return C;
 }
 
-// The outputs of a node from its coefficients: emit(i, v) receives output i in storage units (relative
-// to the stream offset of the stored state when it is on: He and Ho of |c_x| leave the even and odd
-// parts).  Plain BGK reads the pulled populations h (absolute ones), the regularized collision does
-// not.
-template <class L, class ST, int COLL, class V, bool SOURCE, class H, class Emit>
+// The outputs of a node from its coefficients: emit(i, v) receives output i in storage units, relative to the
+// stream offset of the stored state when it is on (regularized: its even and odd parts He and Ho of |c_x| leave
+// the even and odd parts; plain BGK with OFFSET: off_s leaves the output).  Plain BGK reads the pulled populations h
+// (absolute ones), the regularized collision does not.
+template <class L, class ST, int COLL, class V, bool OFFSET, class H, class Emit>
 __device__ __forceinline__ void emit_outputs_s(const InstDev& P, const Coef<V>& C, H&& h, Emit&& emit) {
     using T = typename Lane<V>::T;
     constexpr int R = L::R;
     constexpr bool H4 = R == 3;
     constexpr bool SCALED = sizeof(ST) == 2, REG = COLL == COLL_REG;
-    const T om = kconst<T>(P.omega_c, P.omega_c_f);
-    constexpr bool source = !REG && SOURCE;
+    const V om = vconst<V>(kconst<T>(P.omega_c, P.omega_c_f));
     V EA[R + 1], EB[R + 1], OX[R + 1], OY[R + 1], U[R + 1];
-    V Sa[R + 1], So[R + 1];  // plain BGK: source parts per |c_x|, less the stored state's stream offset
 #pragma unroll
-    for (int m = 0; m <= R; ++m) {
-        EA[m] = REG && SCALED ? vadds(C.c0, -(T)P.He[m]) : C.c0;
-        if (!REG && source) {
-            Sa[m] = m ? vfmak((double)m * m, C.kfx, C.kfu) : C.kfu;
-            So[m] = m ? vmulk((double)m, C.kf) : vset<V>((T)0);
-            if (SCALED) {
-                Sa[m] = vadds(Sa[m], -(T)P.He[m]);
-                So[m] = vadds(So[m], -(T)P.Ho[m]);
-            }
-        }
-    }
+    for (int m = 0; m <= R; ++m) EA[m] = REG && SCALED ? vadds(C.c0, -(T)P.He[m]) : C.c0;
     // even axis parts of (m, .) and (., n); odd ones
 #pragma unroll
     for (int m = 1; m <= R; ++m) {
@@ -426,40 +417,31 @@ __device__ __forceinline__ void emit_outputs_s(const InstDev& P, const Coef<V>& 
         if (REG && SCALED) OX[m] = vadds(OX[m], -(T)P.Ho[m]);
         U[m] = H4 ? vfmak(4.0 * m2, C.q31, C.q11) : C.q11;
     }
-    auto out = [&](int i, V eq, int mx, V src_even, V src_odd, int sign) {
+    auto out = [&](int i, V eq) {
         if (REG) {
             emit(i, eq);
         } else {
-            // Eq. 14 discretized: f - (f - f^eq)/tau + source
+            // Eq. 14 discretized: f - (f - f^eq)/tau, with the source in f^eq
             const V hi = h(i);
-            V v = vfmas<V>(om, vsub(eq, hi), hi);
-            if (source) v = vadd(v, sign > 0 ? vadd(src_even, src_odd) : vsub(src_even, src_odd));
-            emit(i, v);
+            const V v = vfma(om, vsub(eq, hi), hi);
+            emit(i, OFFSET ? vadds(v, -(T)off_s<L>(P, i)) : v);
         }
     };
-    if (REG) {
-        emit(0, EA[0]);
-    } else {
-        const V h0 = h(0);
-        V v = vfmas<V>(om, vsub(C.c0, h0), h0);
-        if (source) v = vadd(v, Sa[0]);
-        emit(0, v);
-    }
+    out(0, EA[0]);
     const V rest = EA[0];
 #pragma unroll
     for (int m = 1; m <= R; ++m) EA[m] = vfmak((double)m * m, H4 ? vfmak((double)m * m, C.q40, C.q20) : C.q20, EA[m]);
-    const V none = vset<V>((T)0);
 #pragma unroll
     for (int k = 0; k < L::NP; k += 2) {
         const int m = L::px(k), n = L::py(k);
         const int i = 1 + 2 * k;  // +p_k, -p_k, +p_(k+1), -p_(k+1)
         if (n == 0) {
-            out(i, vadd(EA[m], OX[m]), m, Sa[m], So[m], 1);
-            out(i + 1, vsub(EA[m], OX[m]), m, Sa[m], So[m], -1);
+            out(i, vadd(EA[m], OX[m]));
+            out(i + 1, vsub(EA[m], OX[m]));
             const V E = vadd(rest, EB[m]);
             // (0, m): c_x = 0, so the odd part holds no offset (Ho[0] = 0)
-            out(i + 2, vadd(E, OY[m]), 0, Sa[0], none, 1);
-            out(i + 3, vsub(E, OY[m]), 0, Sa[0], none, -1);
+            out(i + 2, vadd(E, OY[m]));
+            out(i + 3, vsub(E, OY[m]));
         } else {
             const double mn = (double)m * n, m2 = (double)m * m, n2 = (double)n * n;
             V S = vadd(EA[m], EB[n]);
@@ -469,30 +451,24 @@ __device__ __forceinline__ void emit_outputs_s(const InstDev& P, const Coef<V>& 
             const V ox = H4 ? vfmak(3.0 * m * n2, C.c12, OX[m]) : OX[m];
             const V oy = H4 ? vfmak(3.0 * n * m2, C.c21, OY[n]) : OY[n];
             const V Op = vadd(ox, oy), Om = vsub(ox, oy);
-            V sp = none, sm = none;
-            if (!REG && source) {
-                sp = vfmak(mn, C.kfy, Sa[m]);
-                sm = vfmak(-mn, C.kfy, Sa[m]);
-            }
-            out(i, vadd(Ep, Op), m, sp, So[m], 1);
-            out(i + 1, vsub(Ep, Op), m, sp, So[m], -1);
-            out(i + 2, vadd(Em, Om), m, sm, So[m], 1);
-            out(i + 3, vsub(Em, Om), m, sm, So[m], -1);
+            out(i, vadd(Ep, Op));
+            out(i + 1, vsub(Ep, Op));
+            out(i + 2, vadd(Em, Om));
+            out(i + 3, vsub(Em, Om));
         }
     }
 }
 
-// The same; plain BGK adds its source where the launch has one (a branch, not predicated operations).
-template <class L, class ST, int COLL, class V, int BODY = -1, class H, class Emit>
+// The same; plain BGK takes its offset out where the launch has one (a branch, not predicated operations).
+template <class L, class ST, int COLL, class V, class H, class Emit>
 __device__ __forceinline__ void emit_outputs(const InstDev& P, const Coef<V>& C, H&& h, Emit&& emit) {
-    if constexpr (COLL == COLL_REG || BODY == 0)
-        emit_outputs_s<L, ST, COLL, V, false>(P, C, h, emit);
-    else if constexpr (BODY == 1)
-        emit_outputs_s<L, ST, COLL, V, true>(P, C, h, emit);
-    else if (P.body_force || (sizeof(ST) == 2 && P.stream_off))
-        emit_outputs_s<L, ST, COLL, V, true>(P, C, h, emit);
-    else
-        emit_outputs_s<L, ST, COLL, V, false>(P, C, h, emit);
+    if constexpr (COLL == COLL_BGK && sizeof(ST) == 2) {
+        if (P.stream_off) {
+            emit_outputs_s<L, ST, COLL, V, true>(P, C, h, emit);
+            return;
+        }
+    }
+    emit_outputs_s<L, ST, COLL, V, false>(P, C, h, emit);
 }
 
 }  // namespace lbm

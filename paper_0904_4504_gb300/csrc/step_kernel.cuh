@@ -204,10 +204,8 @@ __device__ __forceinline__ void collide_emit(const InstDev& P, double dv, float 
     const auto at = [&](int i) { return h[i]; };
     const Moments<V> M = moments<L, V>(at);
     if constexpr (sizeof(ST) == 8) {
-        if (P.body_force)
-            emit_outputs<L, ST, COLL, V, 1>(P, coefficients<L, ST, COLL, V, 1>(P, dv, dv_f, M), at, emit);
-        else
-            emit_outputs<L, ST, COLL, V, 0>(P, coefficients<L, ST, COLL, V, 0>(P, dv, dv_f, M), at, emit);
+        const Coef<V> C = P.body_force ? coefficients<L, ST, COLL, V, 1>(P, dv, dv_f, M) : coefficients<L, ST, COLL, V, 0>(P, dv, dv_f, M);
+        emit_outputs<L, ST, COLL, V>(P, C, at, emit);
     } else {
         emit_outputs<L, ST, COLL, V>(P, coefficients<L, ST, COLL, V>(P, dv, dv_f, M), at, emit);
     }
@@ -466,11 +464,11 @@ inline dim3 edge_grid(const InstDev& P, int threads) {
 // Node (x, y) inside the grid, of class cls (already loaded), in a bulk block.  With 4- and 8-byte
 // storage its pulls are issued whatever the class (the pulls of any node inside the grid are in bounds,
 // so they need not wait for the class test), then a bulk node collides and stores; the others load for
-// nothing, a small fraction of a grid.  The 16-bit kernels run at a register budget where that spills,
-// so they test the class first.
+// nothing, a small fraction of a grid.  The 16-bit kernels, and plain BGK in FP32, run at a register budget
+// where that spills, so they test the class first.
 template <class L, class ST, int COLL>
 __device__ __forceinline__ void bulk_node(const InstDev& P, int x, int y, int cls) {
-    if (sizeof(ST) == 2 && cls != NODE_BULK) return;
+    if ((sizeof(ST) == 2 || (sizeof(ST) == 4 && L::Q == 37 && COLL == COLL_BGK)) && cls != NODE_BULK) return;
     typename StoreT<ST>::CT h[L::Q];
     gather_global<L, ST>(P, static_cast<const ST*>(P.src), x, y, h);
     if (cls != NODE_BULK) return;

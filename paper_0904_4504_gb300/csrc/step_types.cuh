@@ -66,11 +66,12 @@ struct InstDev {
     double s, inv_s;             // storage scale
     double omega_c;              // 1/tau
     double reg_a, reg_a2;        // (1 - 1/tau) / (2 theta^2), and twice that
-    double src_k;                // (1 - 1/(2 tau)) / theta
+    double src_k, src_t;         // (1 - 1/(2 tau)) / theta, and tau times that
     double mw_k;                 // 2 rho0 / (theta s): moving-wall term per unit c_i.U_w
     // FP32 copies of the constants above (and of dv), so that FP32 arithmetic converts nothing per
     // node: double -> float conversions run on the FP64 pipe, which is slow on this GPU
-    float dv_f, rho0_f, s_f, inv_s_f, omega_c_f, reg_pad, src_k_f, dv2_f;
+    float dv_f, rho0_f, s_f, inv_s_f, omega_c_f, src_k_f;
+    float src_t_f[2];            // src_k over omega_c_f, as the sum of two floats (collision.cuh)
     // FP32 regularization factors of P_xx, P_yy and of P_xy, each as the sum of two floats (collision.cuh)
     float reg_f[4];
     // 16-bit body-frame runs store h_i - H_i(n), with H_i(n) the (scaled) equilibrium deviation of
