@@ -422,12 +422,13 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         rc = b->pvariant ? lbm_set_variant(sim, b->pvariant) : lbm_set_tile(sim, 32, 4);
         if (rc == LBM_OK) rc = sim_tile_links(sim);
     } else {
-        // default kernels, fastest measured in this mode: for D2Q37 with 16-bit storage the staged
-        // kernel with two nodes per thread (32; plain BGK: the staged one with three rows per thread,
-        // 27), with FP32 the plain kernel with 7 resident blocks per SM (2); 16-bit D2Q9 takes the
-        // four-nodes-per-thread kernel (30); else the plain kernel
+        // default kernels, fastest measured in this mode: for D2Q37 with 16-bit storage that of the grid's sides
+        // (pair_variant; plain BGK: the staged one with three rows per thread, 27), with FP32 the plain kernel with
+        // 7 resident blocks per SM (2); D2Q9 with FP32 or 16-bit storage takes several nodes per thread (30); else
+        // the plain kernel
+        const bool pairs = b->Q == 37 && b->collision == LBM_COLL_REGULARIZED;
         const int want = b->variant >= 0 ? b->variant
-                         : half ? (b->Q != 37 ? 30 : b->collision == LBM_COLL_REGULARIZED ? 32 : 27)
+                         : half ? (b->Q != 37 ? 30 : pairs ? pair_variant(d->nx, d->ny, 0, true) : 27)
                          : b->storage == LBM_STORE_F32 ? (b->Q == 37 ? 2 : 30) : 0;
         if (want == 0 || lbm_set_variant(sim, want) != LBM_OK) rc = lbm_set_tile(sim, b->bx, b->by);
     }

@@ -1176,19 +1176,18 @@ int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const
     d.src_t_f[1] = (float)(src_t - (double)d.src_t_f[0]);
     s->stream_off = es == 2 && g.drive == LBM_DRIVE_BODYFORCE;
     d.stream_off = s->stream_off ? 1 : 0;
-    // default kernel: the fastest measured single-instance form -- for D2Q37 the plain kernel with
-    // an occupancy floor on the default 32 x 4 tile (variant 1 for FP32, 2 for 16-bit storage), for
-    // the regularized collision of 16-bit storage two nodes per thread (31; 32, staged, where the two
-    // buffers hold over 200 MB; step_q37v.cuh has the measurements), for FP32 and 16-bit D2Q9 several
-    // nodes per thread (30) but on small grids, where fewer nodes per thread mean more warps (FP32: 2048^2
-    // 44.7 us against 55.4, 1024^2 9.6 / 12.0, 512^2 3.9 / 3.7, 128^2 2.2 / 1.8; FP16: 512^2 4.1 / 4.2, 128^2
-    // 3.1 / 1.8)
+    // default kernel: the fastest measured single-instance form -- for D2Q37 the plain kernel with an occupancy
+    // floor on the default 32 x 4 tile (variant 1 for FP32, 2 for plain BGK with 16-bit storage), for the
+    // regularized collision of 16-bit storage two nodes per thread where that pays (pair_variant); for FP32 and 16-bit
+    // D2Q9 several nodes per thread (30) but on small grids, where fewer nodes per thread mean more warps (us a
+    // step, 30 / 0; FP32: 2048^2 43.5 / 55.4, 1024^2 9.1 / 11.8, 512^2 3.6 / 3.7, 430^2 3.5 / 2.8, 128^2 2.1 / 1.9;
+    // FP16: 1024^2 7.5 / 13.3, 512^2 3.6 / 4.3, 430^2 3.5 / 3.6, 362^2 3.2 / 2.7, 128^2 2.9 / 2.2)
     if (!s->aa && g.wall_scheme == LBM_SCHEME_BOUNCEBACK) {
         int v = 0;
         if (lattice == LBM_D2Q9) v = es <= 4 && (size_t)nx * ny > ((size_t)1 << (es == 4 ? 18 : 17)) ? 30 : 0;
         else if (es == 4) v = 1;
         else if (es == 2)
-            v = g.collision != LBM_COLL_REGULARIZED || nx < 48 ? 2 : 2 * plane * H.Q * es > (size_t)200000000 ? 32 : 31;
+            v = g.collision != LBM_COLL_REGULARIZED ? 2 : pair_variant(nx, ny, 2 * plane * H.Q * es, false);
         if (v) TRY_OR_FREE(use_variant(s, v));
     }
     TRY_OR_FREE(setup_tiles(s));

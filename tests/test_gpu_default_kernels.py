@@ -1,0 +1,43 @@
+"""The kernel that lbm_create and a batch choose by themselves for regularized D2Q37 with 16-bit storage, around
+the lines of the rule: few columns that would leave half a block idle, small grids, and where staging pays."""
+import pytest
+
+from paper_0904_4504_gb300 import lbm as L
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+
+def _kw(storage, collision):
+    return dict(kind=L.LBM_GEOM_NONE, u0=1e-3, eq_order=4, storage=storage, collision=collision)
+
+
+@pytest.mark.parametrize("storage", [L.LBM_STORE_F16, L.LBM_STORE_BF16], ids=["f16", "bf16"])
+@pytest.mark.parametrize("nx,ny,alone,batch", [
+    (24, 24, 2, 2), (32, 9000, 2, 2), (33, 9000, 31, 31), (64, 64, 2, 31), (65, 4000, 2, 2), (96, 4000, 2, 2),
+    (97, 4000, 31, 31), (160, 2000, 2, 2), (161, 2000, 31, 31), (447, 367, 31, 31), (448, 365, 2, 32), (448, 366, 31, 32),
+    (512, 320, 2, 32), (512, 321, 31, 32), (639, 2200, 31, 32), (640, 2200, 32, 32), (1024, 1024, 31, 32)])
+def test_pairs_by_the_grids_sides(nx, ny, alone, batch, storage):
+    kw = _kw(storage, L.LBM_COLL_REGULARIZED)
+    sim = L.lbm_create(37, nx, ny, 0.8, 0.05, L.make_geometry(**kw))
+    try:
+        assert L.lbm_info(sim)["variant"] == alone
+    finally:
+        L.lbm_destroy(sim)
+    b = L.lbm_batch_create(37, storage, L.LBM_COLL_REGULARIZED)
+    try:
+        inst = L.lbm_batch_instance(b, L.lbm_batch_add(b, L.make_instance(37, nx, ny, 0.8, 0.05, 4, **kw)))
+        assert L.lbm_info(inst)["variant"] == batch
+    finally:
+        L.lbm_batch_destroy(b)
+
+
+def test_plain_bgk_keeps_one_node_per_thread():
+    sim = L.lbm_create(37, 1024, 1024, 0.8, 0.05, L.make_geometry(**_kw(L.LBM_STORE_F16, L.LBM_COLL_BGK)))
+    try:
+        assert L.lbm_info(sim)["variant"] == 2
+    finally:
+        L.lbm_destroy(sim)

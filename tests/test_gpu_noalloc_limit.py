@@ -20,10 +20,10 @@ def _sim(Q, nx, ny, lx, ly, storage):
     return L.lbm_create(Q, nx, ny, 0.8, 0.05, geom)
 
 
-# 2064, 3088 and about 8000 tiles of 32 x 4 nodes hold body links (of the pairs' own 64 x 1: 8212)
+# 2064, 2064 and about 8000 tiles of 32 x 4 nodes hold body links (of the pairs' own 64 x 1: 8212)
 @pytest.mark.parametrize("Q,nx,ny,lx,ly,storage,variant", [
     (37, 128, 4200, 70, 4100, L.LBM_STORE_F16, 31),
-    (37, 330, 4200, 70, 4100, L.LBM_STORE_F16, 32),
+    (37, 640, 4200, 70, 4100, L.LBM_STORE_F16, 32),
     (9, 100, 17000, 70, 16000, L.LBM_STORE_F32, 30)], ids=["pairs", "staged-pairs", "q9"])
 def test_tall_bodies_on_the_default_kernels(Q, nx, ny, lx, ly, storage, variant):
     sim, plain = _sim(Q, nx, ny, lx, ly, storage), _sim(Q, nx, ny, lx, ly, storage)
