@@ -191,7 +191,7 @@ int lbm_set_tile(lbm_sim* sim, int block_x, int block_y);
  * two-buffer bounce-back runs on the fastest single-instance kernel measured: D2Q37 on 1 (FP32); 31 (16-bit,
  * regularized, above 163840 nodes), or 32 where the two buffers exceed 200 MB and the rows 639 nodes; 2 (16-bit
  * else: plain BGK, smaller grids, and rows of 1-32, 65-96 or 129-160 nodes); D2Q9 above 2^18 nodes (FP32) or
- * 2^17 (16-bit) on 30; else 0.
+ * 2^17 (16-bit), on rows of more than 32 nodes, on 30; else 0.
  * lbm_set_tile selects variant 0.
  * Staged kernels (FP32/BF16/FP16 storage), whose interior tiles are copied to shared memory by
  * bulk tensor copies (TMA), one box per direction plane:
@@ -334,7 +334,8 @@ int lbm_batch_set_mode(lbm_batch* batch, int mode);
 
 /* Step kernel of the instances added after this call, in the streams mode (lbm_set_variant
  * numbers; -1, the default: for D2Q37 with 16-bit storage variant 32, on rows shorter than 448 nodes 31 (2 for
- * 1-32, 65-96 or 129-160 nodes), for plain BGK 27, and with FP32 variant 2; for D2Q9 with FP32 or 16-bit storage variant 30; else the plain kernel on 32 x 4 tiles).  An
+ * 1-32, 65-96 or 129-160 nodes), for plain BGK 27, and with FP32 variant 2; for D2Q9 with FP32 or 16-bit storage, on rows of more than 32 nodes,
+ * variant 30; else the plain kernel on 32 x 4 tiles).  An
  * instance whose layout or wall scheme the variant does not support falls back to the plain
  * kernel.  In the persistent mode (before the first lbm_batch_add) it picks the tile code the
  * persistent kernel runs: 27 staged 64 x 3 tiles, 28 staged 128 x 3 (D2Q37), 31 plain 64 x 8, two

@@ -424,12 +424,14 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
     } else {
         // default kernels, fastest measured in this mode: for D2Q37 with 16-bit storage that of the grid's sides
         // (pair_variant; plain BGK: the staged one with three rows per thread, 27), with FP32 the plain kernel with
-        // 7 resident blocks per SM (2); D2Q9 with FP32 or 16-bit storage takes several nodes per thread (30); else
-        // the plain kernel
+        // 7 resident blocks per SM (2); D2Q9 with FP32 or 16-bit storage takes several nodes per thread (30) on rows
+        // of more than 32 nodes (16 of 24 x 8000 FP32 30 / 0: 70 / 59 us a step, 80 x 4000 80 / 83); else the plain
+        // kernel
         const bool pairs = b->Q == 37 && b->collision == LBM_COLL_REGULARIZED;
+        const int q9 = d->nx > 32 ? 30 : 0;
         const int want = b->variant >= 0 ? b->variant
-                         : half ? (b->Q != 37 ? 30 : pairs ? pair_variant(d->nx, d->ny, 0, true) : 27)
-                         : b->storage == LBM_STORE_F32 ? (b->Q == 37 ? 2 : 30) : 0;
+                         : half ? (b->Q != 37 ? q9 : pairs ? pair_variant(d->nx, d->ny, 0, true) : 27)
+                         : b->storage == LBM_STORE_F32 ? (b->Q == 37 ? 2 : q9) : 0;
         if (want == 0 || lbm_set_variant(sim, want) != LBM_OK) rc = lbm_set_tile(sim, b->bx, b->by);
     }
     if (rc) return undo(rc);

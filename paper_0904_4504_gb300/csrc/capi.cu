@@ -1181,10 +1181,11 @@ int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const
     // regularized collision of 16-bit storage two nodes per thread where that pays (pair_variant); for FP32 and 16-bit
     // D2Q9 several nodes per thread (30) but on small grids, where fewer nodes per thread mean more warps (us a
     // step, 30 / 0; FP32: 2048^2 43.5 / 55.4, 1024^2 9.1 / 11.8, 512^2 3.6 / 3.7, 430^2 3.5 / 2.8, 128^2 2.1 / 1.9;
-    // FP16: 1024^2 7.5 / 13.3, 512^2 3.6 / 4.3, 430^2 3.5 / 3.6, 362^2 3.2 / 2.7, 128^2 2.9 / 2.2)
+    // FP16: 1024^2 7.5 / 13.3, 512^2 3.6 / 4.3, 430^2 3.5 / 3.6, 362^2 3.2 / 2.7, 128^2 2.9 / 2.2) and on rows of
+    // half a tile or less (24 x 60000 FP32 29.1 / 22.7, FP16 47 / 26)
     if (!s->aa && g.wall_scheme == LBM_SCHEME_BOUNCEBACK) {
         int v = 0;
-        if (lattice == LBM_D2Q9) v = es <= 4 && (size_t)nx * ny > ((size_t)1 << (es == 4 ? 18 : 17)) ? 30 : 0;
+        if (lattice == LBM_D2Q9) v = es <= 4 && nx > 32 && (size_t)nx * ny > ((size_t)1 << (es == 4 ? 18 : 17)) ? 30 : 0;
         else if (es == 4) v = 1;
         else if (es == 2)
             v = g.collision != LBM_COLL_REGULARIZED ? 2 : pair_variant(nx, ny, 2 * plane * H.Q * es, false);

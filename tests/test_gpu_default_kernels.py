@@ -1,5 +1,6 @@
-"""The kernel that lbm_create and a batch choose by themselves for regularized D2Q37 with 16-bit storage, around
-the lines of the rule: few columns that would leave half a block idle, small grids, and where staging pays."""
+"""The kernel that lbm_create and a batch choose by themselves, around the lines of the rules.  Regularized D2Q37
+with 16-bit storage: few columns that would leave half a block idle, small grids, and where staging pays; D2Q9:
+narrow and small grids."""
 import pytest
 
 from paper_0904_4504_gb300 import lbm as L
@@ -40,4 +41,21 @@ def test_plain_bgk_keeps_one_node_per_thread():
     try:
         assert L.lbm_info(sim)["variant"] == 2
     finally:
+        L.lbm_destroy(sim)
+
+
+@pytest.mark.parametrize("storage,nx,ny,alone,batch", [
+    (L.LBM_STORE_F32, 32, 9000, 0, 0), (L.LBM_STORE_F32, 33, 9000, 30, 30), (L.LBM_STORE_F32, 512, 512, 0, 30),
+    (L.LBM_STORE_F32, 512, 513, 30, 30), (L.LBM_STORE_F16, 24, 9000, 0, 0), (L.LBM_STORE_F16, 256, 512, 0, 30),
+    (L.LBM_STORE_F16, 256, 513, 30, 30), (L.LBM_STORE_F64, 1024, 512, 0, 0)])
+def test_d2q9(storage, nx, ny, alone, batch):
+    kw = dict(kind=L.LBM_GEOM_NONE, u0=1e-3, storage=storage)
+    sim = L.lbm_create(9, nx, ny, 0.8, 0.05, L.make_geometry(**kw))
+    b = L.lbm_batch_create(9, storage, L.LBM_COLL_REGULARIZED)
+    try:
+        assert L.lbm_info(sim)["variant"] == alone
+        inst = L.lbm_batch_instance(b, L.lbm_batch_add(b, L.make_instance(9, nx, ny, 0.8, 0.05, 4, **kw)))
+        assert L.lbm_info(inst)["variant"] == batch
+    finally:
+        L.lbm_batch_destroy(b)
         L.lbm_destroy(sim)
