@@ -333,8 +333,9 @@ int lbm_batch_remove(lbm_batch* batch, int slot);
 int lbm_batch_set_mode(lbm_batch* batch, int mode);
 
 /* Step kernel of the instances added after this call, in the streams mode (lbm_set_variant
- * numbers; -1, the default: for D2Q37 with 16-bit storage variant 32, on rows shorter than 448 nodes 31 (2 for
- * 1-32, 65-96 or 129-160 nodes), for plain BGK 27, and with FP32 variant 2; for D2Q9 with FP32 or 16-bit storage, on rows of more than 32 nodes,
+ * numbers; -1, the default: for D2Q37 with 16-bit storage variant 32, on grids of fewer than 448 columns and
+ * at least twice as many rows 31 (2 for 1-32, 65-96 or 129-160 columns), for plain BGK 27, and with FP32 variant 2;
+ * for D2Q9 with FP32 or 16-bit storage, on rows of more than 32 nodes,
  * variant 30; else the plain kernel on 32 x 4 tiles).  An
  * instance whose layout or wall scheme the variant does not support falls back to the plain
  * kernel.  In the persistent mode (before the first lbm_batch_add) it picks the tile code the
