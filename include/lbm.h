@@ -483,13 +483,13 @@ void lbm_server_destroy(lbm_server* server);
  * before it runs.
  *
  * Scratch: the kernel's force partials live in one static device array of the library
- * (LBM_NOALLOC_MAX_SLOTS * 256 + 256 bytes), held by every GPU that loads the library until the process
+ * (LBM_NOALLOC_MAX_SLOTS * 256 + 8448 bytes), held by every GPU that loads the library until the process
  * exits.  A geometry with more than LBM_NOALLOC_MAX_SLOTS tiles holding body links is rejected with
  * LBM_ERANGE (a larger tile, lbm_set_tile, needs fewer; the variants 30 with FP32, 31 and 32 count tiles of
  * 32 x 4 nodes).  All calls in the process share that array: calls whose work overlaps on the GPU (two streams, or two host threads) race and give wrong forces;
  * serialize them.  Nothing is carried from one call to the next, so a call that never completed, or that
  * overlapped another, does not affect the calls after it.  While the stream is being captured, a clear of one
- * word of the scratch is recorded before the step.
+ * word of the scratch is recorded before the step; otherwise one call in 1024 enqueues such a clear.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress) with
  * that device current; make that first call before any stream capture (a lookup that fails is
  * not remembered: the next call tries again).

@@ -11,11 +11,12 @@
 // until the process exits.
 //
 // The kernel is the simulation's own step kernel, where it reads the populations directly and the
-// caller's buffers are aligned for it, else the plain one.  The force groups of a call count themselves in one
-// word under the call's number (take_ticket): whatever earlier calls have left there, completed or not, alone or
-// overlapping, the call starts from zero, and no launch is needed before the step (a clear took 4 x 256 D2Q9 FP64
-// from 6.9 to 9 us).  A call recorded into a graph keeps its number, so there a clear of the word is recorded
-// before the step.
+// caller's buffers are aligned for it, else the plain one.  The last force group of a call is found by a ticket
+// that starts at zero and that it leaves at zero; one that a call left otherwise (it never completed, or overlapped
+// another) must not be met again.  So every call takes the next of two halves of tickets, and a half is cleared
+// as a whole before its first ticket is taken again: a call is one launch, but one call in kHalf (a clear before each
+// took 4 x 256 D2Q9 FP64 from 6.8 to 9.2 us, numbered counts in one 64-bit word cost small grids 3 to 6 %).  A call
+// recorded into a graph keeps its ticket for good, so there it is one of its own, and its clear is recorded too.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -26,19 +27,20 @@
 
 namespace {
 
-// Scratch: the group partials of the force (16 B each), then the non-finite flag and the ticket.  With bounce-back walls a
-// step has at most kMaxForceGroups groups; with diffuse walls one per 32 nodes with body links, and a
-// geometry is accepted with up to LBM_NOALLOC_MAX_SLOTS tiles holding such nodes, 512 in a tile at most.
-// Shared by every call in the process on a given device.
+// Scratch: the group partials of the force (16 B each), then the non-finite flag, the ticket of recorded calls and
+// the tickets of the others.  With bounce-back walls a step has at most kMaxForceGroups groups; with diffuse walls
+// one per 32 nodes with body links, and a geometry is accepted with up to LBM_NOALLOC_MAX_SLOTS tiles holding such
+// nodes, 512 in a tile at most.  Shared by every call in the process on a given device.
 constexpr size_t kPartialBytes = (size_t)LBM_NOALLOC_MAX_SLOTS * 16 * sizeof(double2);
-constexpr size_t kScratchBytes = kPartialBytes + 256;  // flag at 0, ticket at 128
-static_assert((size_t)LBM_NOALLOC_MAX_SLOTS * 16 < (1u << lbm::kTicketBits), "a call's groups fit the ticket's count");
+constexpr unsigned kHalf = 1024;
+constexpr size_t kTickets = kPartialBytes + 256;       // flag at kPartialBytes, recorded calls' ticket 128 above it
+constexpr size_t kScratchBytes = kTickets + 2 * kHalf * sizeof(unsigned);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_addr_mutex;
-std::mutex g_call_mutex;           // a call's number and its launch: the order of a stream is that of the numbers
-unsigned long long g_calls = 0;
+std::mutex g_call_mutex;           // a call's ticket, the clear before it and its launch
+unsigned g_calls[kMaxDevices] = {};
 void* g_addr[kMaxDevices] = {};  // null until a lookup on that device has succeeded
 
 // Device address of the scratch array on `device` (looked up with that device current; the name
@@ -101,7 +103,6 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     P.src = g_in;
     P.dst = g_out;
     P.partials = reinterpret_cast<double2*>(b);
-    P.ticket = reinterpret_cast<unsigned int*>(b + kPartialBytes + 128);
     P.err = reinterpret_cast<int*>(b + kPartialBytes);
     P.force_out = reinterpret_cast<double2*>(force_out);
     P.ngroups = v.nlf;
@@ -111,13 +112,20 @@ extern "C" int lbm_step_noalloc(const lbm_sim* sim, long n, const void* g_in, vo
     for (int m = 0; m < 4; ++m) P.He[m] = P.Ho[m] = 0.f;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(st, &capture);
-    if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone)
-        e = cudaMemsetAsync(P.ticket, 0, sizeof(unsigned long long), st);
+    cudaError_t e = cudaSuccess;
+    // (the legacy default stream cannot be captured; the question costs a tenth of a short call)
+    if (st != nullptr && st != cudaStreamLegacy) e = cudaStreamIsCapturing(st, &capture);
     if (e == cudaSuccess) {
         std::lock_guard<std::mutex> lock(g_call_mutex);
-        P.call = ++g_calls;
-        e = fn(P, dim3(v.bx, v.by), st);
+        if (capture != cudaStreamCaptureStatusNone) {
+            P.ticket = reinterpret_cast<unsigned int*>(b + kPartialBytes + 128);
+            if (P.ngroups > 0) e = cudaMemsetAsync(P.ticket, 0, sizeof(unsigned), st);
+        } else if (P.ngroups > 0) {
+            const unsigned at = g_calls[v.device]++ % (2 * kHalf);
+            P.ticket = reinterpret_cast<unsigned int*>(b + kTickets) + at;
+            if (at % kHalf == 0) e = cudaMemsetAsync(P.ticket, 0, kHalf * sizeof(unsigned), st);
+        }
+        if (e == cudaSuccess) e = fn(P, dim3(v.bx, v.by), st);
     }
     if (e == cudaSuccess && P.ngroups == 0) e = cudaMemsetAsync(force_out, 0, 2 * sizeof(double), st);
     if (cur != v.device) cudaSetDevice(cur);

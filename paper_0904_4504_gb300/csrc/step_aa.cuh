@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(512) step_kernel_aa(const __grid_constant__ In
         if (lane >= 32) return;
         double2 F[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
         if (k < P.nb) aa_pull_push<L, ST, COLL, true>(P, A, at.x, at.y, lk, F);
-        if ((int)blockIdx.x < P.ngroups) group_force<2, false>(P, blockIdx.x, P.force_out, F, 1.0, lane);
+        if ((int)blockIdx.x < P.ngroups) group_force<2>(P, blockIdx.x, P.force_out, F, 1.0, lane);
         return;
     }
     const int tile = P.flip ? P.ntiles - 1 - (int)(blockIdx.x - nbb) : blockIdx.x - nbb;

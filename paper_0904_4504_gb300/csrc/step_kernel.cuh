@@ -308,22 +308,9 @@ static __global__ void __launch_bounds__(128) sum_forces(const __grid_constant__
         force_sum(P, P.partials + (size_t)k * P.ngroups, 1, F.dv[k], F.force_out + k, F.scale, threadIdx.x & 31);
 }
 
-// One lane: how many groups of the step have taken a ticket before this one.  Where calls share the ticket
-// (P.call, their increasing numbers) it holds the number of the newest call above kTicketBits bits of count: the
-// first group of a call raises it to the call's own, whatever an earlier call has left there.
-constexpr int kTicketBits = 20;
-template <bool CALLS>
-__device__ __forceinline__ unsigned long long take_ticket(const InstDev& P) {
-    if (!CALLS || !P.call) return atomicAdd(P.ticket, 1u);
-    unsigned long long* word = reinterpret_cast<unsigned long long*>(P.ticket);
-    const unsigned long long first = P.call << kTicketBits;
-    atomicMax(word, first);
-    return atomicAdd(word, 1ull) - first;
-}
-
 // One warp, force group g: the lanes' parts F into the group's partial; the last group of the step to
-// finish sums them all (and returns true).  CALLS: whether lbm_step_noalloc's calls run this code (take_ticket).
-template <int NF, bool CALLS>
+// finish sums them all (and returns true).
+template <int NF>
 __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* force_out, const double2 (&F)[NF],
                                             double scale, int lane) {
 #pragma unroll
@@ -334,14 +321,14 @@ __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* fo
     if (!P.ticket) return false;  // summed for several steps at once (sum_forces)
     __threadfence();
     __syncwarp();
-    bool last = false;
-    if (lane == 0) last = take_ticket<CALLS>(P) == (unsigned long long)(P.ngroups - 1);
-    last = __shfl_sync(0xffffffffu, last, 0);
+    unsigned t = 0;
+    if (lane == 0) t = atomicAdd(P.ticket, 1u);
+    const bool last = __shfl_sync(0xffffffffu, t, 0) == (unsigned)(P.ngroups - 1);
     if (last) {
         __threadfence();
 #pragma unroll
         for (int f = 0; f < NF; ++f) force_sum(P, P.partials + f, NF, f == 0 ? P.dv : P.dv2, force_out + f, scale, lane);
-        if (lane == 0 && (!CALLS || !P.call)) *P.ticket = 0u;
+        if (lane == 0) *P.ticket = 0u;
     }
     return last;
 }
@@ -351,7 +338,7 @@ __device__ __forceinline__ bool group_force(const InstDev& P, int g, double2* fo
 // FP64 multiply-adds a link.  FP64 is slow here (an instruction holds its sub-partition's unit for 64
 // cycles whatever its active lanes), so a warp takes 32 links at a time, whoever their nodes are, and
 // the factors and the moving-wall term (geometry only) come in once per step.  `wait` runs between the
-// loads of the list and those of the populations.  Lanes past the end of the list read the last link's
+// loads of the list and those of the populations.  Lanes past the end of the list read the group's first
 // population with a weight of 0, never a place that is no body link's: solid nodes are not written and may hold
 // NaN or infinities, which that weight would not keep out of the sum.
 template <class L, class ST, bool COH = false, class Wait>
@@ -371,7 +358,7 @@ __device__ __forceinline__ bool link_force(const InstDev& P, const void* src_v, 
         for (int j = 0; j < 4; ++j) {
             const long long k = first + 32ll * (j0 + j);
             const bool has = j0 + j < P.glen && k < P.nfl;
-            e[j] = list[has ? k : P.nfl - 1];
+            e[j] = list[has ? k : (long long)g * 32 * P.glen];
             cw[j] = has ? weights[e[j].y & 0xffu] : make_double2(0.0, 0.0);
         }
         if (j0 == 0) wait();
@@ -386,7 +373,7 @@ __device__ __forceinline__ bool link_force(const InstDev& P, const void* src_v, 
             F[0].y = __fma_rn(cw[j].y, (double)own[j], F[0].y);
         }
     }
-    return group_force<1, !COH>(P, g, force_out, F, -2.0 * P.s, lane);
+    return group_force<1>(P, g, force_out, F, -2.0 * P.s, lane);
 }
 
 // Blocks of `threads` that hold the force groups, and the f-th of them.
@@ -438,7 +425,7 @@ __device__ __forceinline__ void boundary_block(const InstDev& P, int b) {
     if (WALL) F[0] = ds_apply<L, ST, COLL>(P, lk, P.dv, P.dv_f, h);  // whole warps: votes
     else bb_apply<L, ST, COLL>(P, lk, h);
     if (has) collide_store<L, ST, COLL>(P, P.dst, at.x, at.y, P.dv, P.dv_f, h);
-    if (WALL && b < P.ngroups) group_force<1, true>(P, b, P.force_out, F, 1.0, lane);
+    if (WALL && b < P.ngroups) group_force<1>(P, b, P.force_out, F, 1.0, lane);
 }
 
 // Blocks of a grid before the bulk tiles: boundary blocks, then force blocks.  Returns true if this block

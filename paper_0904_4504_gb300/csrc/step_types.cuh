@@ -41,8 +41,6 @@ struct InstDev {
                                  // links first, then the others, each part in increasing node order
     const ulonglong2* blinks;    // [nb] their links, as in `links`
     const void* flinks;          // body links for the force (flink_entries)
-    unsigned long long call;     // lbm_step_noalloc: the call's number, which marks its counts in the ticket, a
-                                 // 64-bit word there (take_ticket); else 0
     double2 fconst;              // geometry-only part of the force, -sum c_i 2 w_i rho0
     double2 fmov;                // moving-wall part of the force per unit drive, -sum c_i c_ix 2 w_i rho0 / theta
                                  // (body links, bounce-back, wall drive; 0 otherwise)

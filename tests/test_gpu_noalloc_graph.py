@@ -70,7 +70,7 @@ def test_recorded_and_ordinary_calls(shape, wall):
             if k % 3 == 0:
                 c.two_steps()
                 assert c.right(), k
-        for k in range(150):  # and without waiting between them
+        for k in range(1300):  # and without waiting between them, past each half of the tickets
             c.two_steps()
             if k % 50 == 7:
                 graph.replay()
