@@ -37,17 +37,18 @@ __device__ __forceinline__ float vrcp(float a) { return __frcp_rn(a); }
 // add, a multiply, or a multiply-add with a constant or uniform operand 20.0 (measured, independent chains).
 // So every FP64 operation below is a multiply-add of registers: an add multiplies by a 1 and a multiply adds
 // a 0 that the compiler cannot know, and constants go through a register it cannot know either (their bits
-// xor an unknown zero: two integer instructions, whose units idle).  The results are the same.  1024^2
+// xor an unknown zero: two integer instructions, whose units idle; a zero of each lane's own, since one that is the
+// same for a warp may end up in a uniform register: plain BGK 1024 x 700 D2Q37 415 -> 373 us a step).  The results are the same.  1024^2
 // D2Q37 579 -> 493 us a step, 512^2 152 -> 129; 2048^2 D2Q9 558 -> 482.
-static __device__ int fp64_zero_word = 0;
+static __device__ int fp64_zero_word[32] = {};
 __device__ __forceinline__ double opaque(double k) {
-    const int z = __ldg(&fp64_zero_word);
+    const int z = __ldg(&fp64_zero_word[threadIdx.x & 31]);
     return __hiloint2double(__double2hiint(k) ^ z, __double2loint(k) ^ z);
 }
 // Reads the unknown zero now (before a wait), so that the collision need not wait for it.
 template <class ST>
 __device__ __forceinline__ void prepare_collision() {
-    if (sizeof(ST) == 8) asm volatile("" ::"r"(__ldg(&fp64_zero_word)));
+    if (sizeof(ST) == 8) asm volatile("" ::"r"(__ldg(&fp64_zero_word[threadIdx.x & 31])));
 }
 __device__ __forceinline__ double vadd(double a, double b) { return __fma_rn(a, opaque(1.0), b); }
 __device__ __forceinline__ double vsub(double a, double b) { return __fma_rn(b, -opaque(1.0), a); }
@@ -110,9 +111,12 @@ template <>
 __device__ __forceinline__ double vadds<double>(double b, double k) { return __fma_rn(b, opaque(1.0), opaque(k)); }
 template <>
 __device__ __forceinline__ V2 vadds<V2>(V2 b, float k) { return V2{__fadd_rn(b.x, k), __fadd_rn(b.y, k)}; }
-// A launch constant in every lane, as an operand in registers.
-template <class V> __device__ __forceinline__ V vconst(typename Lane<V>::T k) { return vset<V>(k); }
-template <> __device__ __forceinline__ double vconst<double>(double k) { return opaque(k); }
+// k b + c where many of them share the launch constant k: two nodes at a time with it in registers (kv), one packed
+// operation instead of two.
+template <class V>
+__device__ __forceinline__ V vfmac(typename Lane<V>::T k, V, V b, V c) { return vfmas<V>(k, b, c); }
+template <>
+__device__ __forceinline__ V2 vfmac<V2>(float, V2 kv, V2 b, V2 c) { return vfma(kv, b, c); }
 // The same for compile-time constants (after inlining): a factor of 1 or -1 is an add or a subtract.
 template <class V>
 __device__ __forceinline__ V vfmak(double k, V b, V c) {
@@ -403,7 +407,8 @@ __device__ __forceinline__ void emit_outputs_s(const InstDev& P, const Coef<V>& 
     constexpr int R = L::R;
     constexpr bool H4 = R == 3;
     constexpr bool SCALED = sizeof(ST) == 2, REG = COLL == COLL_REG;
-    const V om = vconst<V>(kconst<T>(P.omega_c, P.omega_c_f));
+    const T om = kconst<T>(P.omega_c, P.omega_c_f);
+    const V omv = vset<V>(om);
     V EA[R + 1], EB[R + 1], OX[R + 1], OY[R + 1], U[R + 1];
 #pragma unroll
     for (int m = 0; m <= R; ++m) EA[m] = REG && SCALED ? vadds(C.c0, -(T)P.He[m]) : C.c0;
@@ -423,7 +428,7 @@ __device__ __forceinline__ void emit_outputs_s(const InstDev& P, const Coef<V>& 
         } else {
             // Eq. 14 discretized: f - (f - f^eq)/tau, with the source in f^eq
             const V hi = h(i);
-            const V v = vfma(om, vsub(eq, hi), hi);
+            const V v = vfmac<V>(om, omv, vsub(eq, hi), hi);
             emit(i, OFFSET ? vadds(v, -(T)off_s<L>(P, i)) : v);
         }
     };

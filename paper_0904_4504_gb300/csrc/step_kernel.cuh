@@ -204,8 +204,15 @@ __device__ __forceinline__ void collide_emit(const InstDev& P, double dv, float 
     const auto at = [&](int i) { return h[i]; };
     const Moments<V> M = moments<L, V>(at);
     if constexpr (sizeof(ST) == 8) {
-        const Coef<V> C = P.body_force ? coefficients<L, ST, COLL, V, 1>(P, dv, dv_f, M) : coefficients<L, ST, COLL, V, 0>(P, dv, dv_f, M);
-        emit_outputs<L, ST, COLL, V>(P, C, at, emit);
+        // (plain BGK: one copy of the outputs, which read the populations)
+        if (COLL == COLL_BGK) {
+            const Coef<V> C = P.body_force ? coefficients<L, ST, COLL, V, 1>(P, dv, dv_f, M) : coefficients<L, ST, COLL, V, 0>(P, dv, dv_f, M);
+            emit_outputs<L, ST, COLL, V>(P, C, at, emit);
+        } else if (P.body_force) {
+            emit_outputs<L, ST, COLL, V>(P, coefficients<L, ST, COLL, V, 1>(P, dv, dv_f, M), at, emit);
+        } else {
+            emit_outputs<L, ST, COLL, V>(P, coefficients<L, ST, COLL, V, 0>(P, dv, dv_f, M), at, emit);
+        }
     } else {
         emit_outputs<L, ST, COLL, V>(P, coefficients<L, ST, COLL, V>(P, dv, dv_f, M), at, emit);
     }
