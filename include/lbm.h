@@ -189,9 +189,9 @@ int lbm_set_tile(lbm_sim* sim, int block_x, int block_y);
  * storage, two with FP32); 31: two
  * neighbouring nodes per thread (D2Q37, 16-bit storage, regularized collision).  lbm_create starts
  * two-buffer bounce-back runs on the fastest single-instance kernel measured: D2Q37 on 1 (FP32); 31 (16-bit,
- * regularized, above 163840 nodes), or 32 where the two buffers exceed 200 MB and the rows 639 nodes; 2 (16-bit
- * else: plain BGK, smaller grids, and rows of 1-32, 65-96 or 129-160 nodes); D2Q9 above 2^18 nodes (FP32) or
- * 2^17 (16-bit), on rows of more than 32 nodes, on 30; else 0.
+ * regularized, above 40000 nodes, 160000 without boundary nodes), or 32 where the two buffers exceed 200 MB and
+ * the rows 639 nodes; 2 (16-bit else: plain BGK, smaller grids, and rows of 1-32, 65-96 or 129-160 nodes); D2Q9
+ * above 2^18 nodes (FP32) or 2^17 (16-bit), on rows of more than 32 nodes, on 30; else 0.
  * lbm_set_tile selects variant 0.
  * Staged kernels (FP32/BF16/FP16 storage), whose interior tiles are copied to shared memory by
  * bulk tensor copies (TMA), one box per direction plane:

@@ -430,7 +430,7 @@ int lbm_batch_add(lbm_batch* b, const lbm_instance_desc* d, int* slot) {
         const bool pairs = b->Q == 37 && b->collision == LBM_COLL_REGULARIZED;
         const int q9 = d->nx > 32 ? 30 : 0;
         const int want = b->variant >= 0 ? b->variant
-                         : half ? (b->Q != 37 ? q9 : pairs ? pair_variant(d->nx, d->ny, 0, true) : 27)
+                         : half ? (b->Q != 37 ? q9 : pairs ? pair_variant(d->nx, d->ny, true, 0, true) : 27)
                          : b->storage == LBM_STORE_F32 ? (b->Q == 37 ? 2 : q9) : 0;
         if (want == 0 || lbm_set_variant(sim, want) != LBM_OK) rc = lbm_set_tile(sim, b->bx, b->by);
     }

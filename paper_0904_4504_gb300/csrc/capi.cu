@@ -1188,7 +1188,7 @@ int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const
         if (lattice == LBM_D2Q9) v = es <= 4 && nx > 32 && (size_t)nx * ny > ((size_t)1 << (es == 4 ? 18 : 17)) ? 30 : 0;
         else if (es == 4) v = 1;
         else if (es == 2)
-            v = g.collision != LBM_COLL_REGULARIZED ? 2 : pair_variant(nx, ny, 2 * plane * H.Q * es, false);
+            v = g.collision != LBM_COLL_REGULARIZED ? 2 : pair_variant(nx, ny, d.nb > 0, 2 * plane * H.Q * es, false);
         if (v) TRY_OR_FREE(use_variant(s, v));
     }
     TRY_OR_FREE(setup_tiles(s));

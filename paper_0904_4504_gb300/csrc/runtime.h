@@ -38,19 +38,20 @@ int fit_sincos(const double* fx, size_t stride, long n0, long n1, double omega, 
 // two neighbouring nodes per thread, direct (31) or staged (32).  A block of 31 covers 64 nodes of a row, where
 // an odd number of 32-node columns, one, three or five, leaves more idle than two nodes per thread gain (us a step, 2 /
 // 31: 32 x 9375 10.7 / 17.0, 96 x 3125 9.8 / 11.8, 160 x 1875 9.8 / 10.4; 224 x 1339 9.8 / 9.8, 64 x 4687 9.7 / 9.1,
-// 1024 x 292 9.7 / 8.0), and a small grid has too few warps of two nodes (none solid: 64^2 2.2 / 3.0, 256 x 512
-// 4.7 / 6.0, 384^2 5.6 / 5.9, 448^2 7.0 / 6.4, 512 x 384 6.9 / 6.2).  The staged tiles, 128 wide and direct at the
+// 1024 x 292 9.7 / 8.0), and a small grid has too few warps of two nodes: without boundary nodes 64^2 2.2 / 3.0,
+// 256 x 512 4.7 / 6.0, 384^2 5.6 / 5.9, 448^2 7.0 / 6.4; with them, whose own latency hides the others', plates of
+// 64^2 3.1 / 3.2, 181^2 3.8 / 4.5, 256^2 4.7 / 4.3.  The staged tiles, 128 wide and direct at the
 // seam, pay on wide grids well past the L2, of more than 200 MB (31 / 32: 128 x 23437 87 / 102, 384 x 7812 81 / 85,
 // 640 x 4687 78 / 76, 2048 x 1464 76 / 70).  In a batch, which keeps the chip full whatever one grid's size, they do
 // unless the grid is narrow and tall (16 instances of 256 x 600 31 / 32: 74 / 89; 24 of 384^2 104 / 104, 16 of 512^2
 // 116 / 111); and kernels with and without staging do not share an SM well (16 grids of 288 to 864 a side all 32:
 // 137 us a step, those below 448 on 31: 147), so a square grid takes 32 whatever its size.
-inline int pair_variant(int nx, int ny, size_t bytes, bool batch) {
+inline int pair_variant(int nx, int ny, bool boundary, size_t bytes, bool batch) {
     const int c = (nx + 31) / 32;
     if (batch && (nx >= 448 || ny < 2 * nx)) return 32;
     if (c % 2 == 1 && c < 7) return 2;
     if (batch) return 31;
-    if ((size_t)nx * ny <= (size_t)5 << 15) return 2;
+    if ((size_t)nx * ny <= (size_t)(boundary ? 40000 : 160000)) return 2;
     return nx >= 640 && bytes > (size_t)200000000 ? 32 : 31;
 }
 

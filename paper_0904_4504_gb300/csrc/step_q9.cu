@@ -58,7 +58,12 @@ PbKernel find_pbatch_q9(int storage, int coll, int variant) {
 // The kernel of several nodes per thread (variant 30; step_q9v.cuh): 128 x 4 tiles with 16-bit storage,
 // 64 x 4 with FP32.  At least 8 blocks of 128 threads per SM (9 and 10 measured 0 to 12 % slower with 16-bit
 // storage, 10 % slower on a 512^2 FP32 grid; 5 and 6 no better; plain BGK FP16 7 / 8: 2048^2 32.2 / 30.7 us a step,
-// 4096^2 139 / 133, 512^2 3.6 / 3.9).
+// 4096^2 139 / 133, but 512^2 3.6 / 3.9, where a grid is a wave of blocks or less: there 7, which spills nothing).
+template <class ST, int COLL>
+static cudaError_t launch_step_q9v_sized(const InstDev& P, dim3 block, cudaStream_t stream) {
+    return P.ntiles <= 1024 ? launch_step_q9v<ST, COLL, 7>(P, block, stream) : launch_step_q9v<ST, COLL, 8>(P, block, stream);
+}
+
 void* find_q9v_launcher(int storage, int coll, int variant) {
     if (variant != 30) return nullptr;
     switch (storage * 2 + coll) {
@@ -66,7 +71,7 @@ void* find_q9v_launcher(int storage, int coll, int variant) {
         case ST_F32 * 2 + COLL_REG: return (void*)&launch_step_q9v<float, COLL_REG, 8>;
         case ST_BF16 * 2 + COLL_BGK: return (void*)&launch_step_q9v<__nv_bfloat16, COLL_BGK, 8>;
         case ST_BF16 * 2 + COLL_REG: return (void*)&launch_step_q9v<__nv_bfloat16, COLL_REG, 8>;
-        case ST_F16 * 2 + COLL_BGK: return (void*)&launch_step_q9v<__half, COLL_BGK, 8>;
+        case ST_F16 * 2 + COLL_BGK: return (void*)&launch_step_q9v_sized<__half, COLL_BGK>;
         case ST_F16 * 2 + COLL_REG: return (void*)&launch_step_q9v<__half, COLL_REG, 8>;
         default: return nullptr;
     }

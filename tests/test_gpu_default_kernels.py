@@ -20,7 +20,7 @@ def _kw(storage, collision):
 @pytest.mark.parametrize("nx,ny,alone,batch", [
     (24, 24, 2, 32), (32, 9000, 2, 2), (33, 9000, 31, 31), (64, 64, 2, 32), (65, 4000, 2, 2), (96, 4000, 2, 2),
     (97, 4000, 31, 31), (160, 2000, 2, 2), (161, 2000, 31, 31), (300, 599, 31, 32), (300, 600, 31, 31), (447, 894, 31, 31),
-    (448, 365, 2, 32), (448, 896, 31, 32), (512, 320, 2, 32), (512, 321, 31, 32), (639, 2200, 31, 32), (640, 2200, 32, 32),
+    (448, 357, 2, 32), (448, 896, 31, 32), (512, 312, 2, 32), (512, 313, 31, 32), (639, 2200, 31, 32), (640, 2200, 32, 32),
     (1024, 1024, 31, 32)])
 def test_pairs_by_the_grids_sides(nx, ny, alone, batch, storage):
     kw = _kw(storage, L.LBM_COLL_REGULARIZED)
@@ -35,6 +35,16 @@ def test_pairs_by_the_grids_sides(nx, ny, alone, batch, storage):
         assert L.lbm_info(inst)["variant"] == batch
     finally:
         L.lbm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("nx,ny,variant", [(200, 200, 2), (200, 201, 31), (96, 900, 2), (256, 256, 31)])
+def test_pairs_on_small_grids_with_boundary_nodes(nx, ny, variant):
+    kw = dict(_kw(L.LBM_STORE_F16, L.LBM_COLL_REGULARIZED), kind=L.LBM_GEOM_PLATE)
+    sim = L.lbm_create(37, nx, ny, 0.8, 0.05, L.make_geometry(**kw))
+    try:
+        assert L.lbm_info(sim)["variant"] == variant
+    finally:
+        L.lbm_destroy(sim)
 
 
 def test_plain_bgk_keeps_one_node_per_thread():
