@@ -22,7 +22,10 @@
  *     lbm_lattice_velocities() returns the table.
  *   - Every call returns 0 on success or a negative LBM_E* code; lbm_last_error() then holds a
  *     message for the calling thread.  No call aborts the process.
- *   - All device memory of a simulation is allocated by lbm_create() and freed by lbm_destroy().
+ *   - The device memory of a simulation is allocated by lbm_create() and freed by lbm_destroy().  Two calls
+ *     may allocate more: lbm_step(), for a force history that outgrows its room (1024 steps at first), and
+ *     lbm_set_variant(), for the link masks by node (16 bytes a node) that most staged kernels read; they
+ *     return LBM_ENOMEM where that fails and leave the simulation as it was.
  *     Host buffers passed in are owned by the caller and are not kept after the call returns.
  *   - A simulation is used by one host thread at a time.
  */

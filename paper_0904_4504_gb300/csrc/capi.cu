@@ -873,7 +873,6 @@ void sim_step_constants(const lbm_sim* s, long count, StepConst* out) {
         StepConst& c = out[k];
         std::memset(&c, 0, sizeof(c));
         c.dv = drive_value(s->geom.drive, s->geom.u0, s->omega, s->steps_done + k);
-        c.dv_f = (float)c.dv;
         if (s->stream_off) {
             float* H = c.H;  // HM[6], Hl[7], Hs[7], He[4], Ho[4]
             stream_offset_cx(s, U, H + 6, H);
@@ -1180,8 +1179,8 @@ int lbm::sim_create(int lattice, int nx, int ny, double tau, double omega, const
     // floor on the default 32 x 4 tile (variant 1 for FP32, 2 for plain BGK with 16-bit storage), for the
     // regularized collision of 16-bit storage two nodes per thread where that pays (pair_variant); for FP32 and 16-bit
     // D2Q9 several nodes per thread (30) but on small grids, where fewer nodes per thread mean more warps (us a
-    // step, 30 / 0; FP32: 2048^2 43.5 / 55.4, 1024^2 9.1 / 11.8, 512^2 3.6 / 3.7, 430^2 3.5 / 2.8, 128^2 2.1 / 1.9;
-    // FP16: 1024^2 7.5 / 13.3, 512^2 3.6 / 4.3, 430^2 3.5 / 3.6, 362^2 3.2 / 2.7, 128^2 2.9 / 2.2) and on rows of
+    // step, 30 / 0; FP32: 2048^2 44.5 / 58.5, 1024^2 9.1 / 11.8, 512^2 3.6 / 3.7, 430^2 3.5 / 2.8, 128^2 2.1 / 1.9;
+    // FP16: 2048^2 28.9 / 53.7, 1024^2 7.4 / 13.3, 512^2 3.6 / 4.3, 430^2 3.5 / 3.6, 362^2 3.2 / 2.7, 128^2 2.9 / 2.2) and on rows of
     // half a tile or less (24 x 60000 FP32 29.1 / 22.7, FP16 47 / 26)
     if (!s->aa && g.wall_scheme == LBM_SCHEME_BOUNCEBACK) {
         int v = 0;
@@ -1259,7 +1258,9 @@ int lbm_step(lbm_sim* s, long n) {
         }
         return LBM_OK;
     }
-    // a short call sums each step's force in the step; 8 steps are where one launch for all is worth it
+    // a short call sums each step's force in the step; 8 steps are where one launch for all is worth it (us a step in
+    // calls of 7 / 8 steps: 64^2 FP32 3.6 / 2.6, 256^2 5.5 / 3.8, D2Q9 256^2 4.6 / 2.3, where the step is longer than its
+    // sum 512^2 FP16 7.6 / 7.9, the same from 32 steps on)
     const bool defer = s->defers_forces() && n >= 8;
     unsigned int* const ticket = s->dev.ticket;
     double2* const partials = s->dev.partials;

@@ -45,9 +45,8 @@ constexpr int kRing = 4;  // steps of one instance whose forces may be in flight
 // 16-bit stream-offset constants (see InstDev).
 struct StepConst {
     double dv;
-    float dv_f;
     float H[28];  // HM[6], Hl[7], Hs[7], He[4], Ho[4], in InstDev's order
-    float pad;
+    float pad[2];
 };
 static_assert(sizeof(StepConst) == 128, "one step's constants are one 128-byte line");
 static_assert(offsetof(InstDev, Ho) + 4 * sizeof(float) - offsetof(InstDev, HM) == 28 * sizeof(float),
@@ -79,7 +78,8 @@ constexpr int kForceItemGroups = 4;  // force groups per warp of a force item
 // PB_PAIR: plain, two nodes per thread; each of four warps takes every fourth row of its 64 x 8 tile.  Bound
 // by the strips' load latency: 16 warps of 57 loads each, 128 registers, and the bulk of a step's items is long
 // enough that the item's prologue (about 3 us of 90) does not show.  16 FP16 instances of 256 to 1024 a side
-// 205 us a step (0.75 of the copy bandwidth; staged one node per thread 235 to 245), 64 of them 868 (950).  Not
+// 205 us a step (0.75 of the copy bandwidth; staged one node per thread 235 to 245), 64 of them 868 (950; 866 before
+// the staged tiles shared the collision that spills there).  Not
 // faster: 64 x 4 tiles at 20 warps of 96 registers 208 and 881, 128-node rows 252 and 924, staged 128 x 2
 // pairs 366 and 1057 (blocks too short-lived between waits).
 enum PbPath { PB_STAGED = 0, PB_PLAIN = 1, PB_PAIR = 2 };

@@ -12,10 +12,11 @@
 // Two forms.  Direct (variant 31): the 57 loads of a thread are independent and all in flight at once; 96
 // registers, 20 warps per SM.  Staged (variant 32): bulk tensor copies bring a block's rows to shared
 // memory; more bytes in flight, but block by block.  Measured, us a step (direct / staged / one node per
-// thread): 512^2 7.6 / 10.6 / 8.9, 768^2 13.7 / 16.3 / 18.7, 1024^2 28.0 / 29.1 / 34.9, 1280^2 43.0 / 41.8 /
-// 52.7, 2048^2 107 / 96 / 138.  So a single simulation stages when its two buffers hold more than about
-// 200 MB, well past the L2; a batch of instances, which keeps the SMs full whatever a launch's ramp, always
-// does (64 instances of 256 to 1024 a side: 757 us a step staged, 807 direct, 865 one node per thread).
+// thread): 256^2 4.6 / 5.1 / 4.7, 512^2 7.6 / 10.4 / 8.7, 768^2 13.8 / 15.8 / 17.9, 1024^2 26.8 / 27.5 / 33.6, 1280^2
+// 42.2 / 40.9 / 51.7, 2048^2 105 / 94 / 142.  So a single simulation stages when its two buffers hold more than about
+// 200 MB, well past the L2; a batch of instances, which keeps the SMs full whatever a launch's ramp, nearly
+// always does (64 instances of 256 to 1024 a side: 757 us a step staged, 807 direct, 865 one node per thread).
+// pair_variant (runtime.h) draws the lines, narrow and small grids included.
 #pragma once
 
 #include "step_tma.cuh"
@@ -185,7 +186,8 @@ cudaError_t launch_pair16(const InstDev& P, cudaStream_t stream) {
 }
 
 // Rows shorter than 512 nodes take blocks of one warp (64 nodes), so that at most an eighth of the lanes
-// of a long row idle (256^2 4.75 us a step against 5.09, 1024^2 30.3 against 29.9).
+// of a long row idle (the two compared in this kernel's first form: 256^2 4.75 us a step against 5.09, 1024^2 30.3
+// against 29.9).
 template <class L, class ST, int COLL>
 cudaError_t launch_step_pair16(const InstDev& P, dim3, cudaStream_t stream) {
     return P.nx < 512 ? launch_pair16<L, ST, COLL, 32, 20>(P, stream) : launch_pair16<L, ST, COLL, 64, 10>(P, stream);

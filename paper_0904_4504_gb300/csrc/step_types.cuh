@@ -47,7 +47,6 @@ struct InstDev {
     int nb, nbf;                 // nodes listed, and those of them with body links
     int nfl, glen;               // body links, and links per lane of a force group
     int ngroups;                 // force groups of a step
-    int force_pad;
     long long plane;             // ny * pitch
     int nx, ny, pitch;
     int ntx;                     // tiles along x
