@@ -80,9 +80,10 @@ def kernel_source_hash():
 # ncu capture each, with the digest of the sources they were captured from: once any source
 # changes, the entry no longer applies and the line reports traffic null.
 TRAFFIC = {
-    ("beam1024", 1): (263564288, "6cb49ca6ec672d3b"),          # 156.4 MB read + 107.2 MB written
-    ("beam1024x1-f16", 26): (109641984, "6cb49ca6ec672d3b"),   # 78.8 + 30.8 MB
-    ("beam1024x1-f16", 27): (109117184, "6cb49ca6ec672d3b"),   # 78.8 + 30.3 MB
+    ("beam1024", 1): (263856896, "d9ca23a23d116e43"),          # 156.8 MB read + 107.1 MB written
+    ("beam1024x1-f16", 31): (109507584, "d9ca23a23d116e43"),   # 78.8 + 30.7 MB
+    ("beam1024x1-f16", 32): (108165888, "d9ca23a23d116e43"),   # 78.8 + 29.3 MB
+    ("beam1024x1-f16", 27): (112966400, "d9ca23a23d116e43"),   # 78.8 + 34.2 MB
 }
 
 
@@ -96,9 +97,10 @@ def traffic_for(workload, variant):
 # is bound by instruction issue, so the batched line also reports the issue rate against the SMs'
 # issue peak.
 INST_PER_NODE = {
-    ("beam1024", 1): (739.3, "6cb49ca6ec672d3b"),              # 24,202,187 warp instructions, 1,047,552 fluid nodes
-    ("beam1024x1-f16", 26): (770.8, "6cb49ca6ec672d3b"),       # 25,232,720
-    ("beam1024x1-f16", 27): (763.4, "6cb49ca6ec672d3b"),       # 24,990,376
+    ("beam1024", 1): (742.4, "d9ca23a23d116e43"),              # 24,301,892 warp instructions, 1,047,552 fluid nodes
+    ("beam1024x1-f16", 31): (514.7, "d9ca23a23d116e43"),       # 16,848,127
+    ("beam1024x1-f16", 32): (512.2, "d9ca23a23d116e43"),       # 16,768,631
+    ("beam1024x1-f16", 27): (760.9, "d9ca23a23d116e43"),       # 24,908,609
 }
 
 
