@@ -80,10 +80,10 @@ def kernel_source_hash():
 # ncu capture each, with the digest of the sources they were captured from: once any source
 # changes, the entry no longer applies and the line reports traffic null.
 TRAFFIC = {
-    ("beam1024", 1): (263856896, "d9ca23a23d116e43"),          # 156.8 MB read + 107.1 MB written
-    ("beam1024x1-f16", 31): (109507584, "d9ca23a23d116e43"),   # 78.8 + 30.7 MB
-    ("beam1024x1-f16", 32): (108165888, "d9ca23a23d116e43"),   # 78.8 + 29.3 MB
-    ("beam1024x1-f16", 27): (112966400, "d9ca23a23d116e43"),   # 78.8 + 34.2 MB
+    ("beam1024", 1): (263801600, "0c35ba7cc673ab01"),          # 156.8 MB read + 107.0 MB written
+    ("beam1024x1-f16", 31): (109613312, "0c35ba7cc673ab01"),   # 78.8 + 30.8 MB
+    ("beam1024x1-f16", 32): (108287488, "0c35ba7cc673ab01"),   # 78.8 + 29.5 MB
+    ("beam1024x1-f16", 27): (113044480, "0c35ba7cc673ab01"),   # 78.8 + 34.2 MB
 }
 
 
@@ -97,10 +97,10 @@ def traffic_for(workload, variant):
 # is bound by instruction issue, so the batched line also reports the issue rate against the SMs'
 # issue peak.
 INST_PER_NODE = {
-    ("beam1024", 1): (742.4, "d9ca23a23d116e43"),              # 24,301,892 warp instructions, 1,047,552 fluid nodes
-    ("beam1024x1-f16", 31): (514.7, "d9ca23a23d116e43"),       # 16,848,127
-    ("beam1024x1-f16", 32): (512.2, "d9ca23a23d116e43"),       # 16,768,631
-    ("beam1024x1-f16", 27): (760.9, "d9ca23a23d116e43"),       # 24,908,609
+    ("beam1024", 1): (742.4, "0c35ba7cc673ab01"),              # 24,301,917 warp instructions, 1,047,552 fluid nodes
+    ("beam1024x1-f16", 31): (514.7, "0c35ba7cc673ab01"),       # 16,848,074
+    ("beam1024x1-f16", 32): (512.2, "0c35ba7cc673ab01"),       # 16,768,569
+    ("beam1024x1-f16", 27): (760.9, "0c35ba7cc673ab01"),       # 24,908,547
 }
 
 
